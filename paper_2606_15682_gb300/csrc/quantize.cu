@@ -102,17 +102,19 @@ __global__ void tensor_scale_finalize(float* g) {
 // Where one pass of the quantizer reads: the thread's kUnroll 16-element
 // blocks of the iteration that starts at the warp-uniform block index bidx0
 // (block bidx0 + u * stride + lane).
+template <int U = kUnroll>
 struct BlockSlots {
-  uint4 v0[kUnroll], v1[kUnroll];
-  uint32_t row[kUnroll], kb[kUnroll];
+  uint4 v0[U], v1[U];
+  uint32_t row[U], kb[U];
 };
 
+template <int U>
 __device__ __forceinline__ void load_blocks(const uint16_t* __restrict__ x, FastDiv kblocks_div, uint32_t total_blocks,
                                             int64_t ld, bool dense, uint32_t bidx0, uint32_t stride, uint32_t lane,
-                                            BlockSlots& sl) {
+                                            BlockSlots<U>& sl) {
   const uint32_t kblocks = kblocks_div.d;
 #pragma unroll
-  for (int u = 0; u < kUnroll; ++u) {
+  for (int u = 0; u < U; ++u) {
     const uint32_t b = bidx0 + u * stride + lane;
     sl.row[u] = kblocks_div.div(b);
     sl.kb[u] = b - sl.row[u] * kblocks;
@@ -124,17 +126,18 @@ __device__ __forceinline__ void load_blocks(const uint16_t* __restrict__ x, Fast
   }
 }
 
-__device__ __forceinline__ uint32_t amax_bits_of(const BlockSlots& sl) {
+template <int U>
+__device__ __forceinline__ uint32_t amax_bits_of(const BlockSlots<U>& sl) {
   uint32_t m = 0;
 #pragma unroll
-  for (int u = 0; u < kUnroll; ++u) m = max(m, max(amax_bits_bf16x8(sl.v0[u]), amax_bits_bf16x8(sl.v1[u])));
+  for (int u = 0; u < U; ++u) m = max(m, max(amax_bits_bf16x8(sl.v0[u]), amax_bits_bf16x8(sl.v1[u])));
   return m;
 }
 
 // Quantize the loaded blocks with tensor scale g.  Every lane of the warp
 // takes part (the MMA-layout scale gather shuffles across lanes).
-template <bool kMMA>
-__device__ __forceinline__ void quantize_loaded(const BlockSlots& sl, uint32_t total_blocks, uint32_t kblocks,
+template <bool kMMA, int U>
+__device__ __forceinline__ void quantize_loaded(const BlockSlots<U>& sl, uint32_t total_blocks, uint32_t kblocks,
                                                 uint32_t bidx0, uint32_t stride, uint32_t lane, float g, float six_g,
                                                 bool g_ok, uint2* __restrict__ codes, uint8_t* __restrict__ scales, int* status) {
   const uint32_t kgroups = kblocks >> 2;
@@ -142,7 +145,7 @@ __device__ __forceinline__ void quantize_loaded(const BlockSlots& sl, uint32_t t
   const uint64_t scale_bytes =
       kMMA ? static_cast<uint64_t>((total_blocks / kblocks + 127u) & ~127u) * kblocks : total_blocks;
 #pragma unroll
-  for (int u = 0; u < kUnroll; ++u) {
+  for (int u = 0; u < U; ++u) {
     const uint32_t b = bidx0 + u * stride + lane;
     const bool live = b < total_blocks;
     float xf[16];
@@ -174,15 +177,29 @@ __device__ __forceinline__ void quantize_loaded(const BlockSlots& sl, uint32_t t
 }
 
 // Zero the MMA-layout scales of the padding rows up to the next multiple of 128.
+// They all lie in the last row tile, whose atoms are contiguous: 16-byte chunk
+// i of the tile (k group i / 32, l = i % 32) holds the four-scale words of
+// rows l, l + 32, l + 64 and l + 96, so the padding is a suffix of each chunk
+// and, from l = rows % 128 on, whole chunks (one 16-byte store where the
+// buffer allows it).  One byte at a time, the 127 padding rows of a one-row
+// activation took most of the call: 1 x 5120 15.5 us, 1 x 13824 33.7 us.
 __device__ __forceinline__ void zero_scale_padding(uint32_t rows, uint32_t kblocks, uint8_t* __restrict__ scales,
                                                    int* status) {
-  const uint32_t kgroups = kblocks >> 2;
-  const uint32_t padded = (rows + 127u) & ~127u;
-  const uint32_t pad = (padded - rows) * kblocks;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < pad; i += gridDim.x * blockDim.x) {
-    const uint32_t r = rows + i / kblocks, k = i % kblocks;
-    const uint64_t off = mma_scale_offset(r, k, kgroups);
-    if (in_bounds(status, off < static_cast<uint64_t>(padded) * kblocks)) scales[off] = 0;
+  const uint32_t kgroups = kblocks >> 2, used = rows & 127u;
+  if (used == 0) return;
+  const uint64_t tile_off = static_cast<uint64_t>(rows >> 7) * kgroups * 512u;
+  const uint64_t scale_bytes = tile_off + static_cast<uint64_t>(kgroups) * 512u;
+  const bool wide = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < kgroups * 32u; i += gridDim.x * blockDim.x) {
+    const uint32_t l = i & 31u;
+    const uint32_t first = used > l ? (used - l + 31u) >> 5 : 0u;  // first padding word of the chunk
+    const uint64_t off = tile_off + static_cast<uint64_t>(i) * 16u;
+    if (!in_bounds(status, off + 16 <= scale_bytes)) continue;
+    if (first == 0 && wide) {
+      *reinterpret_cast<uint4*>(scales + off) = make_uint4(0, 0, 0, 0);
+    } else {
+      for (uint32_t j = first; j < 4; ++j) *reinterpret_cast<uint32_t*>(scales + off + 4 * j) = 0u;
+    }
   }
 }
 
@@ -200,7 +217,7 @@ __device__ __forceinline__ void quantize_blocks(const uint16_t* __restrict__ x, 
   const uint32_t stride = gridDim.x * blockDim.x;
   // bidx0 is warp-uniform so every lane takes part in the scale gather.
   for (uint32_t bidx0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); bidx0 < total_blocks; bidx0 += stride * kUnroll) {
-    BlockSlots sl;
+    BlockSlots<> sl;
     load_blocks(x, kblocks_div, total_blocks, ld, dense, bidx0, stride, lane, sl);
     quantize_loaded<kMMA>(sl, total_blocks, kblocks_div.d, bidx0, stride, lane, g, six_g, g_ok, codes, scales,
                           status);
@@ -262,13 +279,13 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
 // with one release store that also carries the amax, so the waiting blocks
 // learn both from the load that ends their wait.  The epoch is read before
 // the loads of phase 1: it cannot change until every block has arrived.
-template <bool kMMA>
+template <bool kMMA, int U>
 __global__ void __launch_bounds__(kThreads) quantize_dynamic_kernel(
     const uint16_t* __restrict__ x, FastDiv kblocks_div, uint32_t total_blocks, int64_t ld, bool dense, uint32_t rows,
     unsigned long long* state, float* __restrict__ g_out, uint2* __restrict__ codes, uint8_t* __restrict__ scales,
     int* status, int stash_iters) {
   // Shared-memory stash: the blocks of the first stash_iters phase-1
-  // iterations, [iteration * kUnroll + slot][half][thread] as 16-byte words.
+  // iterations, [iteration * U + slot][half][thread] as 16-byte words.
   extern __shared__ uint4 stash[];
   griddep_wait_and_release();
   timeline_stamp(0);
@@ -282,17 +299,17 @@ __global__ void __launch_bounds__(kThreads) quantize_dynamic_kernel(
   // stash_iters iterations in shared memory, and phase 2 reads from x again
   // only the iterations in between.
   const uint32_t bidx_first = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
-  BlockSlots sl;
+  BlockSlots<U> sl;
   uint32_t m = 0, bidx_last = bidx_first;
   int it = 0;
-  for (uint32_t bidx0 = bidx_first; bidx0 < total_blocks || bidx0 == bidx_first; bidx0 += stride * kUnroll, ++it) {
+  for (uint32_t bidx0 = bidx_first; bidx0 < total_blocks || bidx0 == bidx_first; bidx0 += stride * U, ++it) {
     load_blocks(x, kblocks_div, total_blocks, ld, dense, bidx0, stride, lane, sl);
     m = max(m, amax_bits_of(sl));
     if (it < stash_iters) {
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        stash[((it * kUnroll + u) * 2) * kThreads + threadIdx.x] = sl.v0[u];
-        stash[((it * kUnroll + u) * 2 + 1) * kThreads + threadIdx.x] = sl.v1[u];
+      for (int u = 0; u < U; ++u) {
+        stash[((it * U + u) * 2) * kThreads + threadIdx.x] = sl.v0[u];
+        stash[((it * U + u) * 2 + 1) * kThreads + threadIdx.x] = sl.v1[u];
       }
     }
     bidx_last = bidx0;
@@ -346,6 +363,7 @@ __global__ void __launch_bounds__(kThreads) quantize_dynamic_kernel(
   const float g = amax > 0.0f ? __fdiv_rn(amax, 2688.0f) : 1.0f;
   const float six_g = __fmul_rn(6.0f, g);
   if (blockIdx.x == 0 && threadIdx.x == 0) *g_out = g;
+  if (kMMA) zero_scale_padding(rows, kblocks_div.d, scales, status);
   if (bidx_last < total_blocks)
     quantize_loaded<kMMA>(sl, total_blocks, kblocks_div.d, bidx_last, stride, lane, g, six_g, true, codes, scales,
                           status);
@@ -354,28 +372,60 @@ __global__ void __launch_bounds__(kThreads) quantize_dynamic_kernel(
   // latest of them in L2.  The stashed ones come from shared memory.
   const int n_iter = it;
   for (int k = n_iter - 2; k >= 0; --k) {
-    const uint32_t bidx0 = bidx_first + static_cast<uint32_t>(k) * stride * kUnroll;
-    BlockSlots t;
+    const uint32_t bidx0 = bidx_first + static_cast<uint32_t>(k) * stride * U;
+    BlockSlots<U> t;
     if (k < stash_iters) {
       const uint32_t kblocks = kblocks_div.d;
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
+      for (int u = 0; u < U; ++u) {
         const uint32_t b = bidx0 + u * stride + lane;
         t.row[u] = kblocks_div.div(b);
         t.kb[u] = b - t.row[u] * kblocks;
-        t.v0[u] = stash[((k * kUnroll + u) * 2) * kThreads + threadIdx.x];
-        t.v1[u] = stash[((k * kUnroll + u) * 2 + 1) * kThreads + threadIdx.x];
+        t.v0[u] = stash[((k * U + u) * 2) * kThreads + threadIdx.x];
+        t.v1[u] = stash[((k * U + u) * 2 + 1) * kThreads + threadIdx.x];
       }
     } else {
       load_blocks(x, kblocks_div, total_blocks, ld, dense, bidx0, stride, lane, t);
     }
     quantize_loaded<kMMA>(t, total_blocks, kblocks_div.d, bidx0, stride, lane, g, six_g, true, codes, scales, status);
   }
-  if (kMMA) zero_scale_padding(rows, kblocks_div.d, scales, status);
 #ifdef NVFP4_TIMELINE
   __syncthreads();
   timeline_stamp(4);
 #endif
+}
+
+// a1 + a2 of an activation of at most kSmallBlocks 16-element blocks, in one
+// CTA: the amax needs no grid barrier, so the launch need not be cooperative
+// and overlaps the previous kernel's tail.  Same results as the kernel above.
+// Latency-bound: one load, one reduction, one block scale per block.  GB300,
+// back to back in a graph, against the grid-wide kernel (one block per
+// thread): 1 x 5120 4.87 -> 2.68 us, 1 x 13824 5.18 -> 4.05, 4 x 5120 4.68 ->
+// 3.70, 16 x 1536 4.34 -> 3.18; with four blocks a thread (8 x 5120) it would
+// be no faster.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallUnroll = 2;
+constexpr uint32_t kSmallBlocks = kSmallThreads * kSmallUnroll;
+
+template <bool kMMA, int U>
+__global__ void __launch_bounds__(kSmallThreads) quantize_dynamic_small_kernel(
+    const uint16_t* __restrict__ x, FastDiv kblocks_div, uint32_t total_blocks, int64_t ld, bool dense, uint32_t rows,
+    float* __restrict__ g_out, uint2* __restrict__ codes, uint8_t* __restrict__ scales, int* status) {
+  griddep_wait_and_release();
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t bidx0 = threadIdx.x & ~31u;
+  BlockSlots<U> sl;
+  load_blocks(x, kblocks_div, total_blocks, ld, dense, bidx0, kSmallThreads, lane, sl);
+  if (kMMA) zero_scale_padding(rows, kblocks_div.d, scales, status);  // while the loads are in flight
+  __shared__ uint32_t warp_max[kSmallThreads / 32];
+  const uint32_t wm = __reduce_max_sync(0xffffffffu, amax_bits_of(sl));
+  if (lane == 0) warp_max[warp] = wm;
+  __syncthreads();
+  const float amax = __uint_as_float(__reduce_max_sync(0xffffffffu, warp_max[lane]) << 16);
+  const float g = amax > 0.0f ? __fdiv_rn(amax, 2688.0f) : 1.0f;
+  if (threadIdx.x == 0) *g_out = g;
+  quantize_loaded<kMMA>(sl, total_blocks, kblocks_div.d, bidx0, kSmallThreads, lane, g, __fmul_rn(6.0f, g), true,
+                        codes, scales, status);
 }
 
 // Blocks of quantize_dynamic_kernel that fit on the device at once (a
@@ -385,7 +435,7 @@ __global__ void __launch_bounds__(kThreads) quantize_dynamic_kernel(
 constexpr size_t kStashIterBytes = static_cast<size_t>(kUnroll) * 2 * kThreads * 16;
 constexpr int kMaxStashIters = 2;
 
-template <bool kMMA>
+template <bool kMMA, int U>
 int dynamic_capacity(int stash_iters) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, int> cache;
@@ -396,13 +446,13 @@ int dynamic_capacity(int stash_iters) {
   if (it != cache.end()) return it->second;
   const size_t smem = stash_iters * kStashIterBytes;
   if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(quantize_dynamic_kernel<kMMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      cudaFuncSetAttribute(quantize_dynamic_kernel<kMMA, U>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(kMaxStashIters * kStashIterBytes)) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quantize_dynamic_kernel<kMMA>, kThreads, smem) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quantize_dynamic_kernel<kMMA, U>, kThreads, smem) !=
           cudaSuccess ||
       per_sm <= 0) {
     cudaGetLastError();
@@ -601,18 +651,48 @@ NVFP4_API nvfp4_status nvfp4_quantize_dynamic(const void* x_bf16, int64_t rows, 
   const bool mma = layout == NVFP4_SCALES_MMA;
   const uint32_t kblocks = static_cast<uint32_t>(cols / 16);
   const uint32_t total_blocks = static_cast<uint32_t>(rows * kblocks);
-  // kUnroll blocks per thread per pass, as few CTAs as that allows (each CTA
-  // is one arrival at the grid barrier); x stays in registers across the
-  // barrier when one pass covers it, and up to kMaxStashIters more passes
-  // wait in shared memory.
-  int grid = grid_for(total_blocks, kThreads * kUnroll);
-  int cap = mma ? dynamic_capacity<true>(0) : dynamic_capacity<false>(0);
+  const bool dense = ld == cols;
+  const uint16_t* x = static_cast<const uint16_t*>(x_bf16);
+  uint2* out_codes = reinterpret_cast<uint2*>(codes);
+  const uint32_t n_rows = static_cast<uint32_t>(rows);
+  if (total_blocks <= kSmallBlocks) {
+    const bool one = total_blocks <= kSmallThreads;
+    const auto kernel = mma ? (one ? quantize_dynamic_small_kernel<true, 1> : quantize_dynamic_small_kernel<true, 2>)
+                            : (one ? quantize_dynamic_small_kernel<false, 1> : quantize_dynamic_small_kernel<false, 2>);
+    if (launch_pdl(kernel, dim3(1), dim3(kSmallThreads), 0, static_cast<cudaStream_t>(stream), x, FastDiv(kblocks),
+                   total_blocks, ld, dense, n_rows, g_dev, out_codes, scales, status_word_dev()) != cudaSuccess)
+      return NVFP4_ERR_CUDA;
+    count_launches(1);
+    return launch_status();
+  }
+  // Blocks per thread and pass: 1 while that gives at most one CTA per SM, 2
+  // while two cover the tensor in one pass, else 4.  More per thread means
+  // fewer arrivals at the barrier but a longer serial chain of block scales on
+  // fewer SMs.  GB300, back to back in a graph, 1 / 2 / 4 per thread: 16 x 5120
+  // 4.50 / 4.67 / 5.57 us, 64 x 5120 4.56 / 4.72 / 5.38, 256 x 5120 5.08 / 4.88
+  // / 5.24, 2048 x 1536 6.26 / 5.72 / 6.08, 1000 x 13824 (several passes) 15.0
+  // / 13.7 / 13.1.
+  int unroll = 1;
+  const auto capacity = [&](int stash) {
+    return unroll == 1   ? (mma ? dynamic_capacity<true, 1>(stash) : dynamic_capacity<false, 1>(stash))
+           : unroll == 2 ? (mma ? dynamic_capacity<true, 2>(stash) : dynamic_capacity<false, 2>(stash))
+                         : (mma ? dynamic_capacity<true, kUnroll>(stash) : dynamic_capacity<false, kUnroll>(stash));
+  };
+  if (total_blocks > static_cast<uint32_t>(sm_count()) * kThreads) {
+    unroll = 2;
+    if (total_blocks > static_cast<uint64_t>(capacity(0)) * kThreads * 2) unroll = kUnroll;
+  }
+  // As few CTAs as `unroll` blocks per thread allow (each CTA is one arrival
+  // at the grid barrier); x stays in registers across the barrier when one
+  // pass covers it, and up to kMaxStashIters more passes wait in shared memory.
+  int grid = grid_for(total_blocks, kThreads * unroll);
+  int cap = capacity(0);
   if (cap <= 0) return NVFP4_ERR_CUDA;
   int stash_iters = 0;
   if (grid > cap) {
-    const int cap_stash = mma ? dynamic_capacity<true>(kMaxStashIters) : dynamic_capacity<false>(kMaxStashIters);
+    const int cap_stash = capacity(kMaxStashIters);
     if (cap_stash > 0) {
-      const uint64_t per_iter = static_cast<uint64_t>(cap_stash) * kThreads * kUnroll;
+      const uint64_t per_iter = static_cast<uint64_t>(cap_stash) * kThreads * unroll;
       const uint64_t iters = (total_blocks + per_iter - 1) / per_iter;
       stash_iters = static_cast<int>(iters - 1 < kMaxStashIters ? iters - 1 : kMaxStashIters);
       cap = cap_stash;
@@ -636,11 +716,13 @@ NVFP4_API nvfp4_status nvfp4_quantize_dynamic(const void* x_bf16, int64_t rows, 
   cfg.stream = static_cast<cudaStream_t>(stream);
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e =
-      cudaLaunchKernelEx(&cfg, mma ? quantize_dynamic_kernel<true> : quantize_dynamic_kernel<false>,
-                         static_cast<const uint16_t*>(x_bf16), FastDiv(kblocks), total_blocks, ld, ld == cols,
-                         static_cast<uint32_t>(rows), static_cast<unsigned long long*>(state_dev), g_dev,
-                         reinterpret_cast<uint2*>(codes), scales, status_word_dev(), stash_iters);
+  const auto kernel =
+      unroll == 1   ? (mma ? quantize_dynamic_kernel<true, 1> : quantize_dynamic_kernel<false, 1>)
+      : unroll == 2 ? (mma ? quantize_dynamic_kernel<true, 2> : quantize_dynamic_kernel<false, 2>)
+                    : (mma ? quantize_dynamic_kernel<true, kUnroll> : quantize_dynamic_kernel<false, kUnroll>);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, x, FastDiv(kblocks), total_blocks, ld, dense, n_rows,
+                                           static_cast<unsigned long long*>(state_dev), g_dev, out_codes, scales,
+                                           status_word_dev(), stash_iters);
   if (e != cudaSuccess) return NVFP4_ERR_CUDA;
   count_launches(1);
   return launch_status();

@@ -277,3 +277,28 @@ def test_dynamic_barrier_wait_runs_out_and_reports_timeout(N):
     torch.cuda.synchronize()
     assert N.nvfp4_get_device_status() == 0
     assert np.float32(g.item()) == O.tensor_scale(f32(x))
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 64), (1, 16384), (2, 16384), (2, 16448), (3, 10880), (31, 64), (33, 960),
+                                       (127, 256), (129, 256), (64, 5120), (127, 5120), (160, 5120)])
+@pytest.mark.parametrize("offset", [0, 4])
+def test_dynamic_small_paths_and_padding_rows(N, rows, cols, offset):
+    """Edges of the one-CTA form (1024 and 2048 blocks), of the blocks per
+    thread, and the padding rows' zero scales in a 16-byte and in a 4-byte
+    aligned buffer; bytes around the buffer stay as they were."""
+    x = torch.randn(rows, cols, device="cuda").to(torch.bfloat16)
+    state = torch.zeros(N.DYNAMIC_STATE_BYTES, dtype=torch.uint8, device="cuda")
+    g = torch.empty(1, dtype=torch.float32, device="cuda")
+    codes = torch.empty(rows, cols // 2, dtype=torch.uint8, device="cuda")
+    size = N.nvfp4_scales_bytes(rows, cols, N.SCALES_MMA)
+    buf = torch.full((size + 32,), 0xEE, dtype=torch.uint8, device="cuda")
+    scales = buf[offset:offset + size]
+    torch.cuda.synchronize()
+    N.nvfp4_quantize_dynamic(x, state, g, codes, scales, N.SCALES_MMA)
+    torch.cuda.synchronize()
+    assert N.nvfp4_get_device_status() == 0
+    g_ref = O.tensor_scale(f32(x))
+    rc, rs = O.quantize(f32(x), g_ref)
+    assert np.float32(g.item()) == g_ref and np.array_equal(u8(codes), rc)
+    assert np.array_equal(u8(scales), O.scales_to_mma(rs))
+    assert (u8(buf[:offset]) == 0xEE).all() and (u8(buf[offset + size:]) == 0xEE).all()
