@@ -215,8 +215,11 @@ struct GemmArgs {
   int fault_skip_stage;
   // Row super-tiles per raster group (unit_coords).
   int group_m;
-  // Split-K kernel: CTA pairs per cluster, each taking one range of K.
+  // Split-K kernel: CTA pairs per cluster, each taking one range of K; skinny
+  // kernel: CTAs per cluster.
   int splits;
+  // Skinny kernel: rows of the A box, and W k-blocks prefetched into L2.
+  int a_box_rows, prefetch_kb;
   // bf16 output [M, N] with row pitch ldo elements (the stores that do not
   // go through the output tensor map).
   uint16_t* out;
@@ -1320,6 +1323,271 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   if (warp == 1) tmem_dealloc_pair(tmem, kTmemCols);
 }
 
+// ------------------------------------------------ skinny (M <= 128) kernel ---
+// One row tile of activations: the call streams W once and the time is W's
+// bytes.  A tile is 128 W rows; a cluster of S CTAs splits its K, so that
+// every SM holds W loads in flight whatever N is, and two CTAs share an SM
+// (one's set-up, drain and reduction under the other's stream).  The A box
+// carries only the M rows rounded up to 8; the MMA's 128 A rows read on into
+// whatever follows in shared memory, which only reaches accumulator rows that
+// are never stored (E2M1 codes are finite, and padding rows have zero scales).
+// One thread issues a k-block's scale copies and then its MMAs: the tensor
+// core runs copy -> MMA of one thread in order, so no barrier lies between.
+// The S fp32 partials ([rows, 128], 512-byte rows with swizzled 16-byte
+// chunks, in the idle ring) are added across the cluster in split order, each
+// CTA taking a share of the columns: deterministic for a given shape.
+//   warp 0  TMA producer; before it waits for the previous kernel it
+//           prefetches its first W k-blocks into L2, while the activation is
+//           still being quantized (a prefetch of something that kernel writes
+//           would be harmless: L2 is the point of coherence)
+//   warp 1  TMEM allocation, MMAs
+//   warp 2  scale copies into TMEM, ahead of the MMAs (one thread doing both
+//           in order was 10-20 % slower per k-block)
+//   warps 3-6  drain, reduction, stores
+// Measured with the activation's quantization before it (graph replay, W from
+// DRAM), against the kernels that served these shapes before, 1 row: 5120 x
+// 5120 13.6 -> 8.6 us, 7168 x 5120 14.5 -> 9.2, 27648 x 5120 31.1 -> 18.5 (W's
+// bytes at the copy rate: 11.7), 5120 x 13824 23.1 -> 13.4.
+template <int ROWS_>
+struct SkinnyCfg {
+  static constexpr int kRows = ROWS_;                      // A rows held per k-block: 32, 64 or 128
+  static constexpr int kStages = ROWS_ == 32 ? 4 : 3;
+  static constexpr int kEpiWarps = 4;
+  static constexpr int kThreads = 96 + 32 * kEpiWarps;
+  static constexpr uint32_t kTileBytesA = kRows * BK / 2;
+  static constexpr uint32_t kTileBytesB = 128 * BK / 2;
+  static constexpr uint32_t kSfBytes = 128 * (BK / 16);    // of A and of W: four 512-byte atoms
+  static constexpr uint32_t kTmemCols = 256;               // two CTAs per SM
+  static constexpr uint32_t kSfTmemCol = 128;              // 32 columns per stage after the accumulator
+  static constexpr size_t kSmemBytes = 1024 + kStages * (kTileBytesA + kTileBytesB + 2 * kSfBytes) + 256 /*barriers*/;
+  static constexpr uint32_t kIdesc = (1u << 7) | (1u << 10) | (static_cast<uint32_t>(128 >> 3) << 17) |
+                                     (static_cast<uint32_t>(BM >> 4) << 24);
+  static_assert(kSfTmemCol + kStages * 32 <= kTmemCols, "TMEM budget");
+  static_assert(2 * (kSmemBytes + 1024) <= 228 * 1024, "two CTAs per SM");
+  static_assert(kRows * 512u <= kStages * (kTileBytesA + kTileBytesB), "the partial fits in the ring");
+};
+
+constexpr int kSkinnyPrefetch = 4;  // W k-blocks per CTA: what arrives while a small activation is quantized
+
+// Prefetch one 2-D box into L2.
+__device__ __forceinline__ void tma_prefetch_2d(const void* tmap, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                   reinterpret_cast<uint64_t>(tmap)),
+               "r"(x), "r"(y)
+               : "memory");
+}
+
+// 16-byte chunk j (0..31) of row `row` of the skinny partial (512-byte rows).
+__device__ __forceinline__ uint32_t skinny_part_offset(uint32_t row, uint32_t j) {
+  return row * 512u + ((j ^ (row & 7u)) << 4);
+}
+
+// Add the cluster's S partials over this CTA's share of the 32 column chunks in
+// split order, scale, round to bf16 and store; 128 threads, one chunk of one row each per step.
+template <int S>
+__device__ __forceinline__ void skinny_reduce(uint32_t part0, uint32_t rank, uint32_t tid, int n0, float scale,
+                                              const GemmArgs& args) {
+  uint32_t base[S];
+#pragma unroll
+  for (int t = 0; t < S; ++t)
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(base[t]) : "r"(part0), "r"(t));
+  const uint32_t j0 = 32 * rank / S, chunks = 32 * (rank + 1) / S - j0, items = args.M * chunks;
+  constexpr int kBatch = S > 4 ? 1 : 2;  // loads of kBatch x S partial chunks in flight per thread
+  for (uint32_t i0 = tid; i0 < items; i0 += 128 * kBatch) {
+    float4 v[kBatch][S];
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const uint32_t i = i0 + 128 * b, row = i / chunks, j = j0 + i - row * chunks;
+      if (i < items) {
+#pragma unroll
+        for (int t = 0; t < S; ++t) v[b][t] = ld_cluster_f4(base[t] + skinny_part_offset(row, j));
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < kBatch; ++b) {
+      const uint32_t i = i0 + 128 * b, row = i / chunks, j = j0 + i - row * chunks;
+      const int n = n0 + static_cast<int>(4 * j);
+      if (i >= items || n >= args.N) continue;  // N % 16 == 0: a chunk is inside or outside
+      float4 acc = v[b][0];
+#pragma unroll
+      for (int t = 1; t < S; ++t) {
+        acc.x += v[b][t].x;
+        acc.y += v[b][t].y;
+        acc.z += v[b][t].z;
+        acc.w += v[b][t].w;
+      }
+      if (in_bounds(args.status, row < static_cast<uint32_t>(args.M) && n + 4 <= args.N))
+        *reinterpret_cast<uint2*>(args.out + static_cast<int64_t>(row) * args.ldo + n) =
+            make_uint2(pack_bf16x2(acc.x * scale, acc.y * scale), pack_bf16x2(acc.z * scale, acc.w * scale));
+    }
+  }
+}
+
+template <class C>
+__global__ void __launch_bounds__(C::kThreads, 2)
+    nvfp4_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
+                             const GemmArgs args) {
+  constexpr int kStages = C::kStages;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sA = smem;  // the MMA's reads past a short A slot end inside sB
+  uint8_t* sB = sA + kStages * C::kTileBytesA;
+  uint8_t* sSFA = sB + kStages * C::kTileBytesB;
+  uint8_t* sSFB = sSFA + kStages * C::kSfBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(sSFB + kStages * C::kSfBytes);
+  uint64_t* empty = full + kStages;
+  uint64_t* sfready = empty + kStages;
+  uint64_t* tfull = sfready + kStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
+  __shared__ volatile int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int S = args.splits;
+  const int kblocks = args.K / BK;
+  const int split = static_cast<int>(cluster_ctarank());
+  const int nb = blockIdx.x / S;
+  const int k0 = split * kblocks / S, k1 = (split + 1) * kblocks / S;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+      mbar_init(&sfready[s], 1);
+    }
+    mbar_init(tfull, 1);
+    abort_flag = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tmap_a);
+    prefetch_tmap(&tmap_b);
+    for (int kb = k0; kb < min(k1, k0 + args.prefetch_kb); ++kb) tma_prefetch_2d(&tmap_b, kb * (BK / 2), nb * 128);
+  }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, C::kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  griddep_wait_and_release();
+  const uint32_t tmem = *tmem_slot;
+
+  auto fail = [&]() {
+    set_status(args.status, NVFP4_ERR_TIMEOUT);
+    abort_flag = 1;
+  };
+
+  bool have_partial = false;
+  if (warp == 0 && lane == 0) {
+    // ------------------------------------------------------ TMA producer ---
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t issued = 0, issued_parity = 0;  // one bit per stage
+    const uint8_t* sfb_tile = args.sfb + static_cast<size_t>(nb) * kblocks * C::kSfBytes;
+    const uint32_t bytes = static_cast<uint32_t>(args.a_box_rows) * (BK / 2) + C::kTileBytesB + 2 * C::kSfBytes;
+    for (int kb = k0; kb < k1; ++kb) {
+      if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
+      mbar_arrive_expect_tx(&full[stage], bytes);
+      bulk_load(sSFB + stage * C::kSfBytes, sfb_tile + static_cast<size_t>(kb) * C::kSfBytes, C::kSfBytes, &full[stage]);
+      tma_load_2d(sB + stage * C::kTileBytesB, &tmap_b, &full[stage], kb * (BK / 2), nb * 128);
+      bulk_load(sSFA + stage * C::kSfBytes, args.sfa + static_cast<size_t>(kb) * C::kSfBytes, C::kSfBytes, &full[stage]);
+      tma_load_2d(sA + stage * C::kTileBytesA, &tmap_a, &full[stage], kb * (BK / 2), 0);
+      issued |= 1u << stage;
+      issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+    if (abort_flag)
+      for (int s = 0; s < kStages; ++s)
+        if (issued >> s & 1u) mbar_wait_bounded(&full[s], issued_parity >> s & 1u, nullptr);
+  } else if (warp == 1 && lane == 0) {
+    // ------------------------------------------------------- MMA issuer ---
+    int stage = 0;
+    uint32_t phase = 0;
+    const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+    for (int kb = k0; kb < k1; ++kb) {
+      if (!mbar_wait_bounded(&sfready[stage], phase, &abort_flag)) { fail(); break; }
+      tc_fence_after();
+      const uint32_t sfa_col = tmem + C::kSfTmemCol + stage * 32, sfb_col = sfa_col + 16;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        mma_fp4(tmem, desc_sw128(sA0 + stage * C::kTileBytesA + kk * 32),
+                desc_sw128(sB0 + stage * C::kTileBytesB + kk * 32), C::kIdesc | args.idesc_fmt, sfa_col + kk * 4,
+                sfb_col + kk * 4, (kb != k0) | (kk != 0));
+      tc_commit(&empty[stage]);
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+    // Also on the timeout path: every MMA issued has retired before TMEM is freed.
+    tc_commit(tfull);
+    mbar_wait_bounded(tfull, 0, nullptr);
+  } else if (warp == 2 && lane == 0) {
+    int stage = 0;
+    uint32_t phase = 0;
+    const uint32_t sSFA0 = smem_u32(sSFA), sSFB0 = smem_u32(sSFB);
+    for (int kb = k0; kb < k1; ++kb) {
+      if (!mbar_wait_bounded(&full[stage], phase, &abort_flag)) { fail(); break; }
+      tc_fence_after();
+      const uint32_t sfa_col = tmem + C::kSfTmemCol + stage * 32, sfb_col = sfa_col + 16;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        copy_sf_to_tmem(sfa_col + kk * 4, desc_sf(sSFA0 + stage * C::kSfBytes + kk * 512));
+        copy_sf_to_tmem(sfb_col + kk * 4, desc_sf(sSFB0 + stage * C::kSfBytes + kk * 512));
+      }
+      tc_commit(&sfready[stage]);
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+  } else if (warp >= 3) {
+    // ------------------------------- drain the partial into shared memory ---
+    const int quarter = warp & 3;  // TMEM lanes this warp may access = accumulator rows
+    int ok = 1;
+    if (lane == 0) {
+      ok = mbar_wait_bounded(tfull, 0, &abort_flag) && !abort_flag;
+      if (!ok && !abort_flag) fail();
+    }
+    if (__shfl_sync(0xffffffffu, ok, 0)) {
+      tc_fence_after();
+      if (quarter * 32 < C::kRows) {
+        const uint32_t row = static_cast<uint32_t>(quarter * 32 + lane), part0 = smem_u32(smem);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t r[32];
+          tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c * 32, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            st_shared_v4(part0 + skinny_part_offset(row, static_cast<uint32_t>(8 * c + q)), r[4 * q], r[4 * q + 1],
+                         r[4 * q + 2], r[4 * q + 3]);
+        }
+      }
+      have_partial = true;
+    }
+  }
+
+  // Every CTA's partial is written (or its CTA gave up) before any is read.
+  tc_fence_before();
+  cluster_sync_all();
+  tc_fence_after();
+
+  if (warp >= 3 && !abort_flag && __all_sync(0xffffffffu, have_partial ? 1 : 0)) {
+    const float scale = args.ga ? __fmul_rn(__ldg(args.ga), __ldg(args.gb)) : 1.0f;
+    const uint32_t part0 = smem_u32(smem);
+    const uint32_t tid = threadIdx.x - 96;
+    const int n0 = nb * 128;
+    switch (S) {
+      case 1: skinny_reduce<1>(part0, split, tid, n0, scale, args); break;
+      case 2: skinny_reduce<2>(part0, split, tid, n0, scale, args); break;
+      case 3: skinny_reduce<3>(part0, split, tid, n0, scale, args); break;
+      case 4: skinny_reduce<4>(part0, split, tid, n0, scale, args); break;
+      case 5: skinny_reduce<5>(part0, split, tid, n0, scale, args); break;
+      case 6: skinny_reduce<6>(part0, split, tid, n0, scale, args); break;
+      case 7: skinny_reduce<7>(part0, split, tid, n0, scale, args); break;
+      default: skinny_reduce<8>(part0, split, tid, n0, scale, args); break;
+    }
+  }
+
+  // No CTA leaves while another may still read its partial.
+  cluster_sync_all();
+  if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
+}
+
 // ------------------------------------- quantize-in-prologue linear kernel ---
 // a1 + a2 + a3 in one launch for an activation of at most 32 rows and K of
 // at most 1536: every CTA reads the whole bf16 activation x (at most 96 KB,
@@ -1978,6 +2246,114 @@ nvfp4_status launch_splitk(const uint8_t* a_codes, const uint8_t* a_scales, cons
   return launch_status();
 }
 
+// Clusters of `size` CTAs of the skinny kernel resident on the GPU at once
+// (0 if that cluster shape cannot be launched).
+template <class C>
+int resident_skinny_clusters(int size) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> cache;
+  int d = 0;
+  if (cudaGetDevice(&d) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = cache.find({d, size});
+  if (it != cache.end()) return it->second;
+  int clusters = 0;
+  if (cudaFuncSetAttribute(nvfp4_gemm_skinny_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(C::kSmemBytes)) == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(size * (2 * sm_count() / size), 1, 1);
+    cfg.blockDim = dim3(C::kThreads, 1, 1);
+    cfg.dynamicSmemBytes = C::kSmemBytes;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&clusters, nvfp4_gemm_skinny_kernel<C>, &cfg) != cudaSuccess) clusters = 0;
+  }
+  cudaGetLastError();
+  cache[{d, size}] = clusters;
+  return clusters;
+}
+
+// CTAs per tile of the skinny kernel, or 0 where another kernel is faster.
+// The largest S <= 8 whose clusters are all resident at once: a second wave
+// costs more than a longer k-loop, and within one wave more CTAs stream
+// faster (1 row, 5120 x 13824, S = 1, 2, 4, 6, 7: 28.3, 18.5, 14.8, 13.4, 19.1
+// us with the activation's quantization; 27648 x 5120, S = 1, 2, 4: 18.5,
+// 22.7, 25.8).  More rows make the reduction dearer: above 32 rows S stays
+// at 4 unless each CTA keeps 4-5 k-blocks (128 rows, 1536 x 5120, S = 4, 8:
+// 12.2, 14.0; 1536 x 13824: 17.2, 14.9).
+// K <= 1536 is never split: nvfp4_linear_dynamic's sums are in one order.
+// Against the kernels for other shapes: unsplit with a short K and at most one
+// 128 x 128 tile per SM the single-CTA kernel is as fast (1536 x 2048: 8.3
+// against 8.2 us); with 65-128 rows A is half of what an SM takes in, and the
+// skinny kernel is ahead only when it splits by three or more (7168 x 5120:
+// 14.8 against 15.8 us; 14336 x 5120 by two: 17.9 against 17.0) or when the
+// last wave of single CTAs would be mostly empty (27648 x 5120, 216 tiles on
+// 152 SMs: 24.6 against 26.7; 55296 x 5120, 432 tiles: 45.8 against 38.3).
+template <class C>
+int choose_skinny_splits(int64_t tiles, int64_t kblocks) {
+  const int64_t sms = sm_count();
+  if (sms <= 0 || (C::kRows == 128 && kblocks <= 8)) return 0;
+  int best = 1;
+  if (kblocks > DynCfg::kMaxKb) {
+    const int64_t cap = C::kRows == 32 ? 8 : (C::kRows == 64 ? kblocks / 4 : kblocks / 5);
+    for (int s = 2; s <= 8 && s <= kblocks && s <= (cap < 4 ? 4 : cap); ++s)
+      if (tiles <= resident_skinny_clusters<C>(s)) best = s;
+  } else if (tiles <= sms) {
+    return 0;
+  }
+  if (C::kRows == 128 && (best == 2 || (best == 1 && 4 * ((tiles + sms - 1) / sms) * sms <= 5 * tiles))) return 0;
+  return best;
+}
+
+template <class C>
+nvfp4_status launch_skinny(const uint8_t* a_codes, const uint8_t* a_scales, const float* g_a, const uint8_t* w_codes,
+                           const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N, int64_t K, void* out_bf16,
+                           int64_t ldo, cudaStream_t stream, uint32_t idesc_fmt, int splits) {
+  const int64_t tiles_n = (N + 127) / 128;
+  if (resident_skinny_clusters<C>(splits) <= 0) return NVFP4_ERR_CUDA;  // also the shared-memory opt-in
+  if (tiles_n * splits >= (1ll << 31)) return NVFP4_ERR_SHAPE;
+  GemmArgs args = {};
+  args.a_box_rows = static_cast<int>((M + 7) & ~7ll);
+  CUtensorMap ma, mb;
+  if (!make_code_map(&ma, a_codes, M, K, args.a_box_rows) || !make_code_map(&mb, w_codes, N, K, 128))
+    return NVFP4_ERR_CUDA;
+  args.idesc_fmt = idesc_fmt;
+  args.sfa = a_scales;
+  args.sfb = w_scales;
+  args.ga = g_a;
+  args.gb = g_w;
+  args.M = static_cast<int>(M);
+  args.N = static_cast<int>(N);
+  args.K = static_cast<int>(K);
+  args.splits = splits;
+  args.prefetch_kb = kSkinnyPrefetch;
+  args.status = status_word_dev();
+  args.out = static_cast<uint16_t*>(out_bf16);
+  args.ldo = ldo;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = splits;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles_n * splits), 1, 1);
+  cfg.blockDim = dim3(C::kThreads, 1, 1);
+  cfg.dynamicSmemBytes = C::kSmemBytes;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, nvfp4_gemm_skinny_kernel<C>, ma, mb, args) != cudaSuccess) return NVFP4_ERR_CUDA;
+  count_launches(1);
+  return launch_status();
+}
+
 // nvfp4_linear_dynamic: one persistent CTA per 128-column tile of W, at most
 // one per SM.
 nvfp4_status launch_dynamic(const uint16_t* x, int64_t M, int64_t K, int64_t ldx, const uint8_t* w_codes,
@@ -2060,6 +2436,17 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
                              const uint8_t* w_codes, const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N,
                              int64_t K, void* out_bf16, int64_t ldo, cudaStream_t s, uint32_t idesc_fmt) {
   const int64_t tiles_m = (M + BM - 1) / BM;
+  if (tiles_m == 1) {
+    const int64_t tiles = (N + 127) / 128, kblocks = K / BK;
+    const int splits = M <= 32   ? choose_skinny_splits<SkinnyCfg<32>>(tiles, kblocks)
+                       : M <= 64 ? choose_skinny_splits<SkinnyCfg<64>>(tiles, kblocks)
+                                 : choose_skinny_splits<SkinnyCfg<128>>(tiles, kblocks);
+    const auto kernel = M <= 32   ? launch_skinny<SkinnyCfg<32>>
+                        : M <= 64 ? launch_skinny<SkinnyCfg<64>>
+                                  : launch_skinny<SkinnyCfg<128>>;
+    if (splits)
+      return kernel(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, idesc_fmt, splits);
+  }
   // The CTA pair, unless its 256 x 256 tiles would leave most pairs idle
   // (decode-sized M): then, with a long K, the split-K clusters, else 128 x
   // 128 tiles on single CTAs, which spread the W stream over more SMs than

@@ -322,3 +322,48 @@ def test_linear_swiglu_quantize_invalid_g_out_zeroes_and_reports(N):
     torch.cuda.synchronize()
     assert N.nvfp4_get_device_status() == 1
     assert not u8(out_c).any() and not u8(out_s).any()
+
+
+@pytest.mark.parametrize("M,Nn,K,ldo", [
+    # the skinny kernel (one row tile): A box and slot edges, N tails, each split, uneven K ranges
+    (1, 16, 1792, 16), (8, 112, 2048, 120), (9, 144, 2304, 144), (31, 272, 4864, 280), (32, 5136, 1792, 5136),
+    (33, 1536, 2304, 1536), (63, 2064, 4096, 2064), (64, 7168, 2560, 7168), (65, 1296, 5120, 1304),
+    (127, 10240, 2560, 10240), (128, 256, 10240, 256), (5, 14352, 2048, 14352), (17, 20000, 1536, 20000),
+    (128, 20480, 2304, 20480), (32, 28048, 1792, 28048), (1, 128, 27648, 128)])
+def test_skinny_shapes(N, M, Nn, K, ldo):
+    gen = torch.Generator().manual_seed(M * 1000 + Nn * 10 + K)
+    a_c, a_s = random_operand(M, K, gen)
+    w_c, w_s = random_operand(Nn, K, gen)
+    g_a, g_w = np.float32(0.0173), np.float32(0.00091)
+    out = run_linear(N, a_c, a_s, g_a, w_c, w_s, g_w, M, Nn, K, ldo=ldo)
+    ref = O.linear(a_c, a_s, g_a, w_c, w_s, g_w)
+    assert_close(f32(out[:, :Nn]), ref, what=f"{M}x{Nn}x{K}")
+    assert torch.isnan(out[:, Nn:].float()).all()
+    again = run_linear(N, a_c, a_s, g_a, w_c, w_s, g_w, M, Nn, K, ldo=ldo)
+    assert torch.equal(out[:, :Nn], again[:, :Nn])
+
+
+def test_skinny_reads_a_weight_written_by_the_kernel_before_it(N):
+    """The skinny kernel prefetches W into L2 before the preceding kernel has
+    finished; a W that this kernel writes must be read as written."""
+    M, Nn, K = 4, 7168, 2560
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(M, K, generator=gen, device="cuda").to(torch.bfloat16)
+    ws = [(torch.randn(Nn, K, generator=gen, device="cuda") * s).to(torch.bfloat16) for s in (0.02, 0.5)]
+    new = lambda *s, dtype=torch.uint8: torch.zeros(*s, dtype=dtype, device="cuda")  # noqa: E731
+    ac, asf, g = new(M, K // 2), new(N.nvfp4_scales_bytes(M, K, 1)), new(1, dtype=torch.float32)
+    wc, wsf, gw = new(Nn, K // 2), new(N.nvfp4_scales_bytes(Nn, K, 1)), new(1, dtype=torch.float32)
+    outs = [new(M, Nn, dtype=torch.bfloat16) for _ in range(4)]
+    N.nvfp4_tensor_scale(x, g)
+    N.nvfp4_quantize(x, g, ac, asf)
+    gw.fill_(0.001)
+    for i in range(4):
+        if i >= 2:
+            torch.cuda.synchronize()
+        N.nvfp4_quantize(ws[i % 2], gw, wc, wsf)
+        if i >= 2:
+            torch.cuda.synchronize()
+        N.nvfp4_linear(ac, asf, g, wc, wsf, gw, outs[i], M, Nn, K)
+    torch.cuda.synchronize()
+    assert N.nvfp4_get_device_status() == 0
+    assert torch.equal(outs[0], outs[2]) and torch.equal(outs[1], outs[3]) and not torch.equal(outs[0], outs[1])
