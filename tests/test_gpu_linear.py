@@ -268,7 +268,9 @@ def swiglu_case(N, M, I, K, seed, rows=None):
     return h, g_out, rows, u8(out_c), u8(out_s), swiglu_tolerance(G, U, h)
 
 
-@pytest.mark.parametrize("M,I,K", [(256, 128, 256), (129, 384, 512), (300, 256, 1024), (640, 512, 768)])
+@pytest.mark.parametrize("M,I,K", [(256, 128, 256), (129, 384, 512), (300, 256, 1024), (640, 512, 768),
+                                  # last waves in half tiles (76 pairs): 78 and 40 + 76 tiles
+                                  (300, 4992, 768), (256, 14848, 512)])
 def test_linear_swiglu_quantize(N, M, I, K):
     """h = SiLU(gate) * up from the fp32 accumulators, quantized with a static
     scale.  The kernel's SiLU uses the hardware tanh approximation, so every
@@ -367,3 +369,18 @@ def test_skinny_reads_a_weight_written_by_the_kernel_before_it(N):
     torch.cuda.synchronize()
     assert N.nvfp4_get_device_status() == 0
     assert torch.equal(outs[0], outs[2]) and torch.equal(outs[1], outs[3]) and not torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("M,Nn,K", [
+    # last waves whose tiles are split into 256 x 128 halves (76 pairs): only halves, after one
+    # full wave, with M tails and a spare CTA, two k-blocks and more than the ring's
+    (256, 9728, 512), (300, 9984, 768), (256, 27648, 1024), (1000, 5120, 2048), (130, 19712, 1792)])
+def test_last_wave_in_half_tiles(N, M, Nn, K):
+    gen = torch.Generator().manual_seed(M * 1000 + Nn * 10 + K)
+    a_c, a_s = random_operand(M, K, gen)
+    w_c, w_s = random_operand(Nn, K, gen)
+    g_a, g_w = np.float32(0.0173), np.float32(0.00091)
+    out = run_linear(N, a_c, a_s, g_a, w_c, w_s, g_w, M, Nn, K, ldo=Nn + 8)
+    ref = O.linear(a_c, a_s, g_a, w_c, w_s, g_w)
+    assert_close(f32(out[:, :Nn]), ref, what=f"{M}x{Nn}x{K}")
+    assert torch.isnan(out[:, Nn:].float()).all()
