@@ -1417,30 +1417,31 @@ __global__ void __launch_bounds__(C::kThreads, 1)
 // (one's set-up, drain and reduction under the other's stream).  The A box
 // carries only the M rows rounded up to 8; the MMA's 128 A rows read on into
 // whatever follows in shared memory, which only reaches accumulator rows that
-// are never stored (E2M1 codes are finite, and padding rows have zero scales).
-// One thread issues a k-block's scale copies and then its MMAs: the tensor
-// core runs copy -> MMA of one thread in order, so no barrier lies between.
+// are never stored.
 // The S fp32 partials ([rows, 128], 512-byte rows with swizzled 16-byte
 // chunks, in the idle ring) are added across the cluster in split order, each
 // CTA taking a share of the columns: deterministic for a given shape.
-//   warp 0  TMA producer; before it waits for the previous kernel it
-//           prefetches its first W k-blocks into L2, while the activation is
-//           still being quantized (a prefetch of something that kernel writes
-//           would be harmless: L2 is the point of coherence)
+//   warp 0  TMA producer of the codes; before it waits for the previous kernel
+//           it prefetches its first W k-blocks into L2, while the activation
+//           is still being quantized (a prefetch of something that kernel
+//           writes would be harmless: L2 is the point of coherence)
 //   warp 1  TMEM allocation, MMAs
-//   warp 2  scale copies into TMEM, ahead of the MMAs (one thread doing both
-//           in order was 10-20 % slower per k-block)
-//   warps 3-6  drain, reduction, stores
+//   warp 2  scale copies into TMEM, ahead of the MMAs
+//   warp 3  producer of the block scales
+//   warps 4-7  drain, reduction, stores
+// Each role is a converged warp that issues through one elected lane, as in
+// the pair kernel.
 // Measured with the activation's quantization before it (graph replay, W from
 // DRAM), against the kernels that served these shapes before, 1 row: 5120 x
-// 5120 13.6 -> 8.6 us, 7168 x 5120 14.5 -> 9.2, 27648 x 5120 31.1 -> 18.5 (W's
-// bytes at the copy rate: 11.7), 5120 x 13824 23.1 -> 13.4.
+// 5120 13.6 -> 8.3 us, 7168 x 5120 14.5 -> 8.9, 27648 x 5120 31.1 -> 17.3 (W's
+// bytes at the copy rate: 11.7), 5120 x 13824 23.1 -> 12.8; 32 rows: 14.6 ->
+// 11.3, 15.1 -> 12.0, 29.4 -> 19.7, 19.5 -> 14.8.
 template <int ROWS_>
 struct SkinnyCfg {
   static constexpr int kRows = ROWS_;                      // A rows held per k-block: 32, 64 or 128
   static constexpr int kStages = ROWS_ == 32 ? 4 : 3;
   static constexpr int kEpiWarps = 4;
-  static constexpr int kThreads = 96 + 32 * kEpiWarps;
+  static constexpr int kThreads = 128 + 32 * kEpiWarps;
   static constexpr uint32_t kTileBytesA = kRows * BK / 2;
   static constexpr uint32_t kTileBytesB = 128 * BK / 2;
   static constexpr uint32_t kSfBytes = 128 * (BK / 16);    // of A and of W: four 512-byte atoms
@@ -1523,8 +1524,8 @@ __global__ void __launch_bounds__(C::kThreads, 2)
   uint8_t* sSFB = sSFA + kStages * C::kSfBytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(sSFB + kStages * C::kSfBytes);
   uint64_t* empty = full + kStages;
-  uint64_t* sfready = empty + kStages;
-  uint64_t* tfull = sfready + kStages;
+  uint64_t* sffull = empty + kStages;
+  uint64_t* tfull = sffull + kStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
   __shared__ volatile int abort_flag;
 
@@ -1537,9 +1538,9 @@ __global__ void __launch_bounds__(C::kThreads, 2)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], 1);
+      mbar_init(&full[s], 2);  // the codes' expect_tx, and the commit of the scale copies
       mbar_init(&empty[s], 1);
-      mbar_init(&sfready[s], 1);
+      mbar_init(&sffull[s], 1);
     }
     mbar_init(tfull, 1);
     abort_flag = 0;
@@ -1564,64 +1565,90 @@ __global__ void __launch_bounds__(C::kThreads, 2)
   };
 
   bool have_partial = false;
-  if (warp == 0 && lane == 0) {
-    // ------------------------------------------------------ TMA producer ---
+  // Walks this CTA's k-blocks: load(stage, kb) in one lane once `free` allows.
+  auto produce = [&](uint64_t* free, auto&& load) {
+    const bool issuer = elect_one();
     int stage = 0;
     uint32_t phase = 0;
-    uint32_t issued = 0, issued_parity = 0;  // one bit per stage
-    const uint8_t* sfb_tile = args.sfb + static_cast<size_t>(nb) * kblocks * C::kSfBytes;
-    const uint32_t bytes = static_cast<uint32_t>(args.a_box_rows) * (BK / 2) + C::kTileBytesB + 2 * C::kSfBytes;
     for (int kb = k0; kb < k1; ++kb) {
-      if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
+      if (!mbar_wait_bounded(&free[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
+      if (issuer) load(stage, kb);
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+    if (abort_flag) drain_delay();
+  };
+  if (warp == 0) {
+    // ------------------------------------------------------ producer: codes ---
+    const uint32_t bytes = static_cast<uint32_t>(args.a_box_rows) * (BK / 2) + C::kTileBytesB;
+    produce(empty, [&](int stage, int kb) {
       mbar_arrive_expect_tx(&full[stage], bytes);
-      bulk_load(sSFB + stage * C::kSfBytes, sfb_tile + static_cast<size_t>(kb) * C::kSfBytes, C::kSfBytes, &full[stage]);
       tma_load_2d(sB + stage * C::kTileBytesB, &tmap_b, &full[stage], kb * (BK / 2), nb * 128);
-      bulk_load(sSFA + stage * C::kSfBytes, args.sfa + static_cast<size_t>(kb) * C::kSfBytes, C::kSfBytes, &full[stage]);
       tma_load_2d(sA + stage * C::kTileBytesA, &tmap_a, &full[stage], kb * (BK / 2), 0);
-      issued |= 1u << stage;
-      issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-      if (++stage == kStages) { stage = 0; phase ^= 1u; }
-    }
-    if (abort_flag)
-      for (int s = 0; s < kStages; ++s)
-        if (issued >> s & 1u) mbar_wait_bounded(&full[s], issued_parity >> s & 1u, nullptr);
-  } else if (warp == 1 && lane == 0) {
+    });
+  } else if (warp == 3) {
+    // ----------------------------------------------------- producer: scales ---
+    // A stage's scale buffers are free once the previous copies have read
+    // them, which its `full` phase includes.
+    const uint8_t* sfb_tile = args.sfb + static_cast<size_t>(nb) * kblocks * C::kSfBytes;
+    produce(full, [&](int stage, int kb) {
+      const size_t off = static_cast<size_t>(kb) * C::kSfBytes;
+      mbar_arrive_expect_tx(&sffull[stage], 2 * C::kSfBytes);
+      bulk_load(sSFB + stage * C::kSfBytes, sfb_tile + off, C::kSfBytes, &sffull[stage]);
+      bulk_load(sSFA + stage * C::kSfBytes, args.sfa + off, C::kSfBytes, &sffull[stage]);
+    });
+  } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer ---
+    const bool issuer = elect_one();
     int stage = 0;
     uint32_t phase = 0;
-    const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
-    for (int kb = k0; kb < k1; ++kb) {
-      if (!mbar_wait_bounded(&sfready[stage], phase, &abort_flag)) { fail(); break; }
-      tc_fence_after();
-      const uint32_t sfa_col = tmem + C::kSfTmemCol + stage * 32, sfb_col = sfa_col + 16;
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
-        mma_fp4(tmem, desc_sw128(sA0 + stage * C::kTileBytesA + kk * 32),
-                desc_sw128(sB0 + stage * C::kTileBytesB + kk * 32), C::kIdesc | args.idesc_fmt, sfa_col + kk * 4,
-                sfb_col + kk * 4, (kb != k0) | (kk != 0));
-      tc_commit(&empty[stage]);
-      if (++stage == kStages) { stage = 0; phase ^= 1u; }
-    }
-    // Also on the timeout path: every MMA issued has retired before TMEM is freed.
-    tc_commit(tfull);
-    mbar_wait_bounded(tfull, 0, nullptr);
-  } else if (warp == 2 && lane == 0) {
-    int stage = 0;
-    uint32_t phase = 0;
-    const uint32_t sSFA0 = smem_u32(sSFA), sSFB0 = smem_u32(sSFB);
+    const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint64_t a_desc0 = desc_sw128(smem_u32(sA)), b_desc0 = desc_sw128(smem_u32(sB));
     for (int kb = k0; kb < k1; ++kb) {
       if (!mbar_wait_bounded(&full[stage], phase, &abort_flag)) { fail(); break; }
       tc_fence_after();
-      const uint32_t sfa_col = tmem + C::kSfTmemCol + stage * 32, sfb_col = sfa_col + 16;
+      const uint32_t sfa_col = utmem + C::kSfTmemCol + stage * 32, sfb_col = sfa_col + 16;
+      const uint64_t a_desc = a_desc0 + static_cast<uint32_t>(stage) * (C::kTileBytesA >> 4);
+      const uint64_t b_desc = b_desc0 + static_cast<uint32_t>(stage) * (C::kTileBytesB >> 4);
+      if (issuer) {
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        copy_sf_to_tmem(sfa_col + kk * 4, desc_sf(sSFA0 + stage * C::kSfBytes + kk * 512));
-        copy_sf_to_tmem(sfb_col + kk * 4, desc_sf(sSFB0 + stage * C::kSfBytes + kk * 512));
+        for (int kk = 0; kk < 4; ++kk)
+          mma_fp4(utmem, a_desc + 2 * kk, b_desc + 2 * kk, C::kIdesc | args.idesc_fmt, sfa_col + kk * 4,
+                  sfb_col + kk * 4, (kb != k0) | (kk != 0));
+        tc_commit(&empty[stage]);
       }
-      tc_commit(&sfready[stage]);
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
     }
-  } else if (warp >= 3) {
+    // Also on the timeout path: every MMA issued has retired before TMEM is freed.
+    if (issuer) tc_commit(tfull);
+    mbar_wait_bounded(tfull, 0, nullptr);
+  } else if (warp == 2) {
+    // ---------------------------------------------- block scales -> TMEM ---
+    const bool issuer = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint64_t sfa_desc0 = desc_sf(smem_u32(sSFA)), sfb_desc0 = desc_sf(smem_u32(sSFB));
+    for (int kb = k0; kb < k1; ++kb) {
+      // The scales have landed, and the MMAs that read this TMEM slot are done.
+      if (!mbar_wait_bounded(&sffull[stage], phase, &abort_flag) ||
+          !mbar_wait_bounded(&empty[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
+      tc_fence_after();
+      const uint32_t sfa_col = utmem + C::kSfTmemCol + stage * 32, sfb_col = sfa_col + 16;
+      const uint64_t off = static_cast<uint32_t>(stage) * (C::kSfBytes >> 4);
+      if (issuer) {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          copy_sf_to_tmem(sfa_col + kk * 4, sfa_desc0 + off + kk * (512 >> 4));
+          copy_sf_to_tmem(sfb_col + kk * 4, sfb_desc0 + off + kk * (512 >> 4));
+        }
+        tc_commit(&full[stage]);
+      }
+      if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    }
+    // The MMAs that read the last copies are waited for above; on the timeout
+    // path copies may be in flight still.
+    if (abort_flag) drain_delay();
+  } else if (warp >= 4) {
     // ------------------------------- drain the partial into shared memory ---
     const int quarter = warp & 3;  // TMEM lanes this warp may access = accumulator rows
     int ok = 1;
@@ -1653,10 +1680,10 @@ __global__ void __launch_bounds__(C::kThreads, 2)
   cluster_sync_all();
   tc_fence_after();
 
-  if (warp >= 3 && !abort_flag && __all_sync(0xffffffffu, have_partial ? 1 : 0)) {
+  if (warp >= 4 && !abort_flag && __all_sync(0xffffffffu, have_partial ? 1 : 0)) {
     const float scale = args.ga ? __fmul_rn(__ldg(args.ga), __ldg(args.gb)) : 1.0f;
     const uint32_t part0 = smem_u32(smem);
-    const uint32_t tid = threadIdx.x - 96;
+    const uint32_t tid = threadIdx.x - 128;
     const int n0 = nb * 128;
     switch (S) {
       case 1: skinny_reduce<1>(part0, split, tid, n0, scale, args); break;
@@ -2343,7 +2370,11 @@ nvfp4_status launch_splitk(const uint8_t* a_codes, const uint8_t* a_scales, cons
 }
 
 // Clusters of `size` CTAs of the skinny kernel resident on the GPU at once
-// (0 if that cluster shape cannot be launched).
+// (0 if that cluster shape cannot be launched).  The occupancy query counts
+// one CTA of a kernel that allocates TMEM per SM; two of these share one (256
+// of 512 columns each, and their shared memory fits).  Timing agrees: the
+// step from one wave to two lies at twice the query's figures (92 clusters of
+// 3, 72 of 4, 56 of 5, 46 of 6).
 template <class C>
 int resident_skinny_clusters(int size) {
   static std::mutex mu;
@@ -2367,7 +2398,13 @@ int resident_skinny_clusters(int size) {
     cfg.dynamicSmemBytes = C::kSmemBytes;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&clusters, nvfp4_gemm_skinny_kernel<C>, &cfg) != cudaSuccess) clusters = 0;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, nvfp4_gemm_skinny_kernel<C>, &cfg) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nvfp4_gemm_skinny_kernel<C>, C::kThreads,
+                                                      C::kSmemBytes) != cudaSuccess)
+      clusters = 0;
+    else if (per_sm == 1)
+      clusters *= 2;
   }
   cudaGetLastError();
   cache[{d, size}] = clusters;
@@ -2379,7 +2416,7 @@ int resident_skinny_clusters(int size) {
 // costs more than a longer k-loop, and within one wave more CTAs stream
 // faster (1 row, 5120 x 13824, S = 1, 2, 4, 6, 7: 28.3, 18.5, 14.8, 13.4, 19.1
 // us with the activation's quantization; 27648 x 5120, S = 1, 2, 4: 18.5,
-// 22.7, 25.8).  More rows make the reduction dearer: above 32 rows S stays
+// 22.7, 25.8, before the scales had a producer of their own).  More rows make the reduction dearer: above 32 rows S stays
 // at 4 unless each CTA keeps 4-5 k-blocks (128 rows, 1536 x 5120, S = 4, 8:
 // 12.2, 14.0; 1536 x 13824: 17.2, 14.9).
 // K <= 1536 is never split: nvfp4_linear_dynamic's sums are in one order.
