@@ -1,10 +1,10 @@
 // a5: decode attention straight from the NVFP4 KV cache (Sec. 2.1:
 // z = softmax(Q K_hat^T / sqrt(d)) V_hat with quantized K and V).
 //
-// Split-KV ("flash-decoding") with persistent CTAs.  A work item is one
-// (sequence, KV head, 1024-token chunk).  Each CTA has a producer warp that
-// streams the items' FP4 K/V codes and E4M3 scales into a 2-stage ring of
-// 128-token stages with 1-D bulk copies (the ring runs on across items), and
+// Split-KV ("flash-decoding").  The cached tokens of all sequences and KV heads
+// are one list of 128-token stages, cut into equal runs, one per resident CTA
+// (struct Walk).  Each CTA has a producer warp that streams its run's FP4 K/V
+// codes and E4M3 scales into a 2-stage ring with 1-D bulk copies, and
 // four consumer warps that each take two 16-token tiles of every stage (one
 // barrier hand-off per two tiles; measured faster than 4 x 64-token stages).  A consumer
 // dequantizes in registers (cvt e2m1x2 -> f16x2, times the E4M3 block scale:
@@ -14,8 +14,8 @@
 // The up to 8 query heads that share a KV head (grouped-query attention) fill
 // the MMA's N = 8.  Softmax is online, in fp32, in the log2 domain, with lazy
 // rescaling (the running max moves only when a tile exceeds it by 2^8).  At
-// the end of an item the four warps merge their partial (max, sum, O) and
-// write one record; a combine kernel merges the records of all chunks.
+// the end of a (sequence, head) or of the run the four warps merge their
+// partial (max, sum, O) and write one record; a combine kernel merges them.
 //
 // Lane roles (g = lane/4, t = lane%4), fixed by the m16n8k16 fragment layouts:
 //   K: rows g and g+8 of the S tile, channels 32t..32t+31 (16 bytes, blocks 2t, 2t+1)
@@ -38,8 +38,8 @@ namespace nvfp4 {
 namespace {
 
 constexpr int kD = 128;
-constexpr int kChunk = 1024;          // tokens per work item
-constexpr int kStageTok = 128;        // tokens per ring stage
+constexpr int kStageTok = 128;        // tokens per ring stage: the unit of work
+constexpr int kChunk = 1024;          // the workspace holds at least one record per 1024 tokens and head
 #ifndef NVFP4_ATTN_STAGES
 #define NVFP4_ATTN_STAGES 2
 #endif
@@ -50,8 +50,13 @@ constexpr int kStages = NVFP4_ATTN_STAGES;  // 2 x 18 KiB ring + merge buffer: 4
 constexpr int kConsumers = 4;         // consumer warps, 16 tokens of a stage each
 constexpr int kThreads = 32 * (1 + kConsumers);
 constexpr uint32_t kStageBytes = kStageTok * (64 + 8) * 2;  // K, V codes + scales: 18 KiB
-static_assert(kChunk % kStageTok == 0 && kStageTok % (16 * kConsumers) == 0, "stage tiling");
+static_assert(kStageTok % (16 * kConsumers) == 0, "stage tiling");
 constexpr uint32_t kOffKc = 0, kOffVc = kStageTok * 64, kOffKs = 2 * kStageTok * 64, kOffVs = kOffKs + kStageTok * 8;
+// Merge buffer: a head's channels with 2 floats of padding per 16, and heads
+// 148 floats apart, so that a half-warp's 8-byte stores (4 channel groups, 4
+// heads) meet 16 different bank pairs.
+constexpr int kMergeHead = 148;
+__device__ __forceinline__ int merge_channel(int c) { return c + 2 * (c >> 4); }
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleLog2 = 8.0f;  // lazy rescale threshold (P stays <= 2^8 in f16)
 
@@ -153,24 +158,6 @@ __device__ __forceinline__ void named_barrier_consumers() {
 // Token of row / k index m (0..15) of a 16-token tile.
 __device__ __forceinline__ int tile_tok(int m) { return (m & 1) * 4 + ((m >> 1) & 3) + (m & 8); }
 
-struct Item {
-  int b, kvh, split, t_begin, t_end;
-};
-
-__device__ __forceinline__ Item decode_item(int item, int n_splits, int hkv, const int32_t* __restrict__ seq_lens,
-                                            int capacity) {
-  Item it;
-  it.split = item % n_splits;
-  const int rest = item / n_splits;
-  it.kvh = rest % hkv;
-  it.b = rest / hkv;
-  int len = __ldg(seq_lens + it.b);
-  len = max(0, min(len, capacity));
-  it.t_begin = it.split * kChunk;
-  it.t_end = min(it.t_begin + kChunk, len);
-  return it;
-}
-
 struct Params {
   const uint8_t* k_codes;
   const uint8_t* k_scales;
@@ -181,9 +168,115 @@ struct Params {
   float* o_ws;
   float* ml_ws;
   int* status;
-  int hkv, capacity, hq, group, n_splits, n_items;
+  int batch, hkv, capacity, hq, group, records, whole;
   float logit_mult;  // softmax_scale * g_K * log2(e)
   int fault_skip_stage;  // test-only: CTA 0's producer leaves its first stage unissued
+};
+
+// Which stages (128 cached tokens of one sequence and KV head) a CTA takes.
+// The stages of all sequences and heads, sequence-major, are one list of T;
+// CTA c takes stages c R .. c R + R - 1, so every CTA has the same work
+// whatever the lengths.  A (sequence, head)'s s stages then lie with at most
+// (s - 2) / R + 2 CTAs in a row, each of which leaves one record of it; R is
+// at least what keeps that within the workspace's `records` per head.  Where
+// `whole` (room for one record only, or no head longer than a stage), a CTA
+// takes whole (sequence, head)s instead and no lengths need be summed.
+struct Segment {  // a run of stages of one (sequence, KV head)
+  int b, kvh, record, t_begin, t_end;
+  bool last;  // of its (sequence, head)
+};
+
+__device__ __forceinline__ int cached_tokens(const Params& p, int b) {
+  return max(0, min(__ldg(p.seq_lens + b), p.capacity));
+}
+__device__ __forceinline__ uint32_t stages_of(int tokens) {
+  return static_cast<uint32_t>(tokens + kStageTok - 1) / kStageTok;
+}
+
+struct Walk {
+  uint32_t R;        // stages per CTA; 0: whole (sequence, head)s
+  uint32_t at, end;  // next stage and end of this CTA's run; or (sequence, head)s
+  uint32_t before;   // stages before sequence b
+  int b;
+
+  // By one converged warp.
+  __device__ __forceinline__ void start(const Params& p) {
+    if (p.whole) {
+      R = 0;
+      at = blockIdx.x;
+      end = static_cast<uint32_t>(p.batch) * p.hkv;
+      return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int per = (p.batch + 31) / 32, b0 = min(p.batch, lane * per), b1 = min(p.batch, b0 + per);
+    uint32_t sum = 0, most = 0;
+    for (int i = b0; i < b1; ++i) {
+      const uint32_t s = stages_of(cached_tokens(p, i));
+      sum += s;
+      most = max(most, s);
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    uint32_t incl = sum * p.hkv;  // stages up to this lane's last sequence
+#pragma unroll
+    for (int sh = 1; sh < 32; sh <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, sh);
+      if (lane >= sh) incl += v;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    R = max(1u, (total + gridDim.x - 1) / gridDim.x);
+    if (most > R && most <= R + 2) R = most;  // equal lengths: no run crosses a head
+    if (most > 1) R = max(R, (most + p.records - 3) / (p.records - 1));
+    at = min(blockIdx.x * R, total);
+    end = min(at + R, total);
+    // The lane whose sequences hold the first stage looks for its sequence.
+    uint32_t first = incl - sum * p.hkv;
+    int found = p.batch;
+    if (at >= first && at < incl) {
+      for (found = b0; found < b1; ++found) {
+        const uint32_t n = stages_of(cached_tokens(p, found)) * p.hkv;
+        if (at < first + n) break;
+        first += n;
+      }
+    }
+    const uint32_t owner = __ballot_sync(0xffffffffu, found < p.batch);
+    const int src = owner ? __ffs(owner) - 1 : 0;
+    b = __shfl_sync(0xffffffffu, found, src);
+    before = __shfl_sync(0xffffffffu, first, src);
+  }
+
+  __device__ __forceinline__ bool next(const Params& p, Segment* s) {
+    if (R == 0) {
+      if (at >= end) return false;
+      s->b = static_cast<int>(at) / p.hkv;
+      s->kvh = static_cast<int>(at) - s->b * p.hkv;
+      s->record = 0;
+      s->last = true;
+      s->t_begin = 0;
+      s->t_end = cached_tokens(p, s->b);
+      at += gridDim.x;
+      return true;
+    }
+    while (at < end && b < p.batch) {
+      const int len = cached_tokens(p, b);
+      const uint32_t n = stages_of(len);
+      if (at >= before + n * p.hkv) {
+        before += n * p.hkv;
+        ++b;
+        continue;
+      }
+      s->b = b;
+      s->kvh = static_cast<int>((at - before) / n);
+      const uint32_t first = before + s->kvh * n;  // the head's first stage
+      const uint32_t st = at - first, count = min(n - st, end - at);
+      s->record = static_cast<int>(blockIdx.x - first / R);
+      s->last = st + count == n;
+      s->t_begin = static_cast<int>(st) * kStageTok;
+      s->t_end = min(s->t_begin + static_cast<int>(count) * kStageTok, len);
+      at += count;
+      return true;
+    }
+    return false;
+  }
 };
 
 // kE1M2: the cache holds E1M2 elements (decoded to n, the scale carries 1/2).
@@ -191,8 +284,8 @@ template <bool kE1M2>
 __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_kernel(const Params p) {
   extern __shared__ __align__(128) uint8_t smem[];
   uint8_t* ring = smem;
-  float* sh_o = reinterpret_cast<float*>(smem + kStages * kStageBytes);  // [kConsumers][8][128]
-  float* sh_m = sh_o + kConsumers * 8 * kD;                              // [kConsumers][8]
+  float* sh_o = reinterpret_cast<float*>(smem + kStages * kStageBytes);  // [kConsumers][8][merge_channel(128)]
+  float* sh_m = sh_o + kConsumers * 8 * kMergeHead;                      // [kConsumers][8]
   float* sh_l = sh_m + kConsumers * 8;
   uint64_t* full = reinterpret_cast<uint64_t*>(sh_l + kConsumers * 8);
   uint64_t* empty = full + kStages;
@@ -209,11 +302,13 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
   }
   __syncthreads();
   griddep_wait_and_release();
-  if (p.capacity > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
-    for (int b = 0; b < p.n_items / (p.n_splits * p.hkv); ++b)
-      if (__ldg(p.seq_lens + b) > p.capacity) { set_status(p.status, NVFP4_ERR_CAPACITY); break; }
-  }
+  if (blockIdx.x == 0)
+    for (int b = threadIdx.x; b < p.batch; b += kThreads)
+      if (__ldg(p.seq_lens + b) > p.capacity) set_status(p.status, NVFP4_ERR_CAPACITY);
 
+  Walk walk;
+  walk.start(p);
+  Segment it;
   if (warp == 0) {
     // ------------------------------------------------------------ producer ---
     if (lane == 0) {
@@ -223,8 +318,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       bool issued[kStages];
       for (int s = 0; s < kStages; ++s) issued[s] = false;
       bool skip_stage = p.fault_skip_stage && blockIdx.x == 0;
-      for (int item = blockIdx.x; item < p.n_items && !abort_flag; item += gridDim.x) {
-        const Item it = decode_item(item, p.n_splits, p.hkv, p.seq_lens, p.capacity);
+      while (!abort_flag && walk.next(p, &it)) {
         const size_t row0 = (static_cast<size_t>(it.b) * p.hkv + it.kvh) * p.capacity;
         for (int t0 = it.t_begin; t0 < it.t_end; t0 += kStageTok) {
           const int n = min(kStageTok, it.t_end - t0);
@@ -267,8 +361,17 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
   const int rv[4] = {tile_tok(2 * t), tile_tok(2 * t + 1), tile_tok(2 * t + 8), tile_tok(2 * t + 9)};  // V rows
   int stage = 0;
   uint32_t phase = 0;
-  for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
-    const Item it = decode_item(item, p.n_splits, p.hkv, p.seq_lens, p.capacity);
+  if (blockIdx.x == 0) {  // sequences without tokens have no segment
+    for (int b = threadIdx.x - 32; b < p.batch; b += 32 * kConsumers) {
+      if (__ldg(p.seq_lens + b) > 0) continue;
+      float* ml = p.ml_ws + static_cast<size_t>(b) * p.hq * p.records * 2;
+      for (int i = 0; i < p.hq * p.records; ++i) {
+        ml[2 * i] = -INFINITY;
+        ml[2 * i + 1] = 0.0f;
+      }
+    }
+  }
+  while (walk.next(p, &it)) {
     // Queries of head slot g: f16 after an exact power-of-two scaling that
     // keeps |q| < 1; the scaling is undone in the logit multiplier.
     const bool head_live = g < p.group;
@@ -333,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       for (int sub = 0; sub < kStageTok / (16 * kConsumers); ++sub) {
       const int r0 = 16 * (cw + kConsumers * sub);  // this warp's tile within the stage
       const int tile = t0 + r0;
-      const int valid = it.t_end - tile;  // tokens of this warp's tile inside the item (may be <= 0)
+      const int valid = it.t_end - tile;  // tokens of this warp's tile inside the segment (may be <= 0)
       if (valid > 0) {
         // ---- S^T = K_hat Q^T: 8 k-steps of 16 channels ---------------------
         const uint4 ka = *reinterpret_cast<const uint4*>(st + kOffKc + (r0 + rk0) * 64 + 16 * t);
@@ -371,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
           vs01_raw = s0 | (s1 << 8);
           vs89_raw = s2 | (s3 << 8);
         }
-        if (valid < 16) {  // ragged end of the item: mask keys, zero the scales of absent values
+        if (valid < 16) {  // ragged end of the segment: mask keys, zero the scales of absent values
           if (rk0 >= valid) x0 = x1 = -INFINITY;
           if (rk1 >= valid) x2 = x3 = -INFINITY;
           if (rv[0] >= valid) vs01_raw &= 0xFF00u;
@@ -454,21 +557,19 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
     }
 
-    // ---- merge the consumer warps, write this item's partial --------------
+    // ---- merge the consumer warps, write this segment's record ------------
     l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 4);
     l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 4);
     l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 8);
     l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 8);
     l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 16);
     l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 16);
-    float* my_o = sh_o + cw * 8 * kD;
+    float* my_o = sh_o + cw * 8 * kMergeHead;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int c0 = 16 * g + 2 * i;  // channel of accumulator rows g / g+8 of m-tile i
-      my_o[(2 * t) * kD + c0] = o[i][0];
-      my_o[(2 * t + 1) * kD + c0] = o[i][1];
-      my_o[(2 * t) * kD + c0 + 1] = o[i][2];
-      my_o[(2 * t + 1) * kD + c0 + 1] = o[i][3];
+      const int c0 = merge_channel(16 * g + 2 * i);  // channels of accumulator rows g and g+8 of m-tile i
+      *reinterpret_cast<float2*>(my_o + (2 * t) * kMergeHead + c0) = make_float2(o[i][0], o[i][2]);
+      *reinterpret_cast<float2*>(my_o + (2 * t + 1) * kMergeHead + c0) = make_float2(o[i][1], o[i][3]);
     }
     if (g == 0) {
       sh_m[cw * 8 + 2 * t] = m_run[0]; sh_m[cw * 8 + 2 * t + 1] = m_run[1];
@@ -485,18 +586,27 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
 #pragma unroll
         for (int w = 0; w < kConsumers; ++w) {
           const float wt = fast_exp2(sh_m[w * 8 + h] - M);
-          acc += wt * sh_o[(w * 8 + h) * kD + c];
+          acc += wt * sh_o[(w * 8 + h) * kMergeHead + merge_channel(c)];
           L += wt * sh_l[w * 8 + h];
         }
       }
-      const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.n_splits + it.split;
+      const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.records + it.record;
       p.o_ws[rec * kD + c] = acc;
       if (c == 0) {
         p.ml_ws[rec * 2] = M;
         p.ml_ws[rec * 2 + 1] = L;
       }
     }
-    named_barrier_consumers();  // the merge buffer is rewritten by the next item
+    if (it.last) {  // the records of this head that no segment leaves
+      const int rest = p.records - it.record - 1;
+      for (int i = threadIdx.x - 32; i < rest * p.group; i += 32 * kConsumers) {
+        const int h = i / rest;
+        const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.records + it.record + 1 + i - h * rest;
+        p.ml_ws[rec * 2] = -INFINITY;
+        p.ml_ws[rec * 2 + 1] = 0.0f;
+      }
+    }
+    named_barrier_consumers();  // the merge buffer is rewritten by the next segment
   }
 }
 
@@ -516,28 +626,92 @@ struct CombineOut {
   uint32_t kgroups;
 };
 
-template <bool kQuant>
-__global__ void __launch_bounds__(kD) attn_combine_kernel(const float* __restrict__ o_ws,
-                                                         const float* __restrict__ ml_ws, int n_splits, float gv,
-                                                         const CombineOut out) {
+// One block per head, kD threads times kGroups.  A head's records come first
+// in its slots; the others hold (-inf, 0) and an undefined O that is not used.
+// The weights are formed one record per thread, then the records are added,
+// one channel per thread; kGroups = 8 (few heads with many records) lets each
+// group take every eighth one.  The first records' O is loaded beside the
+// weights' inputs: usually that is all there is.
+template <bool kQuant, int kGroups>
+__global__ void __launch_bounds__(kD* kGroups) attn_combine_kernel(const float* __restrict__ o_ws,
+                                                                   const float* __restrict__ ml_ws, int records,
+                                                                   float gv, const CombineOut out) {
+  constexpr int kT = kD * kGroups, kAhead = kGroups > 1 ? 8 : 4;
+  __shared__ float sh_w[kT], sh_acc[kGroups][kD];
+  __shared__ float2 sh_red[kT / 32];
+  __shared__ int sh_used[kT / 32];
   griddep_wait_and_release();
   const size_t bh = static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x;
-  const float* ml = ml_ws + bh * n_splits * 2;
-  float M = -INFINITY;
-  for (int s = 0; s < n_splits; ++s) M = fmaxf(M, __ldg(ml + 2 * s));
-  float acc = 0.0f, L = 0.0f;
-  if (M != -INFINITY) {
-    for (int s = 0; s < n_splits; ++s) {
-      const float w = fast_exp2(__ldg(ml + 2 * s) - M);
-      L += w * __ldg(ml + 2 * s + 1);
-      acc += w * __ldg(o_ws + (bh * n_splits + s) * kD + threadIdx.x);
-    }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = threadIdx.x % kD, group = threadIdx.x / kD;
+  const float2* ml = reinterpret_cast<const float2*>(ml_ws) + bh * records;
+  const float* o = o_ws + bh * records * kD + c;
+  const float2 own = static_cast<int>(threadIdx.x) < records ? __ldg(ml + threadIdx.x) : make_float2(-INFINITY, 0.0f);
+  float ahead[kAhead];
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) {
+    const int i = group + k * kGroups;
+    ahead[k] = i < records ? __ldg(o + static_cast<size_t>(i) * kD) : 0.0f;
   }
+  float m = own.x;
+  int used = own.x != -INFINITY ? static_cast<int>(threadIdx.x) + 1 : 0;  // the records in use come first
+  for (int i = threadIdx.x + kT; i < records; i += kT) {
+    const float x = __ldg(ml + i).x;
+    m = fmaxf(m, x);
+    if (x != -INFINITY) used = i + 1;
+  }
+  used = __reduce_max_sync(0xffffffffu, used);
+#pragma unroll
+  for (int sh = 16; sh; sh >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, sh));
+  if (lane == 0) {
+    sh_red[warp].x = m;
+    sh_used[warp] = used;
+  }
+  __syncthreads();
+  float M = sh_red[0].x;
+  used = sh_used[0];
+#pragma unroll
+  for (int w = 1; w < kT / 32; ++w) {
+    M = fmaxf(M, sh_red[w].x);
+    used = max(used, sh_used[w]);
+  }
+  float acc = 0.0f, l = 0.0f;
+  for (int i0 = 0; i0 < used; i0 += kT) {
+    const int i = i0 + threadIdx.x;
+    float w = 0.0f;
+    if (i < used) {
+      const float2 x = i0 == 0 ? own : __ldg(ml + i);
+      w = fast_exp2(x.x - M);
+      l += w * x.y;
+    }
+    sh_w[threadIdx.x] = w;
+    __syncthreads();
+    const int count = min(kT, used - i0);
+    if (i0 == 0) {
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k)
+        if (group + k * kGroups < count) acc += sh_w[group + k * kGroups] * ahead[k];
+    }
+#pragma unroll 8
+    for (int k = group + (i0 == 0 ? kAhead * kGroups : 0); k < count; k += kGroups)
+      acc += sh_w[k] * __ldg(o + static_cast<size_t>(i0 + k) * kD);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int sh = 16; sh; sh >>= 1) l += __shfl_xor_sync(0xffffffffu, l, sh);
+  if (lane == 0) sh_red[warp].y = l;
+  if (kGroups > 1) sh_acc[group][c] = acc;
+  __syncthreads();
+  if (group) return;
+  float L = sh_red[0].y;
+#pragma unroll
+  for (int w = 1; w < kT / 32; ++w) L += sh_red[w].y;
+#pragma unroll
+  for (int k = 1; k < kGroups; ++k) acc += sh_acc[k][c];
   const float r = L > 0.0f ? __fdiv_rn(acc, L) * gv : 0.0f;
   uint16_t bits;
   asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(bits) : "f"(r));
   if (!kQuant) {
-    out.bf16[bh * kD + threadIdx.x] = bits;
+    out.bf16[bh * kD + c] = bits;
     return;
   }
   // Lanes 16j..16j+15 of a warp hold one 16-channel block of this head.
@@ -557,7 +731,7 @@ __global__ void __launch_bounds__(kD) attn_combine_kernel(const float* __restric
   asm("{\n .reg .b8 t;\n cvt.rn.satfinite.e2m1x2.f32 t, %1, %2;\n cvt.u32.u8 %0, t;\n}"
       : "=r"(pair)
       : "f"(other), "f"(mine));
-  const uint32_t row = blockIdx.y, head = blockIdx.x, c = threadIdx.x;
+  const uint32_t row = blockIdx.y, head = blockIdx.x;
   const uint32_t padded = (static_cast<uint32_t>(out.rows) + 127u) & ~127u;
   const uint64_t code_bytes = static_cast<uint64_t>(out.rows) * gridDim.x * (kD / 2);
   const uint64_t scale_bytes = static_cast<uint64_t>(padded) * out.kgroups * 4;
@@ -577,10 +751,22 @@ __global__ void __launch_bounds__(kD) attn_combine_kernel(const float* __restric
   }
 }
 
-int splits_for(int capacity) { return (capacity + kChunk - 1) / kChunk; }
+// Records per head that the workspace has to hold at least, and those that
+// decode_attention_nvfp4_workspace_size asks for: with few sequences the CTAs
+// (4 on each of 152 SMs) share a head, and lengths up to four times the mean
+// are still spread evenly; S stages never leave more than S records.
+// num_kv_heads is not known there: at least num_q_heads / 8.
+int min_records(int capacity) { return (capacity + kChunk - 1) / kChunk; }
+int64_t preferred_records(int64_t batch, int64_t num_q_heads, int64_t capacity) {
+  const int64_t stages = (capacity + kStageTok - 1) / kStageTok, heads = batch * ((num_q_heads + 7) / 8);
+  const int64_t spread = 4 * ((608 + heads - 1) / heads) + 1, least = min_records(static_cast<int>(capacity)) + 1;
+  const int64_t want = spread > least ? spread : least;
+  return want < stages ? want : stages;
+}
 
+constexpr size_t kRecordBytes = (kD + 2) * sizeof(float);  // O, max and sum of one head's segment
 constexpr size_t kSmemBytes =
-    kStages * kStageBytes + (kConsumers * 8 * kD + 2 * kConsumers * 8) * sizeof(float) + 2 * kStages * 8;
+    kStages * kStageBytes + (kConsumers * 8 * kMergeHead + 2 * kConsumers * 8) * sizeof(float) + 2 * kStages * 8;
 
 template <bool kE1M2>
 int resident_ctas() {
@@ -622,11 +808,17 @@ using namespace nvfp4;
 
 NVFP4_API size_t decode_attention_nvfp4_workspace_size(int32_t batch, int32_t num_q_heads, int32_t capacity) {
   if (batch <= 0 || num_q_heads <= 0 || capacity <= 0) return 0;
-  return static_cast<size_t>(batch) * num_q_heads * splits_for(capacity) * (kD + 2) * sizeof(float);
+  return static_cast<size_t>(batch) * num_q_heads * preferred_records(batch, num_q_heads, capacity) * kRecordBytes;
 }
 
 namespace nvfp4 {
 namespace {
+
+// The smallest workspace that a call accepts; with less than
+// decode_attention_nvfp4_workspace_size bytes fewer CTAs share a head.
+size_t least_workspace(const nvfp4_kv_cache* cache, int32_t num_q_heads) {
+  return static_cast<size_t>(cache->batch) * num_q_heads * min_records(cache->capacity) * kRecordBytes;
+}
 
 // Checks shared by the decode-attention entry points (all but the output
 // buffers and the split-KV partials).
@@ -643,7 +835,7 @@ nvfp4_status attention_validate(const nvfp4_kv_cache* cache, const void* q_bf16,
       num_q_heads / cache->num_kv_heads > 8)
     return NVFP4_ERR_SHAPE;
   if (static_cast<int64_t>(cache->batch) > 65535 || num_q_heads > 65535) return NVFP4_ERR_SHAPE;
-  const int64_t n_items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * splits_for(cache->capacity);
+  const int64_t n_items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * min_records(cache->capacity);
   if (n_items >= (1ll << 31)) return NVFP4_ERR_SHAPE;
   return NVFP4_OK;
 }
@@ -651,13 +843,16 @@ nvfp4_status attention_validate(const nvfp4_kv_cache* cache, const void* q_bf16,
 // Alignment of the query and cache arrays, then the partial kernel's
 // parameters with its partials at `partials` and its grid size.
 nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, int32_t num_q_heads,
-                              float softmax_scale, float* partials, Params* prm, int* grid) {
+                              float softmax_scale, float* partials, size_t partials_bytes, Params* prm,
+                              int* grid) {
   if (!aligned(q_bf16, 16) || !aligned(cache->k_codes, 16) || !aligned(cache->v_codes, 16) ||
       !aligned(cache->k_scales, 16) || !aligned(cache->v_scales, 16))
     return NVFP4_ERR_ALIGN;
   const int ctas_max = resident_ctas(cache);
   if (ctas_max <= 0) return NVFP4_ERR_CUDA;
-  const int64_t n_items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * splits_for(cache->capacity);
+  const int64_t stages = (cache->capacity + kStageTok - 1) / kStageTok;
+  const int64_t items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * stages;
+  const int64_t fit = static_cast<int64_t>(partials_bytes / (kRecordBytes * cache->batch * num_q_heads));
   prm->k_codes = cache->k_codes;
   prm->k_scales = cache->k_scales;
   prm->v_codes = cache->v_codes;
@@ -669,16 +864,36 @@ nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, i
   prm->capacity = cache->capacity;
   prm->hq = num_q_heads;
   prm->group = num_q_heads / cache->num_kv_heads;
-  prm->n_splits = splits_for(cache->capacity);
-  prm->n_items = static_cast<int>(n_items);
+  prm->batch = cache->batch;
+  // Never more than asked for, so that a larger workspace changes no result.
+  const int64_t want = preferred_records(cache->batch, num_q_heads, cache->capacity);
+  prm->records = static_cast<int>(fit < want ? fit : want);
+  prm->whole = stages <= 1 || prm->records < 2;
+  if (prm->whole) prm->records = 1;
   prm->logit_mult = softmax_scale * cache->k_gscale * kLog2e;
   prm->fault_skip_stage = take_fault(NVFP4_FAULT_ATTN_SKIP_STAGE) ? 1 : 0;
   // Every record the combine kernel reads is written by the partial kernel of
   // the same call, so nothing left from an earlier call needs clearing.
   prm->o_ws = partials;
-  prm->ml_ws = prm->o_ws + static_cast<size_t>(cache->batch) * num_q_heads * prm->n_splits * kD;
-  *grid = static_cast<int>(n_items < ctas_max ? n_items : ctas_max);
+  prm->ml_ws = prm->o_ws + static_cast<size_t>(cache->batch) * num_q_heads * prm->records * kD;
+  *grid = static_cast<int>(items < ctas_max ? items : ctas_max);
   return NVFP4_OK;
+}
+
+// The partial and the combine kernel.  With few heads of many records the
+// combine's blocks take 8 x 128 threads (1 x 40 heads of 64 records: 4.3 ->
+// 3.0 us); with many heads more threads per head would only crowd the SMs.
+template <bool kQuant>
+nvfp4_status attention_launch(const nvfp4_kv_cache* cache, const Params& prm, int grid, const CombineOut& out,
+                              cudaStream_t s) {
+  const bool wide = prm.records > 8 && static_cast<int64_t>(prm.hq) * prm.batch <= 2 * sm_count();
+  if (launch_pdl(partial_kernel(cache), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
+      launch_pdl(wide ? attn_combine_kernel<kQuant, 8> : attn_combine_kernel<kQuant, 1>, dim3(prm.hq, prm.batch),
+                 dim3(wide ? 8 * kD : kD), 0, s, static_cast<const float*>(prm.o_ws),
+                 static_cast<const float*>(prm.ml_ws), prm.records, cache->v_gscale, out) != cudaSuccess)
+    return NVFP4_ERR_CUDA;
+  count_launches(2);
+  return launch_status();
 }
 
 }  // namespace
@@ -691,21 +906,15 @@ NVFP4_API nvfp4_status decode_attention_nvfp4(const nvfp4_kv_cache* cache, const
   if (!out_bf16 || !workspace) return NVFP4_ERR_INVALID_ARG;
   nvfp4_status st = attention_validate(cache, q_bf16, num_q_heads, softmax_scale);
   if (st != NVFP4_OK) return st;
-  if (workspace_bytes < decode_attention_nvfp4_workspace_size(cache->batch, num_q_heads, cache->capacity))
-    return NVFP4_ERR_SHAPE;
+  if (workspace_bytes < least_workspace(cache, num_q_heads)) return NVFP4_ERR_SHAPE;
   if (!aligned(out_bf16, 16) || !aligned(workspace, 16)) return NVFP4_ERR_ALIGN;
   Params prm;
   int grid = 0;
-  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), &prm, &grid);
+  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), workspace_bytes, &prm,
+                        &grid);
   if (st != NVFP4_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (launch_pdl(partial_kernel(cache), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
-      launch_pdl(attn_combine_kernel<false>, dim3(num_q_heads, cache->batch), dim3(kD), 0, s,
-                 static_cast<const float*>(prm.o_ws), static_cast<const float*>(prm.ml_ws), prm.n_splits,
-                 cache->v_gscale, CombineOut{static_cast<uint16_t*>(out_bf16)}) != cudaSuccess)
-    return NVFP4_ERR_CUDA;
-  count_launches(2);
-  return launch_status();
+  return attention_launch<false>(cache, prm, grid, CombineOut{static_cast<uint16_t*>(out_bf16)}, s);
 }
 
 NVFP4_API nvfp4_status decode_attention_nvfp4_quantize(const nvfp4_kv_cache* cache, const void* q_bf16,
@@ -716,13 +925,13 @@ NVFP4_API nvfp4_status decode_attention_nvfp4_quantize(const nvfp4_kv_cache* cac
   if (!g_out || !out_codes || !out_scales || !workspace) return NVFP4_ERR_INVALID_ARG;
   nvfp4_status st = attention_validate(cache, q_bf16, num_q_heads, softmax_scale);
   if (st != NVFP4_OK) return st;
-  if (workspace_bytes < decode_attention_nvfp4_workspace_size(cache->batch, num_q_heads, cache->capacity))
-    return NVFP4_ERR_SHAPE;
+  if (workspace_bytes < least_workspace(cache, num_q_heads)) return NVFP4_ERR_SHAPE;
   if (!aligned(out_codes, 16) || !aligned(out_scales, 4) || !aligned(g_out, 4) || !aligned(workspace, 16))
     return NVFP4_ERR_ALIGN;
   Params prm;
   int grid = 0;
-  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), &prm, &grid);
+  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), workspace_bytes, &prm,
+                        &grid);
   if (st != NVFP4_OK) return st;
   CombineOut o{};
   o.codes = out_codes;
@@ -732,13 +941,7 @@ NVFP4_API nvfp4_status decode_attention_nvfp4_quantize(const nvfp4_kv_cache* cac
   o.rows = cache->batch;
   o.kgroups = static_cast<uint32_t>(num_q_heads) * (kD / 64);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (launch_pdl(partial_kernel(cache), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
-      launch_pdl(attn_combine_kernel<true>, dim3(num_q_heads, cache->batch), dim3(kD), 0, s,
-                 static_cast<const float*>(prm.o_ws), static_cast<const float*>(prm.ml_ws), prm.n_splits,
-                 cache->v_gscale, o) != cudaSuccess)
-    return NVFP4_ERR_CUDA;
-  count_launches(2);
-  return launch_status();
+  return attention_launch<true>(cache, prm, grid, o, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -779,22 +982,14 @@ NVFP4_API nvfp4_status decode_attention_nvfp4_static_scratch(const nvfp4_kv_cach
   nvfp4_status st = attention_validate(cache, q_bf16, num_q_heads, softmax_scale);
   if (st != NVFP4_OK) return st;
   // The partials must fit in the static scratch; larger problems are refused.
-  if (decode_attention_nvfp4_workspace_size(cache->batch, num_q_heads, cache->capacity) >
-      NVFP4_ATTN_STATIC_SCRATCH_BYTES)
-    return NVFP4_ERR_SHAPE;
+  if (least_workspace(cache, num_q_heads) > NVFP4_ATTN_STATIC_SCRATCH_BYTES) return NVFP4_ERR_SHAPE;
   if (!aligned(out_bf16, 16)) return NVFP4_ERR_ALIGN;
   float* scratch = attn_static_scratch_dev();
   if (!scratch) return NVFP4_ERR_CUDA;
   Params prm;
   int grid = 0;
-  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, scratch, &prm, &grid);
+  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, scratch, NVFP4_ATTN_STATIC_SCRATCH_BYTES, &prm, &grid);
   if (st != NVFP4_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (launch_pdl(partial_kernel(cache), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
-      launch_pdl(attn_combine_kernel<false>, dim3(num_q_heads, cache->batch), dim3(kD), 0, s,
-                 static_cast<const float*>(prm.o_ws), static_cast<const float*>(prm.ml_ws), prm.n_splits,
-                 cache->v_gscale, CombineOut{static_cast<uint16_t*>(out_bf16)}) != cudaSuccess)
-    return NVFP4_ERR_CUDA;
-  count_launches(2);
-  return launch_status();
+  return attention_launch<false>(cache, prm, grid, CombineOut{static_cast<uint16_t*>(out_bf16)}, s);
 }

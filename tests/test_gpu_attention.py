@@ -526,3 +526,50 @@ def test_injected_missing_stage_times_out_and_device_stays_usable(N):
     ref = O.decode_attention(f32(q), rkc, rks, rvc, rvs, lens, gk, gv, scale)
     for b in range(B):
         assert_close(f32(out)[b], ref[b], what=f"after the injected timeout, seq {b}")
+
+
+@pytest.mark.parametrize("hq,hkv,cap,lens,fmt", [
+    (4, 2, 2048, [0, 128, 129, 2048, 1, 0, 1280, 127], 0),    # empty sequences, stage edges
+    (8, 1, 6144, [6143, 300], 1),                              # one long sequence beside a short one
+    (8, 8, 512, [512] * 40, 0),                                # more heads than a run: several heads per CTA
+    (6, 2, 126, [126, 5, 64], 0),                              # at most one stage per head
+    (5, 1, 1536, [(37 * i) % 1537 for i in range(70)], 0)])    # 70 sequences of all lengths
+@pytest.mark.parametrize("least", [False, True])
+def test_decode_attention_runs_over_ragged_lengths(N, hq, hkv, cap, lens, fmt, least):
+    """Equal runs of stages over ragged caches, with the asked-for workspace
+    and with the smallest one that is accepted."""
+    B = len(lens)
+    gen = torch.Generator(device="cuda").manual_seed(B + cap)
+    cache = N.KVCache(B, hkv, cap, 0.013, 0.021, kv_format=fmt)
+    for t in (cache.k_codes, cache.v_codes):
+        c = torch.randint(0, 256, t.shape, generator=gen, device="cuda", dtype=torch.int32)
+        if fmt:  # E1M2 never holds the nibble 8
+            c = torch.where((c & 15) == 8, c ^ 8, c)
+            c = torch.where((c >> 4) == 8, c ^ 128, c)
+        t.copy_(c.to(torch.uint8))
+    for t in (cache.k_scales, cache.v_scales):
+        t.copy_(torch.randint(0x28, 0x48, t.shape, generator=gen, device="cuda", dtype=torch.int32).to(torch.uint8))
+    cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
+    q = torch.randn(B, hq, 128, generator=gen, device="cuda").to(torch.bfloat16)
+    need = B * hq * ((cap + 1023) // 1024) * 520 if least else N.decode_attention_nvfp4_workspace_size(B, hq, cap)
+    ws = torch.full((need // 4,), float("nan"), dtype=torch.float32, device="cuda")
+    out = torch.full((B, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
+    N.decode_attention_nvfp4(cache, q, 1 / math.sqrt(128), out, ws)
+    torch.cuda.synchronize()
+    assert N.nvfp4_get_device_status() == 0
+    grid = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6] if not fmt else
+                        [n / 2 for n in range(8)] + [(n - 16) / 2 for n in range(8, 16)], dtype=torch.float64, device="cuda")
+
+    def values(codes, scales, g):
+        c = torch.stack([codes & 15, codes >> 4], dim=-1).flatten(-2).long()
+        s = scales.view(torch.float8_e4m3fn).double().repeat_interleave(16, dim=-1)
+        return grid[c] * s * g
+    k, v = values(cache.k_codes, cache.k_scales, 0.013), values(cache.v_codes, cache.v_scales, 0.021)
+    for b, n in enumerate(lens):
+        if n == 0:
+            assert not out[b].float().any()
+            continue
+        qq = q[b].double().view(hkv, hq // hkv, 128)
+        p = torch.softmax(qq @ k[b, :, :n].transpose(1, 2) / math.sqrt(128), dim=-1)
+        ref = (p @ v[b, :, :n]).reshape(hq, 128)
+        assert_close(f32(out[b]), ref.cpu().numpy(), what=f"sequence {b} of {n}")
