@@ -2,9 +2,8 @@
 // m, Eq. 2) and write them into the NVFP4 KV cache; optionally rotate K by
 // RoPE first (the fused RoPE -> shift -> quantize -> append step).
 //
-// Work item = one 16-element block of one 128-channel row (one thread per
-// block: the block scale is computed once).  Item order (token, kv head, K|V,
-// block) keeps each warp's reads contiguous in the [n_new, H_kv, 128] inputs.
+// One thread per 16-element block of a 128-channel row, so the block scale is
+// computed once; reads of 16 threads cover whole K and V rows.
 #include <cfloat>
 
 #include "common.cuh"
@@ -14,61 +13,64 @@ namespace nvfp4 {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kUnroll = 4;  // items (16-element blocks) per thread per pass
 
 // kRope: K arrives before RoPE and is rotated here (rotate-half pairing,
 // channel i with i + 64) with the (cos, sin) table row of its position, in
 // fp32: y_i = x_i c_i - x_{i+64} s_i, y_{i+64} = x_i s_i + x_{i+64} c_i.
 //
-// Work item = one 16-element block of one row (row = token, KV head, K or V):
-// 16 items per (token, head), so a warp covers two.  Lane l of a warp takes
-// (token-head 2w + l/16, K or V by bit 3, block l % 8); the RoPE partner block
-// (channels 64 apart) is on lane l ^ 4.  kUnroll items per thread per pass,
-// all their loads issued first.
-template <bool kRope, bool kE1M2>
+// A thread takes one 16-element block (of K or of V) of U consecutive heads of
+// one token.  Eight lanes cover a row's blocks, a warp four head groups of K or
+// of V (so that no lane idles while K is rotated); the RoPE partner block
+// (channels 64 apart) is on lane l ^ 4.  The rotation depends on the token and the block only, so its (cos,
+// sin) values, four times the bytes of a K block, are loaded once for U heads,
+// and everything else that the thread reads is issued with them.
+template <bool kRope, bool kE1M2, int U>
 __global__ void __launch_bounds__(kThreads) kv_append_kernel(
     const uint16_t* __restrict__ k_in, const uint16_t* __restrict__ v_in, const int32_t* __restrict__ seq_idx,
     const int32_t* __restrict__ pos, const float* __restrict__ k_shift, const float* __restrict__ rope,
-    uint32_t n_rows /* n_new*H_kv */, FastDiv hkv, uint32_t batch, uint32_t capacity, uint8_t* __restrict__ kc,
-    uint8_t* __restrict__ ks, uint8_t* __restrict__ vc, uint8_t* __restrict__ vs, float gk, float gv, int* status) {
+    uint32_t n_new, uint32_t hkv, FastDiv groups /* of U heads per token */, uint32_t batch, uint32_t capacity,
+    uint8_t* __restrict__ kc, uint8_t* __restrict__ ks, uint8_t* __restrict__ vc, uint8_t* __restrict__ vs, float gk,
+    float gv, int* status) {
   griddep_wait_and_release();
-  const uint32_t total = n_rows * 16u;  // 2 tensors x 8 blocks per row: a multiple of the warp
+  const uint32_t n_groups = n_new * groups.d, total = (n_groups + 3u) / 4u * 64u;  // a K and a V warp per four
   const uint32_t lane = threadIdx.x & 31;
   const float qmax = kE1M2 ? 3.5f : 6.0f;  // largest element magnitude of the grid
   const float six_gk = __fmul_rn(qmax, gk), six_gv = __fmul_rn(qmax, gv);
-  const uint32_t stride = gridDim.x * blockDim.x;
-  // Item indices are formed in 64 bits: a pass may reach past 2^32 near the end.
-  for (uint64_t c00 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); c00 < total;
-       c00 += static_cast<uint64_t>(stride) * kUnroll) {
-    uint4 lo[kUnroll], hi[kUnroll];
+  // 64 bits: a step may reach past 2^32 near the end.
+  for (uint64_t c0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); c0 < total;
+       c0 += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+    const uint32_t group = static_cast<uint32_t>(c0 >> 6) * 4u + (lane >> 3);
+    const bool is_v = (c0 >> 5) & 1u;
+    const bool live = group < n_groups;
+    const uint32_t blk = lane & 7u;  // block within the 128-channel row
+    const uint32_t tok = live ? groups.div(group) : 0;
+    const uint32_t h0 = live ? (group - tok * groups.d) * U : 0;
+    const uint64_t row0 = static_cast<uint64_t>(tok) * hkv + h0;
+    const uint4* src = reinterpret_cast<const uint4*>((is_v ? v_in : k_in) + row0 * 128 + blk * 16);
+    const int32_t b = __ldg(seq_idx + tok), p = __ldg(pos + tok);
+    uint4 lo[U], hi[U];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const uint64_t c = c00 + static_cast<uint64_t>(u) * stride + lane;
-      const uint32_t rr = static_cast<uint32_t>(c >> 4);
-      const bool is_v = (c >> 3) & 1u;
-      const uint4* src = reinterpret_cast<const uint4*>((is_v ? v_in : k_in) + static_cast<uint64_t>(rr) * 128 +
-                                                        (c & 7u) * 16);
-      const bool in = c < total;
-      lo[u] = in ? __ldg(src) : make_uint4(0, 0, 0, 0);
-      hi[u] = in ? __ldg(src + 1) : make_uint4(0, 0, 0, 0);
+    for (int u = 0; u < U; ++u) {
+      lo[u] = live ? __ldg(src + 16 * u) : make_uint4(0, 0, 0, 0);
+      hi[u] = live ? __ldg(src + 16 * u + 1) : make_uint4(0, 0, 0, 0);
+    }
+    const bool bad = b < 0 || static_cast<uint32_t>(b) >= batch || p < 0 || static_cast<uint32_t>(p) >= capacity;
+    float4 cs[kRope ? 8 : 1];
+    if (kRope && !is_v) {
+      // A position outside the cache is reported below; it rotates by row 0.
+      const float4* row =
+          reinterpret_cast<const float4*>(rope + (static_cast<uint64_t>(bad ? 0 : p) * 64 + (blk & 3u) * 16) * 2);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) cs[q] = __ldg(row + q);
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const uint64_t c0 = c00 + static_cast<uint64_t>(u) * stride;
-      if (c0 >= total) continue;  // warp-uniform: c0 is the warp's first item
-      const uint32_t c = static_cast<uint32_t>(c0) + lane;  // c0 < total < 2^32
-      const bool live = c < total;         // an odd row count leaves half of the last warp idle
-      const uint32_t blk = c & 7u;         // block within the 128-channel row
-      const bool is_v = (c >> 3) & 1u;
-      const uint32_t rr = c >> 4;          // token * H_kv + head
-      const uint32_t tok = hkv.div(rr);
-      const uint32_t h = rr - tok * hkv.d;
+    for (int u = 0; u < U; ++u) {
+      const uint32_t h = h0 + u;
       float x[16];
       unpack_bf16x8(lo[u], x);
       unpack_bf16x8(hi[u], x + 8);
       if (kRope) {
-        // The partner block (channels 64 apart) is on lane ^ 4; every lane of the warp is live.
-        uint4 plo, phi;
+        uint4 plo, phi;  // the partner block
         plo.x = __shfl_xor_sync(0xffffffffu, lo[u].x, 4);
         plo.y = __shfl_xor_sync(0xffffffffu, lo[u].y, 4);
         plo.z = __shfl_xor_sync(0xffffffffu, lo[u].z, 4);
@@ -77,18 +79,13 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(
         phi.y = __shfl_xor_sync(0xffffffffu, hi[u].y, 4);
         phi.z = __shfl_xor_sync(0xffffffffu, hi[u].z, 4);
         phi.w = __shfl_xor_sync(0xffffffffu, hi[u].w, 4);
-        if (live && !is_v) {
+        if (!is_v) {
           float xp[16];
           unpack_bf16x8(plo, xp);
           unpack_bf16x8(phi, xp + 8);
-          int32_t p = __ldg(pos + tok);
-          if (p < 0 || static_cast<uint32_t>(p) >= capacity) p = 0;  // reported as CAPACITY below
-          const float4* cs =
-              reinterpret_cast<const float4*>(rope + (static_cast<uint64_t>(p) * 64 + (blk & 3u) * 16) * 2);
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
-            const float4 t = __ldg(cs + q);
-            const float cv0 = t.x, sv0 = t.y, cv1 = t.z, sv1 = t.w;
+            const float cv0 = cs[q].x, sv0 = cs[q].y, cv1 = cs[q].z, sv1 = cs[q].w;
             const int e = 2 * q;
             x[e] = blk < 4 ? __fsub_rn(__fmul_rn(x[e], cv0), __fmul_rn(xp[e], sv0))
                            : __fadd_rn(__fmul_rn(xp[e], sv0), __fmul_rn(x[e], cv0));
@@ -97,7 +94,7 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(
           }
         }
       }
-      if (live && !is_v && k_shift) {
+      if (!is_v && k_shift) {
         const float4* m4 = reinterpret_cast<const float4*>(k_shift + h * 128u + blk * 16u);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -116,17 +113,23 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(
       for (int i = 0; i < 16; ++i) x[i] = __fmul_rn(x[i], bs.mult);
       const uint2 packed = kE1M2 ? make_uint2(e1m2x8(x), e1m2x8(x + 8)) : make_uint2(e2m1x8(x), e2m1x8(x + 8));
       if (!live) continue;
-      const int32_t b = __ldg(seq_idx + tok), p = __ldg(pos + tok);
-      if (b < 0 || static_cast<uint32_t>(b) >= batch || p < 0 || static_cast<uint32_t>(p) >= capacity) {
+      if (bad) {
         if (blk == 0 && !is_v) set_status(status, NVFP4_ERR_CAPACITY);
         continue;
       }
-      const uint64_t row = (static_cast<uint64_t>(b) * hkv.d + h) * capacity + static_cast<uint32_t>(p);
-      if (!in_bounds(status, row < static_cast<uint64_t>(batch) * hkv.d * capacity && blk < 8u)) continue;
+      const uint64_t row = (static_cast<uint64_t>(b) * hkv + h) * capacity + static_cast<uint32_t>(p);
+      if (!in_bounds(status, row < static_cast<uint64_t>(batch) * hkv * capacity && blk < 8u)) continue;
       reinterpret_cast<uint2*>((is_v ? vc : kc) + row * 64)[blk] = packed;
       (is_v ? vs : ks)[row * 8 + blk] = static_cast<uint8_t>(bs.code);
     }
   }
+}
+
+// The kernel for U heads per thread.
+template <int U>
+auto append_kernel(bool rope, bool e1m2) {
+  return rope ? (e1m2 ? kv_append_kernel<true, true, U> : kv_append_kernel<true, false, U>)
+              : (e1m2 ? kv_append_kernel<false, true, U> : kv_append_kernel<false, false, U>);
 }
 
 nvfp4_status append(const nvfp4_kv_cache* cache, const void* k_bf16, const void* v_bf16, const int32_t* seq_idx,
@@ -144,19 +147,29 @@ nvfp4_status append(const nvfp4_kv_cache* cache, const void* k_bf16, const void*
       (rope && !aligned(rope, 16)))
     return NVFP4_ERR_ALIGN;
   if (n_new == 0) return NVFP4_OK;
-  const uint32_t n_rows = static_cast<uint32_t>(n_new * cache->num_kv_heads);
-  const uint64_t items = static_cast<uint64_t>(n_rows) * 16;
-  uint64_t grid = (items + kThreads * kUnroll - 1) / (kThreads * kUnroll);
+  const bool e1m2 = cache->kv_format == NVFP4_KV_E1M2;
+  const uint32_t heads = static_cast<uint32_t>(cache->num_kv_heads), tokens = static_cast<uint32_t>(n_new);
+  // Heads per thread.  One while a thread per block does not fill the GPU
+  // (latency); two beyond that; four with RoPE once even those are several
+  // waves (the table's loads count, registers allow two CTAs per SM).  GB300,
+  // U = 1 / 2 / 4, 8 heads with RoPE and shift: 64 tokens 2.2 / 2.8 / 4.0 us,
+  // 1024 4.7 / 3.6 / 4.3, 4093 11.0 / 11.0 / 10.1, 65536 119 / 102 / 81;
+  // without, 262144 tokens: 259 / 208 / 231.  (One block of K or V of one head
+  // per thread with four such items in turn, before: 6.1, 6.4, 15.5, 167; 277.)
+  const uint64_t items = static_cast<uint64_t>(tokens) * heads * 16, per_sm = items / sm_count();
+  const uint32_t U = per_sm <= 512 || heads % 2 ? 1 : (rope && per_sm >= 2048 && heads % 4 == 0 ? 4 : 2);
+  const auto kernel = U == 4   ? append_kernel<4>(rope, e1m2)
+                      : U == 2 ? append_kernel<2>(rope, e1m2)
+                               : append_kernel<1>(rope, e1m2);
+  const uint64_t threads = (static_cast<uint64_t>(tokens) * (heads / U) + 3) / 4 * 64;
+  uint64_t grid = (threads + kThreads - 1) / kThreads;
   const uint64_t cap = static_cast<uint64_t>(sm_count()) * 8;
   if (grid > cap) grid = cap;
-  const bool e1m2 = cache->kv_format == NVFP4_KV_E1M2;
-  const auto kernel = rope ? (e1m2 ? kv_append_kernel<true, true> : kv_append_kernel<true, false>)
-                           : (e1m2 ? kv_append_kernel<false, true> : kv_append_kernel<false, false>);
   const cudaError_t e =
       launch_pdl(kernel, dim3(static_cast<int>(grid)), dim3(kThreads),
                  0, static_cast<cudaStream_t>(stream), static_cast<const uint16_t*>(k_bf16),
-                 static_cast<const uint16_t*>(v_bf16), seq_idx, pos, k_shift, rope, n_rows,
-                 FastDiv(static_cast<uint32_t>(cache->num_kv_heads)), static_cast<uint32_t>(cache->batch),
+                 static_cast<const uint16_t*>(v_bf16), seq_idx, pos, k_shift, rope, tokens, heads,
+                 FastDiv(heads / U), static_cast<uint32_t>(cache->batch),
                  static_cast<uint32_t>(cache->capacity), cache->k_codes, cache->k_scales, cache->v_codes,
                  cache->v_scales, cache->k_gscale, cache->v_gscale, status_word_dev());
   if (e != cudaSuccess) return NVFP4_ERR_CUDA;

@@ -573,3 +573,28 @@ def test_decode_attention_runs_over_ragged_lengths(N, hq, hkv, cap, lens, fmt, l
         p = torch.softmax(qq @ k[b, :, :n].transpose(1, 2) / math.sqrt(128), dim=-1)
         ref = (p @ v[b, :, :n]).reshape(hq, 128)
         assert_close(f32(out[b]), ref.cpu().numpy(), what=f"sequence {b} of {n}")
+
+
+@pytest.mark.parametrize("n_new,hkv", [(1, 1), (3, 3), (7, 8), (608, 8), (611, 8), (1231, 6), (2433, 8), (2431, 4)])
+@pytest.mark.parametrize("fmt", [0, 1])
+def test_append_heads_per_thread(N, n_new, hkv, fmt):
+    """Edges of the heads per thread (1, 2 and 4), head counts that none of
+    them divides, and counts that leave part of the last warp idle."""
+    cap = (n_new + 1) & ~1
+    gen = torch.Generator().manual_seed(n_new * 10 + hkv)
+    k, v = (torch.randn(n_new, hkv, 128, generator=gen).to(torch.bfloat16) for _ in range(2))
+    shift = torch.randn(hkv, 128, generator=gen)
+    pos = torch.randperm(n_new, generator=gen).numpy()
+    table = O.rope_table(cap)
+    cache = N.KVCache(1, hkv, cap, 0.003, 0.002, kv_format=fmt)
+    cache.v_codes.fill_(0xEE)
+    seq, p = torch.zeros(n_new, dtype=torch.int32, device="cuda"), torch.as_tensor(pos, dtype=torch.int32, device="cuda")
+    N.kv_append_rope_nvfp4(cache, k.cuda(), v.cuda(), seq, p, torch.from_numpy(table).cuda(), k_shift=shift.cuda())
+    torch.cuda.synchronize()
+    assert N.nvfp4_get_device_status() == 0
+    ref = [np.zeros((1, hkv, cap, w), np.uint8) for w in (64, 8, 64, 8)]
+    ref[2][:] = 0xEE
+    O.kv_append_rope(*ref, f32(k), f32(v), np.zeros(n_new, np.int64), pos, np.float32(0.003), np.float32(0.002), table,
+                     k_shift=shift.numpy(), element="e1m2" if fmt else "e2m1")
+    for got, want in zip((cache.k_codes, cache.k_scales, cache.v_codes, cache.v_scales), ref):
+        assert np.array_equal(u8(got), want)
