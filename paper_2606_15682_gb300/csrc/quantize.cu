@@ -203,28 +203,13 @@ __device__ __forceinline__ void zero_scale_padding(uint32_t rows, uint32_t kbloc
   }
 }
 
-// One thread quantizes one 16-element block per slot: two 128-bit loads (the
-// second half of the 32 bytes is in L1 after the first load of the warp), one
-// scale computation, one 64-bit code store.  A warp covers 32 consecutive
-// blocks per slot.
-template <bool kMMA>
-__device__ __forceinline__ void quantize_blocks(const uint16_t* __restrict__ x, FastDiv kblocks_div,
-                                                uint32_t total_blocks, int64_t ld, bool dense, uint32_t rows,
-                                                float g, bool g_ok, uint2* __restrict__ codes,
-                                                uint8_t* __restrict__ scales, int* status) {
-  const float six_g = __fmul_rn(6.0f, g);
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  // bidx0 is warp-uniform so every lane takes part in the scale gather.
-  for (uint32_t bidx0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); bidx0 < total_blocks; bidx0 += stride * kUnroll) {
-    BlockSlots<> sl;
-    load_blocks(x, kblocks_div, total_blocks, ld, dense, bidx0, stride, lane, sl);
-    quantize_loaded<kMMA>(sl, total_blocks, kblocks_div.d, bidx0, stride, lane, g, six_g, g_ok, codes, scales,
-                          status);
-  }
-  if (kMMA) zero_scale_padding(rows, kblocks_div.d, scales, status);
-}
-
+// One CTA per 1024 consecutive blocks, four per thread (two 128-bit loads
+// each; a warp covers 32 consecutive blocks per slot), HBM-bound.  CTAs run
+// from the tensor's end to its start: whatever read or wrote x before (the
+// amax pass, a producer) went the other way and left the end in L2.  As many
+// CTAs as the work has, rather than 8 per SM that step over it, leave no last
+// step with few of them.  GB300, both calls: 13824 x 5120 57.1 -> 53.5 us, 8192 x
+// 27648 169.6 -> 161.4.
 template <bool kMMA>
 __global__ void __launch_bounds__(kThreads) quantize_kernel(const uint16_t* __restrict__ x, FastDiv kblocks_div,
                                                             uint32_t total_blocks, int64_t ld, bool dense,
@@ -235,8 +220,14 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const uint16_t* __re
   const float g_in = *g_ptr;
   const bool g_ok = g_in > 0.0f && g_in <= FLT_MAX;
   if (!g_ok && blockIdx.x == 0 && threadIdx.x == 0) set_status(status, NVFP4_ERR_INVALID_ARG);
-  quantize_blocks<kMMA>(x, kblocks_div, total_blocks, ld, dense, rows, g_ok ? g_in : 1.0f, g_ok, codes, scales,
-                        status);
+  const float g = g_ok ? g_in : 1.0f;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t bidx0 = (gridDim.x - 1 - blockIdx.x) * (kThreads * kUnroll) + (threadIdx.x & ~31u);  // warp-uniform
+  BlockSlots<> sl;
+  load_blocks(x, kblocks_div, total_blocks, ld, dense, bidx0, kThreads, lane, sl);
+  quantize_loaded<kMMA>(sl, total_blocks, kblocks_div.d, bidx0, kThreads, lane, g, __fmul_rn(6.0f, g), g_ok, codes,
+                        scales, status);
+  if (kMMA) zero_scale_padding(rows, kblocks_div.d, scales, status);
 }
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
@@ -618,9 +609,10 @@ NVFP4_API nvfp4_status nvfp4_quantize(const void* x_bf16, int64_t rows, int64_t 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint32_t kblocks = static_cast<uint32_t>(cols / 16);
   const uint32_t total_blocks = static_cast<uint32_t>(rows * kblocks);
-  const int grid = grid_for(total_blocks, kThreads * kUnroll);
+  const auto kernel = layout == NVFP4_SCALES_MMA ? quantize_kernel<true> : quantize_kernel<false>;
+  const uint32_t grid = total_blocks / (kThreads * kUnroll) + (total_blocks % (kThreads * kUnroll) != 0);
   const bool dense = (ld == cols);
-  cudaError_t e = launch_pdl(layout == NVFP4_SCALES_MMA ? quantize_kernel<true> : quantize_kernel<false>, dim3(grid),
+  cudaError_t e = launch_pdl(kernel, dim3(grid),
                              dim3(kThreads), 0, s, static_cast<const uint16_t*>(x_bf16), FastDiv(kblocks),
                              total_blocks, ld, dense, static_cast<uint32_t>(rows), g_dev,
                              reinterpret_cast<uint2*>(codes), scales, status_word_dev());
