@@ -1714,16 +1714,25 @@ __global__ void __launch_bounds__(C::kThreads, 2)
 // only W through a 5-stage ring, from the kernel's first instruction on.
 //   warp 0      TMA producer for W codes and scales (skips the prologue)
 //   warps 1-11  prologue (amax, then quantization), then:
-//   warp 1      TMEM allocation; one lane issues the MMAs
-//   warp 2      one lane copies the A scales once, then each stage's W scales
-//   warps 3-6   epilogue (double-buffered 128-column accumulator)
+//   warp 1      TMEM allocation; MMAs
+//   warp 2      scale copies: each stage's W scales, for the CTA's first tile
+//               with that k-block's A scales
+//   warps 4, 8  epilogue, 64 of 128 columns each (the two warps that reach
+//               TMEM lanes 0-31, where the at most 32 rows are)
+// Latency-bound (12 CTAs at N = 1536, 0.02 of HBM): what counts is the chain
+// x -> amax -> block scales -> scale copies -> MMAs -> stores.  A's rows and
+// scales past M are whatever shared memory holds; they only reach accumulator
+// rows that are never stored.  16 x 1536 x 1536 back to back 9.1 -> 6.5 us, 32
+// rows 10.3 -> 7.9, 16 x 17920 x 1536 9.6 -> 7.0 (before: padding zeroed, one
+// thread combining the warps' maxima, all A scales copied before the first
+// MMA, TMA stores).
 struct DynCfg {
   static constexpr int BN = 128;
   static constexpr int kStages = 5;
   static constexpr int kMaxKb = 6;                          // K <= 1536
   static constexpr int kMaxRows = 32;                       // M <= 32
-  static constexpr int kEpiWarps = 4;
-  // Warps 7-11 only help with the prologue, whose per-block arithmetic
+  static constexpr int kEpiWarps = 2;
+  // The others only help with the prologue, whose per-block arithmetic
   // (E4M3 scale, reciprocal, 16 conversions) is latency-bound with few warps.
   static constexpr int kThreads = 384;
   static constexpr int kProThreads = kThreads - 32;          // warps 1-11
@@ -1747,6 +1756,9 @@ struct DynArgs {
   const uint8_t* sfb;
   const float* gb;
   float* g_out;  // optional: g_a
+  uint16_t* out;
+  int64_t ldo;
+  FastDiv kb16;  // 16-element blocks per row
   int M, N, K;
   int tiles_n;
   int* status;
@@ -1767,8 +1779,7 @@ __device__ __forceinline__ void st_shared_u8(uint32_t addr, uint32_t v) {
 
 template <class C>
 __global__ void __launch_bounds__(C::kThreads, 1)
-    nvfp4_linear_dyn_kernel(const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ CUtensorMap tmap_out,
-                            const DynArgs args) {
+    nvfp4_linear_dyn_kernel(const __grid_constant__ CUtensorMap tmap_b, const DynArgs args) {
   constexpr int BN = C::BN;
   constexpr int kStages = C::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -1783,13 +1794,11 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   uint64_t* sfready = empty + kStages;
   uint64_t* tfull = sfready + kStages;
   uint64_t* tempty = tfull + 2;
-  uint64_t* aready = tempty + 2;
-  uint64_t* drain = aready + 1;
+  uint64_t* drain = tempty + 2;
   uint64_t* drain_cp = drain + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_cp + 1);
   __shared__ volatile int abort_flag;
   __shared__ uint32_t warp_max[C::kThreads / 32];
-  __shared__ float s_g;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int kblocks = args.K / BK;
@@ -1807,13 +1816,11 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       mbar_init(&tfull[a], 1);
       mbar_init(&tempty[a], C::kEpiWarps);
     }
-    mbar_init(aready, 1);
     mbar_init(drain, 1);
     mbar_init(drain_cp, 1);
     abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tmap_b);
-    prefetch_tmap(&tmap_out);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, kTmemCols);
@@ -1835,9 +1842,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t issued_parity[kStages];
-      bool issued[kStages];
-      for (int s = 0; s < kStages; ++s) issued[s] = false;
+      uint32_t issued = 0, issued_parity = 0;  // one bit per stage
       for (int u = cta_id; u < total_units && !abort_flag; u += n_ctas) {
         const uint8_t* sfb_tile = args.sfb + (static_cast<size_t>(u) * kgroups) * 512;
         for (int kb = 0; kb < kblocks; ++kb) {
@@ -1846,14 +1851,14 @@ __global__ void __launch_bounds__(C::kThreads, 1)
           bulk_load(sSFB + stage * C::kSfbBytes, sfb_tile + static_cast<size_t>(kb) * C::kSfbBytes, C::kSfbBytes,
                     &full[stage]);
           tma_load_2d(sB + stage * C::kTileBytesB, &tmap_b, &full[stage], kb * (BK / 2), u * BN);
-          issued[stage] = true;
-          issued_parity[stage] = phase;
+          issued |= 1u << stage;
+          issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
       if (abort_flag)
         for (int s = 0; s < kStages; ++s)
-          if (issued[s]) mbar_wait_bounded(&full[s], issued_parity[s], nullptr);
+          if (issued >> s & 1u) mbar_wait_bounded(&full[s], issued_parity >> s & 1u, nullptr, kDrainLimitNs);
     }
   } else {
     // ------------------------------- prologue: g_a and A into shared memory ---
@@ -1863,11 +1868,9 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     constexpr int kKeep = 10;
     static_assert(kKeep * C::kProThreads >= C::kMaxRows * C::kMaxKb * (BK / 16), "x fits in registers");
     const uint32_t pt = threadIdx.x - 32;
-    const uint32_t kb16 = static_cast<uint32_t>(args.K) / 16;
-    const uint32_t M = static_cast<uint32_t>(args.M);
-    const uint32_t live = M * kb16;
+    const uint32_t live = static_cast<uint32_t>(args.M) * args.kb16.d;
     auto block_src = [&](uint32_t b) {
-      const uint32_t r = b / kb16, j = b - r * kb16;
+      const uint32_t r = args.kb16.div(b), j = b - r * args.kb16.d;
       return reinterpret_cast<const uint4*>(args.x + static_cast<int64_t>(r) * args.ldx + j * 16);
     };
     uint4 lo[kKeep], hi[kKeep];
@@ -1882,44 +1885,24 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       }
     }
     const uint32_t sA0 = smem_u32(sA), sSFA0 = smem_u32(sSFA);
-    // Rows M..127 of the tile: zero codes and zero scales, as the two-call
-    // path gets from the TMA fill and the quantizer's padding rows.
-    {
-      const uint32_t pad_chunks = (128u - M) * 8u;  // 16-byte chunks per k-block
-      for (uint32_t i = pt; i < static_cast<uint32_t>(kblocks) * pad_chunks; i += C::kProThreads) {
-        const uint32_t kb = i / pad_chunks, c = i - kb * pad_chunks;
-        st_shared_v4(sA0 + kb * C::kTileBytesA + M * 128u + c * 16u, 0u, 0u, 0u, 0u);
-      }
-      const uint32_t pad_rows = 128u - M;
-      for (uint32_t i = pt; i < static_cast<uint32_t>(kgroups) * pad_rows; i += C::kProThreads) {
-        const uint32_t jg = i / pad_rows, r = M + (i - jg * pad_rows);
-        st_shared_u32(sSFA0 + jg * 512u + (r & 31u) * 16u + ((r >> 5) & 3u) * 4u, 0u);
-      }
-    }
     uint32_t m = 0;
 #pragma unroll
     for (int i = 0; i < kKeep; ++i) m = max(m, max(amax_bits_bf16x8(lo[i]), amax_bits_bf16x8(hi[i])));
     m = __reduce_max_sync(0xffffffffu, m);
     if (lane == 0) warp_max[warp] = m;
     named_barrier(1, C::kProThreads);
-    if (pt == 0) {
-      uint32_t mm = 0;
-      for (int w = 1; w < C::kThreads / 32; ++w) mm = max(mm, warp_max[w]);
-      // g_a = amax / (6 * 448), or 1 for an all-zero tensor: the dynamic
-      // quantizer's tensor scale, bit for bit.
-      const float amax = __uint_as_float(mm << 16);
-      const float gv = amax > 0.0f ? __fdiv_rn(amax, 2688.0f) : 1.0f;
-      s_g = gv;
-      if (blockIdx.x == 0 && args.g_out) *args.g_out = gv;
-    }
-    named_barrier(1, C::kProThreads);
-    const float g = s_g, six_g = __fmul_rn(6.0f, g);
+    // g_a = amax / (6 * 448), or 1 for an all-zero tensor: the dynamic
+    // quantizer's tensor scale, bit for bit, in every thread.
+    const float amax_x = __uint_as_float(
+        __reduce_max_sync(0xffffffffu, lane >= 1 && lane < C::kThreads / 32 ? warp_max[lane] : 0u) << 16);
+    const float g = amax_x > 0.0f ? __fdiv_rn(amax_x, 2688.0f) : 1.0f, six_g = __fmul_rn(6.0f, g);
+    if (blockIdx.x == 0 && pt == 0 && args.g_out) *args.g_out = g;
     // One 16-element block: E4M3 scale and 16 E2M1 codes, stored where the
     // TMA load of the two-call path would have put them (row r at r * 128 in
     // its k-block tile, 16-byte chunk c at (c ^ r % 8) * 16) and the scale
     // byte at its place in the 512-byte atom of its 64-element group.
     auto quantize_block = [&](uint32_t b, const uint4 v0, const uint4 v1) {
-      const uint32_t r = b / kb16, j = b - r * kb16;
+      const uint32_t r = args.kb16.div(b), j = b - r * args.kb16.d;
       float xf[16];
       unpack_bf16x8(v0, xf);
       unpack_bf16x8(v1, xf + 8);
@@ -1941,67 +1924,75 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     fence_proxy_async_smem();  // the tensor core reads A and its scales through the async proxy
     named_barrier(1, C::kProThreads);
 
-    if (warp == 1 && lane == 0) {
+    if (warp == 1) {
       // ------------------------------------------------------- MMA issuer ---
+      const bool issuer = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
-      const uint32_t sB0 = smem_u32(sB);
-      bool ok = mbar_wait_bounded(aready, 0, &abort_flag);
-      if (!ok) fail();
+      const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
+      const uint64_t a_desc0 = desc_sw128(sA0), b_desc0 = desc_sw128(smem_u32(sB));
+      bool ok = true;
       for (int u = cta_id; ok && u < total_units && !abort_flag; u += n_ctas, ++local) {
         const int acc = local & 1;
         const uint32_t acc_phase = (local >> 1) & 1;
         if (!mbar_wait_bounded(&tempty[acc], acc_phase ^ 1u, &abort_flag)) { fail(); break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem + acc * BN;
+        const uint32_t d_tmem = utmem + acc * BN;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait_bounded(&sfready[stage], phase, &abort_flag)) { fail(); ok = false; break; }
           tc_fence_after();
-          const uint32_t sfa_col = tmem + C::kSfaResCol + kb * 16;
-          const uint32_t sfb_col = tmem + C::kSfbCol + stage * 16;
+          const uint32_t sfa_col = utmem + C::kSfaResCol + kb * 16, sfb_col = utmem + C::kSfbCol + stage * 16;
+          const uint64_t a_desc = a_desc0 + static_cast<uint32_t>(kb) * (C::kTileBytesA >> 4);
+          const uint64_t b_desc = b_desc0 + static_cast<uint32_t>(stage) * (C::kTileBytesB >> 4);
+          if (issuer) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_fp4(d_tmem, desc_sw128(sA0 + kb * C::kTileBytesA + kk * 32),
-                    desc_sw128(sB0 + stage * C::kTileBytesB + kk * 32), C::kIdesc, sfa_col + kk * 4,
-                    sfb_col + kk * 4, (kb | kk) != 0);
-          tc_commit(&empty[stage]);
+            for (int kk = 0; kk < 4; ++kk)
+              mma_fp4(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, C::kIdesc, sfa_col + kk * 4, sfb_col + kk * 4,
+                      (kb | kk) != 0);
+            tc_commit(&empty[stage]);
+          }
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        tc_commit(&tfull[acc]);
+        if (ok && issuer) tc_commit(&tfull[acc]);
       }
-      tc_commit(drain);
+      if (issuer) tc_commit(drain);
       mbar_wait_bounded(drain, 0, nullptr);
-    } else if (warp == 2 && lane == 0) {
+    } else if (warp == 2) {
       // ------------------------------------------- block scales -> TMEM ---
-      for (int kb = 0; kb < kblocks; ++kb)
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          copy_sf_to_tmem(tmem + C::kSfaResCol + kb * 16 + kk * 4, desc_sf(sSFA0 + kb * C::kSfaBytes + kk * 512));
-      tc_commit(aready);
+      const bool issuer = elect_one();
       int stage = 0;
       uint32_t phase = 0;
-      const uint32_t sSFB0 = smem_u32(sSFB);
+      const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
+      const uint64_t sfa_desc0 = desc_sf(sSFA0), sfb_desc0 = desc_sf(smem_u32(sSFB));
       bool ok = true;
       for (int u = cta_id; ok && u < total_units && !abort_flag; u += n_ctas) {
+        const bool with_a = u == cta_id;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait_bounded(&full[stage], phase, &abort_flag)) { fail(); ok = false; break; }
           tc_fence_after();
+          const uint32_t sfa_col = utmem + C::kSfaResCol + kb * 16, sfb_col = utmem + C::kSfbCol + stage * 16;
+          const uint64_t sfa_desc = sfa_desc0 + static_cast<uint32_t>(kb) * (C::kSfaBytes >> 4);
+          const uint64_t sfb_desc = sfb_desc0 + static_cast<uint32_t>(stage) * (C::kSfbBytes >> 4);
+          if (issuer) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            copy_sf_to_tmem(tmem + C::kSfbCol + stage * 16 + kk * 4, desc_sf(sSFB0 + stage * C::kSfbBytes + kk * 512));
-          tc_commit(&sfready[stage]);
+            for (int kk = 0; kk < 4; ++kk) {
+              if (with_a) copy_sf_to_tmem(sfa_col + kk * 4, sfa_desc + kk * (512 >> 4));
+              copy_sf_to_tmem(sfb_col + kk * 4, sfb_desc + kk * (512 >> 4));
+            }
+            tc_commit(&sfready[stage]);
+          }
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
-      tc_commit(drain_cp);
+      if (issuer) tc_commit(drain_cp);
       mbar_wait_bounded(drain_cp, 0, nullptr);
-    } else if (warp >= 3 && warp < 3 + C::kEpiWarps) {
+    } else if (warp == 4 || warp == 8) {
       // --------------------------------------------------------- epilogue ---
-      const int quarter = warp & 3;
-      uint8_t* buf_ptr = sEpi + (warp - 3) * kEpiBufBytes;
-      const uint32_t buf = smem_u32(buf_ptr);
+      // 32 rows x 64 columns; row `lane` of the staged box is 8 chunks of 16 B
+      // at chunk position (c ^ lane % 8).
+      const int colbase = warp == 8 ? kEpiCols : 0;
+      const uint32_t buf = smem_u32(sEpi + (warp == 8 ? kEpiBufBytes : 0));
       const float scale = __fmul_rn(g, __ldg(args.gb));
       int local = 0;
       for (int u = cta_id; u < total_units; u += n_ctas, ++local) {
@@ -2014,37 +2005,36 @@ __global__ void __launch_bounds__(C::kThreads, 1)
         }
         if (!__shfl_sync(0xffffffffu, ok, 0)) break;
         tc_fence_after();
-        uint32_t r[128];
-        const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(taddr + c * 32, r + 32 * c);
+        uint32_t r[64];
+        const uint32_t taddr = tmem + acc * BN + colbase;
+        tmem_ld32(taddr, r);
+        tmem_ld32(taddr + 32, r + 32);
         tmem_ld_wait();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[acc]);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (lane == 0) bulk_wait_read_all();
-          __syncwarp();
+        for (int c = 0; c < 8; ++c) {
+          const uint32_t* v = r + 8 * c;
+          st_shared_v4(buf + lane * 128 + ((c ^ (lane & 7)) << 4),
+                       pack_bf16x2(__uint_as_float(v[0]) * scale, __uint_as_float(v[1]) * scale),
+                       pack_bf16x2(__uint_as_float(v[2]) * scale, __uint_as_float(v[3]) * scale),
+                       pack_bf16x2(__uint_as_float(v[4]) * scale, __uint_as_float(v[5]) * scale),
+                       pack_bf16x2(__uint_as_float(v[6]) * scale, __uint_as_float(v[7]) * scale));
+        }
+        __syncwarp();
+        const int cc = lane & 7, x = u * BN + colbase + cc * 8;
+        if (x < args.N) {  // N % 16 == 0: a chunk is inside or outside
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const uint32_t* v = r + 64 * h + 8 * c;
-            st_shared_v4(buf + lane * 128 + ((c ^ (lane & 7)) << 4),
-                         pack_bf16x2(__uint_as_float(v[0]) * scale, __uint_as_float(v[1]) * scale),
-                         pack_bf16x2(__uint_as_float(v[2]) * scale, __uint_as_float(v[3]) * scale),
-                         pack_bf16x2(__uint_as_float(v[4]) * scale, __uint_as_float(v[5]) * scale),
-                         pack_bf16x2(__uint_as_float(v[6]) * scale, __uint_as_float(v[7]) * scale));
-          }
-          fence_proxy_async_smem();
-          __syncwarp();
-          const int x = u * BN + h * kEpiCols, y = quarter * 32;
-          if (lane == 0 && x < args.N && y < args.M) {
-            tma_store_2d(&tmap_out, buf_ptr, x, y);
-            bulk_commit_group();
+          for (int it = 0; it < 8; ++it) {
+            const int rr = 4 * it + (lane >> 3);
+            if (rr < args.M && in_bounds(args.status, x + 8 <= args.N))
+              *reinterpret_cast<uint4*>(args.out + static_cast<int64_t>(rr) * args.ldo + x) =
+                  ld_shared_v4(buf + rr * 128 + ((cc ^ (rr & 7)) << 4));
           }
         }
+        __syncwarp();  // the next tile overwrites the box
       }
-      if (lane == 0) bulk_wait_all();
     }
   }
 
@@ -2507,14 +2497,17 @@ nvfp4_status launch_dynamic(const uint16_t* x, int64_t M, int64_t K, int64_t ldx
     }
   }
   const int64_t tiles_n = (N + C::BN - 1) / C::BN;
-  CUtensorMap mb, mo;
-  if (!make_code_map(&mb, w_codes, N, K, C::BN) || !make_out_map(&mo, out_bf16, M, N, ldo)) return NVFP4_ERR_CUDA;
+  CUtensorMap mb;
+  if (!make_code_map(&mb, w_codes, N, K, C::BN)) return NVFP4_ERR_CUDA;
   DynArgs args = {};
   args.x = x;
   args.ldx = ldx;
   args.sfb = w_scales;
   args.gb = g_w;
   args.g_out = g_out;
+  args.out = static_cast<uint16_t*>(out_bf16);
+  args.ldo = ldo;
+  args.kb16 = FastDiv(static_cast<uint32_t>(K / 16));
   args.M = static_cast<int>(M);
   args.N = static_cast<int>(N);
   args.K = static_cast<int>(K);
@@ -2523,7 +2516,7 @@ nvfp4_status launch_dynamic(const uint16_t* x, int64_t M, int64_t K, int64_t ldx
   const int sms = sm_count();
   if (sms <= 0) return NVFP4_ERR_CUDA;
   const int ctas = static_cast<int>(tiles_n < sms ? tiles_n : sms);
-  if (launch_pdl(nvfp4_linear_dyn_kernel<C>, dim3(ctas), dim3(C::kThreads), C::kSmemBytes, stream, mb, mo, args) !=
+  if (launch_pdl(nvfp4_linear_dyn_kernel<C>, dim3(ctas), dim3(C::kThreads), C::kSmemBytes, stream, mb, args) !=
       cudaSuccess)
     return NVFP4_ERR_CUDA;
   count_launches(1);
