@@ -144,8 +144,8 @@ __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
 
 // Write one staged 32 x 64 bf16 box (rows of 128 B whose 16-byte chunks sit at
 // chunk ^ (row % 8)) to out[y.., x..] with coalesced 16-byte stores: per
-// instruction the warp writes 4 rows x 128 B; rows at or past M are skipped.
-// (In the bounds-checked build each store is also checked against [M, N].)
+// instruction the warp writes 4 rows x 128 B; rows at or past M and chunks at or
+// past N (N % 16 == 0, so a chunk is inside or outside) are skipped.
 __device__ __forceinline__ void store_box_lsu(uint32_t buf, uint16_t* out, int64_t ldo, int x, int y, int M, int N,
                                               int lane, int* status) {
   const int cc = lane & 7;
@@ -153,7 +153,7 @@ __device__ __forceinline__ void store_box_lsu(uint32_t buf, uint16_t* out, int64
   for (int it = 0; it < 8; ++it) {
     const int rr = 4 * it + (lane >> 3);
     const uint4 v = ld_shared_v4(buf + rr * 128 + ((cc ^ (rr & 7)) << 4));
-    if (y + rr < M && in_bounds(status, x + cc * 8 + 8 <= N))
+    if (y + rr < M && x + cc * 8 < N && in_bounds(status, x + cc * 8 + 8 <= N))
       *reinterpret_cast<uint4*>(out + static_cast<int64_t>(y + rr) * ldo + x + cc * 8) = v;
   }
 }
@@ -2198,7 +2198,7 @@ nvfp4_status launch_pair(const uint8_t* a_codes, const uint8_t* a_scales, const 
                          const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N, int64_t K, void* out_bf16,
                          int64_t ldo, cudaStream_t stream, const GemmArgs* extra = nullptr,
                          uint32_t idesc_fmt = 0) {
-  const int64_t tiles_m = (M + BM - 1) / BM, tiles_n = N / C::BN;
+  const int64_t tiles_m = (M + BM - 1) / BM, tiles_n = (N + C::BN - 1) / C::BN;  // a column tail reads zeros
   const int64_t units = ((tiles_m + 1) / 2) * tiles_n;
   if (units >= (1ll << 31)) return NVFP4_ERR_SHAPE;
   CUtensorMap ma, mb, mb_half, msa, msb, mo;
@@ -2579,8 +2579,15 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
   // the pairs would (measured faster at M = 256 with N = 5120 or 7168, slower
   // with N = 27648).
   using Pair = PairCfg<NVFP4_GEMM_PAIR_STAGES>;
-  if (NVFP4_GEMM_PAIR && N % 256 == 0 && tiles_m >= 2) {
-    const int64_t pair_units = ((tiles_m + 1) / 2) * (N / 256);
+  // A column tail (N % 256 != 0) costs the pairs at most one tile column of
+  // zeros, and single CTAs still take twice as long: 8192 x 7296 x 5120 191 ->
+  // 92 us, 256 x 27520 x 5120 28.7 -> 21.3, 2048 x 2176 x 8192 28.8 -> 15.6.
+  // Only with a short K and at most one 128 x 128 tile per SM are single CTAs
+  // as fast or faster (K = 1536: 2048 x 1152 6.3 against 7.2 us, 1024 x 2304
+  // 6.2 / 6.3; K = 2048: 256 x 9728 7.7 / 7.3).
+  const bool single = K / BK <= 6 && tiles_m * ((N + 127) / 128) <= sm_count();
+  if (NVFP4_GEMM_PAIR && tiles_m >= 2 && !single) {
+    const int64_t pair_units = ((tiles_m + 1) / 2) * ((N + 255) / 256);
     if (use_w_resident(pair_units, K, resident_pairs<PairRes, false>()))
       return launch_pair<PairRes>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s,
                                   nullptr, idesc_fmt);

@@ -384,3 +384,19 @@ def test_last_wave_in_half_tiles(N, M, Nn, K):
     ref = O.linear(a_c, a_s, g_a, w_c, w_s, g_w)
     assert_close(f32(out[:, :Nn]), ref, what=f"{M}x{Nn}x{K}")
     assert torch.isnan(out[:, Nn:].float()).all()
+
+
+@pytest.mark.parametrize("M,Nn,K,ldo", [
+    # CTA pairs with a column tail: inside the first and the second half of the last tile, one
+    # 16-column chunk, with half tiles in the last wave, an M tail and a padded pitch
+    (300, 10000, 1792, 10000), (130, 19472, 2304, 19480), (640, 7312, 2048, 7312), (1000, 2576, 4096, 2584),
+    (2000, 1296, 2304, 1296), (600, 15376, 1536, 15376)])
+def test_pair_column_tails(N, M, Nn, K, ldo):
+    gen = torch.Generator().manual_seed(M * 1000 + Nn * 10 + K)
+    a_c, a_s = random_operand(M, K, gen)
+    w_c, w_s = random_operand(Nn, K, gen)
+    g_a, g_w = np.float32(0.0173), np.float32(0.00091)
+    out = run_linear(N, a_c, a_s, g_a, w_c, w_s, g_w, M, Nn, K, ldo=ldo)
+    ref = O.linear(a_c, a_s, g_a, w_c, w_s, g_w)
+    assert_close(f32(out[:, :Nn]), ref, what=f"{M}x{Nn}x{K}")
+    assert torch.isnan(out[:, Nn:].float()).all()
