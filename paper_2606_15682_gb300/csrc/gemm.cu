@@ -504,7 +504,8 @@ __global__ void __launch_bounds__(C::kThreads, 1)
 //   - warps walk these loops converged and one elected lane issues, which
 //     leaves descriptors in uniform registers.
 // GB300, back to back: 8192 x 55296 x 5120 719 -> 638 us, 8192 x 5120 x 27648
-// 366 -> 316, 8192 x 5120 x 8192 113 -> 97, 2048 x 17920 x 1536 29.2 -> 26.4.
+// 366 -> 316, 8192 x 5120 x 8192 113 -> 97, 2048 x 17920 x 1536 29.2 -> 25.4
+// (a form that kept W in shared memory for K <= 1536: 26.5).
 // Sharing W between two pairs by multicast (clusters of four) changed no
 // pair's rate, and only 144 SMs fit such clusters.
 
@@ -590,21 +591,10 @@ __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint64_t* bar, uint3
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
 }
 
-// RES_: the W-resident form for 1024 <= K <= 1536.  A pair walks a run of
-// consecutive units that share one W tile.  The run's first unit loads the W
-// tile's codes for the whole K into shared memory and copies its block scales
-// for the whole K into TMEM (8 columns per 64-deep k group); the run's later
-// units stream only A and its scales (18 KB per k-block and CTA instead of
-// 38 KB).  The A ring keeps 4 stages.
-template <int STAGES_, bool RES_ = false>
+template <int STAGES_>
 struct PairCfg {
   static constexpr int BN = 256;                 // MMA N (both halves of the pair)
   static constexpr int kStages = STAGES_;
-  static constexpr bool kRes = RES_;
-  static constexpr int kResKblocks = 6;                          // K <= 1536 in the resident form
-  static constexpr int kBTiles = kRes ? kResKblocks : kStages;   // W tiles held in shared memory
-  static constexpr uint32_t kSfbResCol = BN;                     // resident W scales
-  static constexpr uint32_t kSfaResCol = BN + 32 * kResKblocks;  // per-stage A scales, 16 columns each
   static constexpr int kEpiWarps = 8;            // 128 rows x 256 accumulator columns per CTA
   static constexpr int kCopyWarps = NVFP4_GEMM_COPY_WARPS;  // warps issuing the scale copies (1, 2 or 4)
   static constexpr int kEpi0 = 2 + kCopyWarps;   // first epilogue warp
@@ -616,14 +606,12 @@ struct PairCfg {
   static constexpr uint32_t kStageBytes = kTileBytesA + kTileBytesB + kSfaBytes + kSfbBytes;
   static constexpr uint32_t kSfCols = 16 + 32;
   static constexpr uint32_t kSfTmemCol = BN;
-  static constexpr size_t kSmemBytes = 1024 + kStages * (kStageBytes - kTileBytesB) + kBTiles * kTileBytesB +
-                                       kEpiWarps * kEpiBufBytes + 512 /*barriers*/;
+  static constexpr size_t kSmemBytes = 1024 + kStages * kStageBytes + kEpiWarps * kEpiBufBytes + 512 /*barriers*/;
   static constexpr uint32_t kIdesc = (1u << 7) | (1u << 10) | (static_cast<uint32_t>(BN >> 3) << 17) |
                                      (static_cast<uint32_t>(256 >> 4) << 24);
   static constexpr uint32_t kIdescHalf = (1u << 7) | (1u << 10) | (static_cast<uint32_t>(BN / 2 >> 3) << 17) |
                                          (static_cast<uint32_t>(256 >> 4) << 24);
-  static_assert(kRes ? kSfaResCol + kStages * 16 <= kTmemCols : kSfTmemCol + kStages * kSfCols <= kTmemCols,
-                "TMEM budget");
+  static_assert(kSfTmemCol + kStages * kSfCols <= kTmemCols, "TMEM budget");
   static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
 };
 
@@ -639,7 +627,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
   uint8_t* sB = sA + kStages * C::kTileBytesA;
-  uint8_t* sEpi = sB + C::kBTiles * C::kTileBytesB;
+  uint8_t* sEpi = sB + kStages * C::kTileBytesB;
   uint8_t* sSFA = sEpi + C::kEpiWarps * kEpiBufBytes;
   uint8_t* sSFB = sSFA + kStages * C::kSfaBytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(sSFB + kStages * C::kSfbBytes);  // codes landed, scales in TMEM
@@ -655,42 +643,23 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int kblocks = args.K / BK;
   const int kgroups = args.K / 64;
-  if (C::kRes && (kblocks < kStages || kblocks > C::kResKblocks)) {
-    // Outside the resident form's K range (the host never launches it so):
-    // the whole grid returns before touching any barrier or TMEM.
-    if (blockIdx.x == 0 && threadIdx.x == 0) set_status(args.status, NVFP4_ERR_SHAPE);
-    return;
-  }
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int msup = (args.tiles_m + 1) / 2;
   const int tiles = msup * args.tiles_n;
   // The tiles of a partly filled last wave are split into two 256 x 128 units
-  // each when all of those fit in it (not in the resident form).
-  const int total_units = C::kRes ? tiles : 2 * tiles - args.full_units;
+  // each when all of those fit in it.
+  const int total_units = 2 * tiles - args.full_units;
   const int pair_id = blockIdx.x / 2, n_pairs = gridDim.x / 2;
-  // Units of this pair: every n_pairs-th one, or (resident form) a
-  // contiguous run in W-tile-major order, so that consecutive units share nb.
-  const int run = C::kRes ? (total_units + n_pairs - 1) / n_pairs : 0;
-  const int u_first = C::kRes ? pair_id * run : pair_id;
-  const int u_end = C::kRes ? min(total_units, u_first + run) : total_units;
-  const int u_step = C::kRes ? 1 : n_pairs;
   // Tile (ms, nb) of unit u and its columns: half -1 all 256, else 128 from 128 * half.
   auto coords = [&](int u, int* ms, int* nb, int* half) {
     *half = -1;
-    if (C::kRes) {
-      // Within a W tile the row super-tiles start at a rotation of nb, so
-      // that the pairs running at the same time read different A tiles.
-      *nb = u / msup;
-      *ms = (u - *nb * msup + *nb) % msup;
-    } else {
-      const int s = u - args.full_units;
-      if (s >= 0) {
-        *half = s & 1;
-        u = args.full_units + (s >> 1);
-      }
-      unit_coords(u, msup, args.tiles_n, args.group_m, ms, nb);
+    const int s = u - args.full_units;
+    if (s >= 0) {
+      *half = s & 1;
+      u = args.full_units + (s >> 1);
     }
+    unit_coords(u, msup, args.tiles_n, args.group_m, ms, nb);
   };
 
   if (threadIdx.x == 0) {
@@ -731,30 +700,24 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   };
 
   // A producer warp walks this pair's units and k-blocks; prep(ms, nb, half)
-  // gives a unit's start rows, and load(stage, kb, rows, wide, load_w), in one
+  // gives a unit's start rows, and load(stage, kb, rows, wide), in one
   // lane, fills a stage once `free` says that it may be rewritten.
   auto produce = [&](uint64_t* free, auto&& prep, auto&& load) {
     const bool issuer = elect_one();
     int stage = 0;
     uint32_t phase = 0;
-    int prev_nb = -1;
     // Test-only injected fault: both CTAs of pair 0 leave their first stage
     // neither armed nor loaded, so no copy is ever in flight for it and the
     // consumers' bounded waits on it run out.
     bool skip = args.fault_skip_stage && pair_id == 0;
-    for (int u = u_first; u < u_end && !abort_flag; u += u_step) {
+    for (int u = pair_id; u < total_units && !abort_flag; u += n_pairs) {
       int ms, nb, half;
       coords(u, &ms, &nb, &half);
-      // W codes and scales: every unit, or (resident form) a run's first.
-      // Resident W tile kb is rewritten only after the MMAs of k-block kb of
-      // the previous unit completed: the stage's barrier covers the MMAs up
-      // to kStages k-blocks back, and kblocks >= kStages.
-      const bool load_w = !C::kRes || nb != prev_nb, wide = C::kRes || half < 0;
-      prev_nb = nb;
+      const bool wide = half < 0;
       const int2 rows = prep(ms, nb, half);
       for (int kb = 0; kb < kblocks; ++kb) {
         if (!mbar_wait_bounded(&free[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
-        if (issuer && !skip) load(stage, kb, rows, wide, load_w);
+        if (issuer && !skip) load(stage, kb, rows, wide);
         skip = false;
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
@@ -767,20 +730,19 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     produce(empty,
             [&](int ms, int nb, int half) {
               return make_int2(min(ms * 2 + static_cast<int>(rank), args.tiles_m - 1) * BM,  // a spare CTA redoes the last tile
-                               nb * BN + (C::kRes || half < 0 ? static_cast<int>(rank) * 128
-                                                              : half * 128 + static_cast<int>(rank) * 64));
+                               nb * BN + (half < 0 ? static_cast<int>(rank) * 128
+                                                   : half * 128 + static_cast<int>(rank) * 64));
             },
-            [&](int stage, int kb, int2 rows, bool wide, bool load_w) {
+            [&](int stage, int kb, int2 rows, bool wide) {
               uint8_t* a_dst = sA + stage * C::kTileBytesA;
-              uint8_t* b_dst = sB + (C::kRes ? kb : stage) * C::kTileBytesB;
+              uint8_t* b_dst = sB + stage * C::kTileBytesB;
               const CUtensorMap* map_b = wide ? &tmap_b : &tmap_b_half;
               const int kx = kb * (BK / 2);
               if (leader)  // both CTAs' codes are counted on the leader's barrier
-                mbar_arrive_expect_tx(
-                    &full[stage],
-                    2 * (C::kTileBytesA + (load_w ? (wide ? C::kTileBytesB : C::kTileBytesB / 2) : 0u)));
+                mbar_arrive_expect_tx(&full[stage],
+                                      2 * (C::kTileBytesA + (wide ? C::kTileBytesB : C::kTileBytesB / 2)));
               tma_load_2d_to(a_dst, &tmap_a, &full[stage], kx, rows.x, 0);
-              if (load_w) tma_load_2d_to(b_dst, map_b, &full[stage], kx, rows.y, 0);
+              tma_load_2d_to(b_dst, map_b, &full[stage], kx, rows.y, 0);
             });
   } else if (warp == 1 && !leader) {
     // --------------------------------- producer (peer): both CTAs' A scales ---
@@ -791,10 +753,10 @@ __global__ void __launch_bounds__(C::kThreads, 1)
               return make_int2(min(ms * 2, args.tiles_m - 1) * kgroups * 2,
                                min(ms * 2 + 1, args.tiles_m - 1) * kgroups * 2);
             },
-            [&](int stage, int kb, int2 rows, bool wide, bool load_w) {
+            [&](int stage, int kb, int2 rows, bool wide) {
               uint8_t* dst = sSFA + stage * C::kSfaBytes;
-              mbar_arrive_expect_tx_cluster(
-                  &sffull[stage], 0, 2 * (C::kSfaBytes + (load_w ? (wide ? C::kSfbBytes : C::kSfaBytes) : 0u)));
+              mbar_arrive_expect_tx_cluster(&sffull[stage], 0,
+                                            2 * (C::kSfaBytes + (wide ? C::kSfbBytes : C::kSfaBytes)));
               tma_load_2d_multicast(dst, &tmap_sfa, &sffull[stage], 0, rows.x + kb * 8, 0, 1u);
               tma_load_2d_to(dst, &tmap_sfa, &sffull[stage], 0, rows.y + kb * 8, 0);
             });
@@ -805,8 +767,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
               const int row = (nb * 2 + max(half, 0)) * kgroups * 2;
               return make_int2(row, row + kgroups * 2);
             },
-            [&](int stage, int kb, int2 rows, bool wide, bool load_w) {
-              if (!load_w) return;
+            [&](int stage, int kb, int2 rows, bool wide) {
               uint8_t* dst = sSFB + stage * C::kSfbBytes;
               tma_load_2d_multicast(dst, &tmap_sfb, &sffull[stage], 0, rows.x + kb * 8, 0, 3u);
               if (wide)
@@ -828,19 +789,18 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     const auto wait = [&](uint64_t* bar, uint32_t parity) {
       return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, &abort_flag)) != 0;
     };
-    for (int u = u_first; u < u_end; u += u_step, ++local) {
+    for (int u = pair_id; u < total_units; u += n_pairs, ++local) {
       if (!wait(tempty, (local & 1) ^ 1u)) { fail(); break; }
       tc_fence_after();
       const uint32_t idesc =
-          (C::kRes || u < args.full_units ? C::kIdesc : C::kIdescHalf) | args.idesc_fmt;
+          (u < args.full_units ? C::kIdesc : C::kIdescHalf) | args.idesc_fmt;
       bool ok = true;
       for (int kb = 0; kb < kblocks; ++kb) {
         if (!ready && !wait(&full[stage], phase)) { fail(); ok = false; break; }
         tc_fence_after();
-        const uint32_t sfa_col = utmem + (C::kRes ? C::kSfaResCol + stage * 16 : C::kSfTmemCol + stage * C::kSfCols);
-        const uint32_t sfb_col = C::kRes ? utmem + C::kSfbResCol + kb * 32 : sfa_col + 16;
+        const uint32_t sfa_col = utmem + C::kSfTmemCol + stage * C::kSfCols, sfb_col = sfa_col + 16;
         const uint64_t a_desc = a_desc0 + static_cast<uint32_t>(stage) * (C::kTileBytesA >> 4);
-        const uint64_t b_desc = b_desc0 + static_cast<uint32_t>(C::kRes ? kb : stage) * (C::kTileBytesB >> 4);
+        const uint64_t b_desc = b_desc0 + static_cast<uint32_t>(stage) * (C::kTileBytesB >> 4);
         const int next = stage + 1 == kStages ? 0 : stage + 1;
         const uint32_t next_phase = next ? phase : phase ^ 1u;
         if (issuer) {
@@ -870,33 +830,25 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     uint32_t phase = 0;
     const uint32_t utmem = __shfl_sync(0xffffffffu, tmem, 0);
     const uint64_t sfa_desc0 = desc_sf(smem_u32(sSFA)), sfb_desc0 = desc_sf(smem_u32(sSFB));
-    int prev_nb = -1;
-    for (int u = u_first; u < u_end && !abort_flag; u += u_step) {
+    for (int u = pair_id; u < total_units && !abort_flag; u += n_pairs) {
       bool ok = true;
       int ms, nb, half;
       coords(u, &ms, &nb, &half);
-      // Resident form: a run's first unit copies the W scales for the whole
-      // K.  The copy of k-block kb's columns waited (through the empty
-      // barrier) for the MMAs of the previous unit's k-block kb.
-      const bool copy_w = !C::kRes || nb != prev_nb, wide = C::kRes || half < 0;
-      prev_nb = nb;
+      const bool wide = half < 0;
       for (int kb = 0; kb < kblocks; ++kb) {
         // The scales have landed, and the MMAs that read this TMEM slot are done.
         if (!mbar_wait_bounded(&sffull[stage], phase, &abort_flag) ||
             !mbar_wait_bounded(&empty[stage], phase ^ 1u, &abort_flag)) { fail(); ok = false; break; }
         tc_fence_after();
-        const uint32_t sfa_col = utmem + (C::kRes ? C::kSfaResCol + stage * 16 : C::kSfTmemCol + stage * C::kSfCols);
-        const uint32_t sfb_col = C::kRes ? utmem + C::kSfbResCol + kb * 32 : sfa_col + 16;
+        const uint32_t sfa_col = utmem + C::kSfTmemCol + stage * C::kSfCols, sfb_col = sfa_col + 16;
         const uint64_t sfa_desc = sfa_desc0 + static_cast<uint32_t>(stage) * (C::kSfaBytes >> 4);
         const uint64_t sfb_desc = sfb_desc0 + static_cast<uint32_t>(stage) * (C::kSfbBytes >> 4);
         if (issuer) {
 #pragma unroll
           for (int kk = kk0; kk < kk0 + kPerWarp; ++kk) {
             copy_sf_to_tmem_pair(sfa_col + kk * 4, sfa_desc + kk * (512 >> 4));
-            if (copy_w) {
-              copy_sf_to_tmem_pair(sfb_col + kk * 8, sfb_desc + kk * (512 >> 4));
-              if (wide) copy_sf_to_tmem_pair(sfb_col + kk * 8 + 4, sfb_desc + (C::kSfaBytes + kk * 512) / 16);
-            }
+            copy_sf_to_tmem_pair(sfb_col + kk * 8, sfb_desc + kk * (512 >> 4));
+            if (wide) copy_sf_to_tmem_pair(sfb_col + kk * 8 + 4, sfb_desc + (C::kSfaBytes + kk * 512) / 16);
           }
           tc_commit_pair(&full[stage], 0x3);
         }
@@ -924,7 +876,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     const uint32_t q_cols = static_cast<uint32_t>(args.N) >> 1;  // SwiGLU outputs per row
     const uint32_t q_kgroups = q_cols >> 6;
     int local = 0;
-    for (int u = u_first; u < u_end; u += u_step, ++local) {
+    for (int u = pair_id; u < total_units; u += n_pairs, ++local) {
       int ms, nb, half;
       coords(u, &ms, &nb, &half);
       const int mb = ms * 2 + static_cast<int>(rank);  // mb >= tiles_m: nothing is stored
@@ -1025,7 +977,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     const uint32_t buf = smem_u32(buf_ptr);
     const float scale = args.ga ? __fmul_rn(__ldg(args.ga), __ldg(args.gb)) : 1.0f;
     int local = 0;
-    for (int u = u_first; u < u_end; u += u_step, ++local) {
+    for (int u = pair_id; u < total_units; u += n_pairs, ++local) {
       int ms, nb, half;
       coords(u, &ms, &nb, &half);
       const int mb = ms * 2 + static_cast<int>(rank);  // mb >= tiles_m: nothing is stored
@@ -1167,7 +1119,6 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   constexpr int BN = C::BN;
   constexpr int kStages = C::kStages;
   constexpr int kEpi0 = C::kEpi0;
-  static_assert(!C::kRes, "streaming form only");
   static_assert(C::kEpiWarps == 8, "eight reduction warps");
   static_assert(128u * 1024u <= kStages * (C::kTileBytesA + C::kTileBytesB), "the partial fits in the ring");
   extern __shared__ uint8_t smem_raw[];
@@ -2232,7 +2183,7 @@ nvfp4_status launch_pair(const uint8_t* a_codes, const uint8_t* a_scales, const 
   // x 5120 x 13824, 80 tiles, 38.5 -> 34.0 us; 256 x 27648 x 5120, 108 tiles,
   // 22.9 -> 21.3; 8192 x 5120 x 27648, 640 tiles, 316.9 -> 312.1).
   const int64_t last = units % pairs_max;
-  const bool split = !C::kRes && last > 0 && 2 * last <= pairs_max;
+  const bool split = last > 0 && 2 * last <= pairs_max;
   args.full_units = static_cast<int>(split ? units - last : units);
   const int64_t total = 2 * units - args.full_units;
   const int pairs = static_cast<int>(total < pairs_max ? total : pairs_max);
@@ -2532,24 +2483,6 @@ nvfp4_status launch_dynamic(const uint16_t* x, int64_t M, int64_t K, int64_t ldx
 #ifndef NVFP4_GEMM_PAIR
 #define NVFP4_GEMM_PAIR 1  // 0: never use the CTA-pair kernel
 #endif
-#ifndef NVFP4_GEMM_RES
-#define NVFP4_GEMM_RES 1  // 0: never use the W-resident form
-#endif
-
-using PairRes = PairCfg<4, true>;
-
-// The W-resident form pays when a pair gets runs of two or more units (more
-// units than pairs); K must fit its shared-memory and TMEM budget, and its
-// copy-after-read order needs at least as many k-blocks as ring stages.
-// Measured on GB300 (graph-replayed, L2 flushed): gate_up of the 1.5B
-// prefill (2048 x 17920 x 1536) 38.0 -> 35.7 us; with 4 k-blocks
-// (8192 x 5120 x 1024) it was slower, so it starts at 5.
-bool use_w_resident(int64_t pair_units, int64_t K, int pairs) {
-  const int64_t kblocks = K / BK;
-  return NVFP4_GEMM_RES && pairs > 0 && pair_units > pairs && kblocks >= PairRes::kStages + 1 &&
-         kblocks <= PairRes::kResKblocks;
-}
-
 }  // namespace
 }  // namespace nvfp4
 
@@ -2588,9 +2521,6 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
   const bool single = K / BK <= 6 && tiles_m * ((N + 127) / 128) <= sm_count();
   if (NVFP4_GEMM_PAIR && tiles_m >= 2 && !single) {
     const int64_t pair_units = ((tiles_m + 1) / 2) * ((N + 255) / 256);
-    if (use_w_resident(pair_units, K, resident_pairs<PairRes, false>()))
-      return launch_pair<PairRes>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s,
-                                  nullptr, idesc_fmt);
     if (2 * pair_units >= resident_pairs<Pair, false>())
       return launch_pair<Pair>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, nullptr,
                                idesc_fmt);
@@ -2671,10 +2601,6 @@ NVFP4_API nvfp4_status nvfp4_linear_swiglu_quantize(const uint8_t* a_codes, cons
   extra.q_codes = out_codes;
   extra.q_scales = out_scales;
   extra.g_out = g_out;
-  const int64_t pair_units = ((M + 2 * BM - 1) / (2 * BM)) * (2 * I / 256);
-  if (use_w_resident(pair_units, K, resident_pairs<PairRes, true>()))
-    return launch_pair<PairRes, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, 2 * I, K, nullptr, 0,
-                                      static_cast<cudaStream_t>(stream), &extra);
   return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, 2 * I,
                                                            K, nullptr, 0, static_cast<cudaStream_t>(stream), &extra);
 }
@@ -2695,10 +2621,6 @@ NVFP4_API nvfp4_status mxfp4_linear_swiglu_quantize(const uint8_t* a_codes, cons
   extra.q_codes = out_codes;
   extra.q_scales = out_scales;
   extra.q_mode = rotate ? 2u : 1u;
-  const int64_t pair_units = ((M + 2 * BM - 1) / (2 * BM)) * (2 * I / 256);
-  if (use_w_resident(pair_units, K, resident_pairs<PairRes, true>()))
-    return launch_pair<PairRes, true>(a_codes, a_scales, nullptr, w_codes, w_scales, nullptr, M, 2 * I, K, nullptr,
-                                      0, static_cast<cudaStream_t>(stream), &extra, kScaleE8M0);
   return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, nullptr, w_codes, w_scales, nullptr, M,
                                                            2 * I, K, nullptr, 0, static_cast<cudaStream_t>(stream),
                                                            &extra, kScaleE8M0);

@@ -127,7 +127,7 @@ def run_mx_linear(N, a_codes, a_scales_rm, w_codes, w_scales_rm, M, Nn, K, ldo=N
 @pytest.mark.parametrize("M,Nn,K", [(128, 128, 256), (1, 16, 256), (130, 144, 512), (257, 384, 1024),
                                     # N % 256 == 0: 256 x 256 CTA-pair tiles (enough of them)
                                     (2048, 1280, 1024),
-                                    # more pair tiles than pairs with 6 k-blocks: the W-resident form
+                                    # more pair tiles than pairs with 6 k-blocks
                                     (2048, 2560, 1536),
                                     # too few pair tiles with a long K: split-K clusters (S = 4, 2)
                                     (256, 768, 4096), (200, 7168, 4608)])
@@ -227,7 +227,7 @@ def test_mx_linear_swiglu_quantize(N, M, I, K, rotate):
 
 @pytest.mark.parametrize("rotate", [False, True], ids=["plain", "rotated"])
 def test_mx_linear_swiglu_quantize_prefill_shape_then_down(N, rotate):
-    """The 1.5B-prefill MLP shape (M=2048, I=8960, K=1536; the W-resident form)
+    """The 1.5B-prefill MLP shape (M=2048, I=8960, K=1536)
     on sampled rows, then fed to the MXFP4 down projection as its A operand."""
     M, I, K, Hd = 2048, 8960, 1536, 1536
     rows = np.sort(np.r_[np.random.default_rng(3).choice(M - 1, 40, replace=False), M - 1])
