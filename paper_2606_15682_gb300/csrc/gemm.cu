@@ -203,7 +203,7 @@ struct GemmArgs {
   // (NVFP4), kScaleE8M0 for UE8M0 (MXFP4).  With ga == nullptr the epilogue
   // applies no global scale (MXFP4 has none).
   uint32_t idesc_fmt;
-  // Fused SwiGLU + quantization epilogue (pair kernel, kSwiGLU): outputs.
+  // Fused SwiGLU + quantization epilogue (kSwiGLU): outputs.
   uint8_t* q_codes;   // [M, N/4] bytes: N/2 SwiGLU outputs per row
   uint8_t* q_scales;  // MMA layout for [M, N/2]
   const float* g_out;
@@ -1462,7 +1462,89 @@ __device__ __forceinline__ void skinny_reduce(uint32_t part0, uint32_t rank, uin
   }
 }
 
-template <class C>
+// SwiGLU and quantization of the fp32 tile in this CTA's own ring (one CTA per
+// tile).  W rows are interleaved in blocks of 16 (gate, then the matching up),
+// so a thread takes 32 columns of a row: one 16-element block c of the output.
+// A warp takes 8 rows and step, lanes 8c..8c+7 those of block c (whose chunks
+// the swizzle spreads over all banks); the two halves of a 32-element block are
+// lanes l and l ^ 8.  The arithmetic is the CTA-pair kernel's, element by
+// element.
+__device__ __forceinline__ void skinny_swiglu(const uint8_t* part, uint32_t warp, uint32_t lane, int nb, float scale,
+                                              const GemmArgs& args) {
+  const float g_in = args.q_mode == 0 ? __ldg(args.g_out) : 1.0f;
+  const bool g_ok = g_in > 0.0f && g_in <= FLT_MAX;
+  if (!g_ok && blockIdx.x == 0 && warp == 0 && lane == 0) set_status(args.status, NVFP4_ERR_INVALID_ARG);
+  const float g = g_ok ? g_in : 1.0f, six_g = __fmul_rn(6.0f, g);
+  const uint32_t q_cols = static_cast<uint32_t>(args.N) >> 1, oc0 = static_cast<uint32_t>(nb) * 64;
+  const uint32_t M = static_cast<uint32_t>(args.M), c = lane >> 3;
+  const uint64_t sc_bytes = 128ull * (q_cols / 16), code_bytes = static_cast<uint64_t>(M) * (q_cols / 2);
+  auto store_scales = [&](uint32_t row, uint32_t sc) {
+    const uint64_t off = mma_scale_offset(row, oc0 / 16, q_cols >> 6);
+    if (in_bounds(args.status, off % 4 == 0 && off + 4 <= sc_bytes)) *reinterpret_cast<uint32_t*>(args.q_scales + off) = sc;
+  };
+  for (uint32_t r0 = 8 * warp; r0 < M; r0 += 32) {
+    const uint32_t row = r0 + (lane & 7);
+    float v[32], h[16];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 x = row < M ? *reinterpret_cast<const float4*>(part + skinny_part_offset(row, 8 * c + q))
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      v[4 * q] = x.x;
+      v[4 * q + 1] = x.y;
+      v[4 * q + 2] = x.z;
+      v[4 * q + 3] = x.w;
+    }
+    float amax = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float half_g = v[i] * (0.5f * scale), up = v[16 + i] * scale;
+      h[i] = fmaf(half_g, tanh_approx(half_g), half_g) * up;
+    }
+    if (args.q_mode == 2) {  // hadamard32, its last stage across the lanes
+#pragma unroll
+      for (int s = 1; s < 16; s <<= 1)
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if ((i & s) == 0) {
+            const float a = h[i], b = h[i + s];
+            h[i] = __fadd_rn(a, b);
+            h[i + s] = __fsub_rn(a, b);
+          }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float other = __shfl_xor_sync(0xffffffffu, h[i], 8);
+        h[i] = __fmul_rn(c & 1 ? __fsub_rn(other, h[i]) : __fadd_rn(h[i], other), __uint_as_float(kInvSqrt32Bits));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) amax = fmaxf(amax, fabsf(h[i]));
+    uint32_t code;
+    float mult;
+    if (args.q_mode == 0) {
+      const BlockScale bs = block_scale(amax, g, six_g);
+      code = g_ok ? bs.code : 0u;
+      mult = bs.mult;
+    } else {
+      code = mx_scale_code(fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 8)));
+      mult = mx_inv_scale(code);
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) h[i] = __fmul_rn(h[i], mult);
+    uint32_t sc = code << (8 * c);
+    sc |= __shfl_xor_sync(0xffffffffu, sc, 8);
+    sc |= __shfl_xor_sync(0xffffffffu, sc, 16);
+    const uint64_t off = static_cast<uint64_t>(row) * (q_cols / 2) + oc0 / 2 + 8 * c;
+    if (row < M && in_bounds(args.status, off + 8 <= code_bytes))
+      *reinterpret_cast<uint2*>(args.q_codes + off) = make_uint2(g_ok ? e2m1x8(h) : 0u, g_ok ? e2m1x8(h + 8) : 0u);
+    if (c == 0) store_scales(row, sc);
+  }
+  // Scales of the 128-row tile's further rows: those of zeros.
+  const uint32_t zero = args.q_mode == 0 ? (g_ok ? block_scale(0.0f, g, six_g).code : 0u) : mx_scale_code(0.0f);
+  for (uint32_t row = ((M + 7) & ~7u) + 32 * warp + lane; row < 128; row += 128) store_scales(row, zero * 0x01010101u);
+}
+
+// kSwiGLU: one CTA per tile (args.splits == 1).
+template <class C, bool kSwiGLU = false>
 __global__ void __launch_bounds__(C::kThreads, 2)
     nvfp4_gemm_skinny_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                              const GemmArgs args) {
@@ -1636,7 +1718,9 @@ __global__ void __launch_bounds__(C::kThreads, 2)
     const uint32_t part0 = smem_u32(smem);
     const uint32_t tid = threadIdx.x - 128;
     const int n0 = nb * 128;
-    switch (S) {
+    if constexpr (kSwiGLU) {
+      skinny_swiglu(smem, tid >> 5, tid & 31, nb, scale, args);
+    } else switch (S) {
       case 1: skinny_reduce<1>(part0, split, tid, n0, scale, args); break;
       case 2: skinny_reduce<2>(part0, split, tid, n0, scale, args); break;
       case 3: skinny_reduce<3>(part0, split, tid, n0, scale, args); break;
@@ -2316,7 +2400,7 @@ nvfp4_status launch_splitk(const uint8_t* a_codes, const uint8_t* a_scales, cons
 // of 512 columns each, and their shared memory fits).  Timing agrees: the
 // step from one wave to two lies at twice the query's figures (92 clusters of
 // 3, 72 of 4, 56 of 5, 46 of 6).
-template <class C>
+template <class C, bool kSwiGLU = false>
 int resident_skinny_clusters(int size) {
   static std::mutex mu;
   static std::map<std::pair<int, int>, int> cache;
@@ -2326,7 +2410,7 @@ int resident_skinny_clusters(int size) {
   auto it = cache.find({d, size});
   if (it != cache.end()) return it->second;
   int clusters = 0;
-  if (cudaFuncSetAttribute(nvfp4_gemm_skinny_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(nvfp4_gemm_skinny_kernel<C, kSwiGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(C::kSmemBytes)) == cudaSuccess) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -2340,8 +2424,8 @@ int resident_skinny_clusters(int size) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, nvfp4_gemm_skinny_kernel<C>, &cfg) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nvfp4_gemm_skinny_kernel<C>, C::kThreads,
+    if (cudaOccupancyMaxActiveClusters(&clusters, nvfp4_gemm_skinny_kernel<C, kSwiGLU>, &cfg) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nvfp4_gemm_skinny_kernel<C, kSwiGLU>, C::kThreads,
                                                       C::kSmemBytes) != cudaSuccess)
       clusters = 0;
     else if (per_sm == 1)
@@ -2384,14 +2468,16 @@ int choose_skinny_splits(int64_t tiles, int64_t kblocks) {
   return best;
 }
 
-template <class C>
+// kSwiGLU: out_bf16 is unused; the fused outputs go through *extra.
+template <class C, bool kSwiGLU = false>
 nvfp4_status launch_skinny(const uint8_t* a_codes, const uint8_t* a_scales, const float* g_a, const uint8_t* w_codes,
                            const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N, int64_t K, void* out_bf16,
-                           int64_t ldo, cudaStream_t stream, uint32_t idesc_fmt, int splits) {
+                           int64_t ldo, cudaStream_t stream, uint32_t idesc_fmt, int splits,
+                           const GemmArgs* extra = nullptr) {
   const int64_t tiles_n = (N + 127) / 128;
-  if (resident_skinny_clusters<C>(splits) <= 0) return NVFP4_ERR_CUDA;  // also the shared-memory opt-in
+  if (resident_skinny_clusters<C, kSwiGLU>(splits) <= 0) return NVFP4_ERR_CUDA;  // also the shared-memory opt-in
   if (tiles_n * splits >= (1ll << 31)) return NVFP4_ERR_SHAPE;
-  GemmArgs args = {};
+  GemmArgs args = kSwiGLU ? *extra : GemmArgs{};
   args.a_box_rows = static_cast<int>((M + 7) & ~7ll);
   CUtensorMap ma, mb;
   if (!make_code_map(&ma, a_codes, M, K, args.a_box_rows) || !make_code_map(&mb, w_codes, N, K, 128))
@@ -2423,7 +2509,7 @@ nvfp4_status launch_skinny(const uint8_t* a_codes, const uint8_t* a_scales, cons
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, nvfp4_gemm_skinny_kernel<C>, ma, mb, args) != cudaSuccess) return NVFP4_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, nvfp4_gemm_skinny_kernel<C, kSwiGLU>, ma, mb, args) != cudaSuccess) return NVFP4_ERR_CUDA;
   count_launches(1);
   return launch_status();
 }
@@ -2504,7 +2590,8 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
                         : M <= 64 ? launch_skinny<SkinnyCfg<64>>
                                   : launch_skinny<SkinnyCfg<128>>;
     if (splits)
-      return kernel(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, idesc_fmt, splits);
+      return kernel(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, idesc_fmt, splits,
+                    nullptr);
   }
   // The CTA pair, unless its 256 x 256 tiles would leave most pairs idle
   // (decode-sized M): then, with a long K, the split-K clusters, else 128 x
@@ -2537,6 +2624,26 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
   if (bn == 256)
     return launch<Cfg<256, 3>>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, idesc_fmt);
   return launch<Cfg<128, 5>>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, idesc_fmt);
+}
+
+// Kernel choice for the fused gate_up + SwiGLU (arguments already validated).
+// Up to 32 rows the skinny kernel, one CTA per 128 W rows: two CTAs share an
+// SM and only the A rows that exist are copied (us, pairs -> skinny, 1 row:
+// 27648 x 5120 27.5 -> 17.2, 17920 x 1536 9.8 -> 7.5, 12288 x 8192 23.6 ->
+// 15.4, 4096 x 2048 7.2 -> 6.3; 32 rows: 22.4 -> 17.2, 9.0 -> 7.3, 16.6 -> 15.4,
+// 6.6 -> 6.2; with 16 tiles, 2048 x 8192, level at 11.9).  K is not split: the
+// sums, and with them every output byte, are those of the pairs.  From 33 rows
+// on the larger A slots leave three ring stages, and the pairs are ahead for
+// some shapes (64 rows, 8192 x 4096: 9.6 against 10.5; 40960 x 5120: 28.8
+// against 32.5; 27648 x 5120: 20.3 against 18.3).
+nvfp4_status swiglu_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, const float* g_a,
+                             const uint8_t* w_codes, const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N,
+                             int64_t K, cudaStream_t s, const GemmArgs& extra, uint32_t idesc_fmt) {
+  if (M <= SkinnyCfg<32>::kRows)
+    return launch_skinny<SkinnyCfg<32>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, nullptr, 0, s,
+                                              idesc_fmt, 1, &extra);
+  return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K,
+                                                           nullptr, 0, s, &extra, idesc_fmt);
 }
 
 }  // namespace
@@ -2601,8 +2708,8 @@ NVFP4_API nvfp4_status nvfp4_linear_swiglu_quantize(const uint8_t* a_codes, cons
   extra.q_codes = out_codes;
   extra.q_scales = out_scales;
   extra.g_out = g_out;
-  return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, 2 * I,
-                                                           K, nullptr, 0, static_cast<cudaStream_t>(stream), &extra);
+  return swiglu_dispatch(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, 2 * I, K,
+                         static_cast<cudaStream_t>(stream), extra, 0);
 }
 
 NVFP4_API nvfp4_status mxfp4_linear_swiglu_quantize(const uint8_t* a_codes, const uint8_t* a_scales,
@@ -2621,9 +2728,8 @@ NVFP4_API nvfp4_status mxfp4_linear_swiglu_quantize(const uint8_t* a_codes, cons
   extra.q_codes = out_codes;
   extra.q_scales = out_scales;
   extra.q_mode = rotate ? 2u : 1u;
-  return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, nullptr, w_codes, w_scales, nullptr, M,
-                                                           2 * I, K, nullptr, 0, static_cast<cudaStream_t>(stream),
-                                                           &extra, kScaleE8M0);
+  return swiglu_dispatch(a_codes, a_scales, nullptr, w_codes, w_scales, nullptr, M, 2 * I, K,
+                         static_cast<cudaStream_t>(stream), extra, kScaleE8M0);
 }
 
 namespace nvfp4 {

@@ -307,6 +307,46 @@ def test_linear_swiglu_quantize_prefill_shape_then_down(N):
     assert_close(f32(out[torch.as_tensor(rows, device="cuda")]), ref, what="down(swiglu)")
 
 
+@pytest.mark.parametrize("M,I,K", [(1, 128, 256), (3, 20480, 512), (8, 256, 1280), (31, 384, 1024),
+                                   (32, 128, 4096), (33, 256, 768)])
+@pytest.mark.parametrize("fmt", ["nvfp4", "mxfp4", "mxfp4_rot"])
+def test_linear_swiglu_quantize_few_rows(N, M, I, K, fmt):
+    """Up to 32 rows run in a kernel of their own, with the same sums and the
+    same epilogue arithmetic as the CTA pairs: its codes and scales equal, byte
+    for byte, those that the pairs give these rows within a taller activation,
+    and the scales of its padding rows those of zeros."""
+    dev, tall = "cuda", 256
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(M + I + K)
+
+    def operand(rows):
+        lo, hi = (0x30, 0x40) if fmt == "nvfp4" else (122, 128)
+        return (torch.randint(0, 256, (rows, K // 2), dtype=torch.uint8, device=dev, generator=gen),
+                torch.randint(lo, hi, (N.nvfp4_scales_bytes(rows, K, 1),), dtype=torch.uint8, device=dev, generator=gen))
+
+    (a_c, a_s), (w_c, w_s) = operand(tall), operand(2 * I)
+    if fmt != "nvfp4":
+        # MXFP4 scales: a byte for each 16-element half of a 32-element block, both equal.
+        a_s[1::2], w_s[1::2] = a_s[::2], w_s[::2]
+    g, g_out = torch.full((1,), 0.05, device=dev), torch.full((1,), 1e-2, device=dev)
+
+    def run(rows):
+        out_c = torch.full((rows, I // 2), 0xEE, dtype=torch.uint8, device=dev)
+        out_s = torch.full((N.nvfp4_scales_bytes(rows, I, 1),), 0xEE, dtype=torch.uint8, device=dev)
+        if fmt == "nvfp4":
+            N.nvfp4_linear_swiglu_quantize(a_c, a_s, g, w_c, w_s, g, rows, I, K, g_out, out_c, out_s)
+        else:
+            N.mxfp4_linear_swiglu_quantize(a_c, a_s, w_c, w_s, rows, I, K, out_c, out_s, rotate=fmt == "mxfp4_rot")
+        torch.cuda.synchronize()
+        assert N.nvfp4_get_device_status() == 0
+        return u8(out_c), O.scales_from_mma(u8(out_s), max(rows, 128), I)
+
+    (codes, scales), (want_c, want_s) = run(M), run(tall)
+    assert (codes == want_c[:M]).all() and (scales[:M] == want_s[:M]).all()
+    assert len(np.unique(codes)) > 8
+    assert not scales[M:].any()
+
+
 def test_linear_swiglu_quantize_invalid_g_out_zeroes_and_reports(N):
     M, I, K = 256, 128, 256
     gen = torch.Generator().manual_seed(3)
