@@ -2631,15 +2631,18 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
 // SM and only the A rows that exist are copied (us, pairs -> skinny, 1 row:
 // 27648 x 5120 27.5 -> 17.2, 17920 x 1536 9.8 -> 7.5, 12288 x 8192 23.6 ->
 // 15.4, 4096 x 2048 7.2 -> 6.3; 32 rows: 22.4 -> 17.2, 9.0 -> 7.3, 16.6 -> 15.4,
-// 6.6 -> 6.2; with 16 tiles, 2048 x 8192, level at 11.9).  K is not split: the
-// sums, and with them every output byte, are those of the pairs.  From 33 rows
+// 6.6 -> 6.2).  K is not split: the sums, and with them every output byte, are
+// those of the pairs.  A few tiles with a long K leave each SM one CTA, whose
+// four ring stages stream slower than the pairs' five (2048 x 8192 12.3 against
+// 11.8, 4096 x 13824, 32 rows, 18.8 against 17.1; 2048 x 4096 7.7 against 7.9,
+// 4096 x 4096 8.4 against 8.9), so those stay with the pairs.  From 33 rows
 // on the larger A slots leave three ring stages, and the pairs are ahead for
 // some shapes (64 rows, 8192 x 4096: 9.6 against 10.5; 40960 x 5120: 28.8
 // against 32.5; 27648 x 5120: 20.3 against 18.3).
 nvfp4_status swiglu_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, const float* g_a,
                              const uint8_t* w_codes, const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N,
                              int64_t K, cudaStream_t s, const GemmArgs& extra, uint32_t idesc_fmt) {
-  if (M <= SkinnyCfg<32>::kRows)
+  if (M <= SkinnyCfg<32>::kRows && (K / BK <= 16 || N / 128 > 32))
     return launch_skinny<SkinnyCfg<32>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, nullptr, 0, s,
                                               idesc_fmt, 1, &extra);
   return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K,

@@ -308,7 +308,7 @@ def test_linear_swiglu_quantize_prefill_shape_then_down(N):
 
 
 @pytest.mark.parametrize("M,I,K", [(1, 128, 256), (3, 20480, 512), (8, 256, 1280), (31, 384, 1024),
-                                   (32, 128, 4096), (33, 256, 768)])
+                                   (32, 128, 4096), (5, 128, 4352), (33, 256, 768)])
 @pytest.mark.parametrize("fmt", ["nvfp4", "mxfp4", "mxfp4_rot"])
 def test_linear_swiglu_quantize_few_rows(N, M, I, K, fmt):
     """Up to 32 rows run in a kernel of their own, with the same sums and the
