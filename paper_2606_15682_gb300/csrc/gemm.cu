@@ -2626,25 +2626,40 @@ nvfp4_status linear_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, co
   return launch<Cfg<128, 5>>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, out_bf16, ldo, s, idesc_fmt);
 }
 
+// Whether the fused gate_up + SwiGLU runs in the skinny kernel, one CTA per 128
+// W rows: two CTAs share an SM and only the A rows that exist are copied.  K is
+// not split: the sums, and with them every output byte, are those of the
+// pairs.  us, pairs -> skinny:
+//   up to 32 rows: 1 row, 27648 x 5120 27.5 -> 17.2, 17920 x 1536 9.8 -> 7.5,
+//     12288 x 8192 23.6 -> 15.4, 4096 x 2048 7.2 -> 6.3; 32 rows: 22.4 -> 17.2,
+//     9.0 -> 7.3, 16.6 -> 15.4, 6.6 -> 6.2.  A few tiles with a long K leave
+//     each SM one CTA, whose ring streams slower than the pairs' (2048 x 8192
+//     12.3 against 11.8, 4096 x 13824, 32 rows, 18.8 against 17.1; 2048 x 4096
+//     7.7 against 7.9): those stay with the pairs;
+//   more rows, whose larger A slots leave three ring stages: ahead when all
+//     tiles are resident at once and some SMs hold two (48 rows: 27648 x 5120
+//     26.2 -> 18.2, 38912 x 1536 12.8 -> 9.9, 22528 x 8192 28.4 -> 23.6; 96 rows
+//     20.6 -> 19.3, 11.7 -> 10.7, 28.4 -> 24.3), and up to 64 rows with fewer
+//     tiles unless K is long (12288 x 5120 14.9 -> 12.7, 16384 x 1536 9.0 -> 7.9;
+//     12288 x 8192 17.0 -> 17.1, 8192 x 4096, 64 rows, 9.6 -> 10.5); not with a
+//     second wave (40960 x 5120, 64 rows, 28.8 -> 32.5).
+bool swiglu_in_skinny(int64_t M, int64_t tiles, int64_t kblocks) {
+  const int64_t sms = sm_count();
+  if (M <= 32) return kblocks <= 16 || tiles > 32;
+  if (M > 128 || tiles > 2 * sms) return false;
+  return tiles > sms || (M <= 64 && kblocks <= 20 && 8 * tiles >= 5 * sms);
+}
+
 // Kernel choice for the fused gate_up + SwiGLU (arguments already validated).
-// Up to 32 rows the skinny kernel, one CTA per 128 W rows: two CTAs share an
-// SM and only the A rows that exist are copied (us, pairs -> skinny, 1 row:
-// 27648 x 5120 27.5 -> 17.2, 17920 x 1536 9.8 -> 7.5, 12288 x 8192 23.6 ->
-// 15.4, 4096 x 2048 7.2 -> 6.3; 32 rows: 22.4 -> 17.2, 9.0 -> 7.3, 16.6 -> 15.4,
-// 6.6 -> 6.2).  K is not split: the sums, and with them every output byte, are
-// those of the pairs.  A few tiles with a long K leave each SM one CTA, whose
-// four ring stages stream slower than the pairs' five (2048 x 8192 12.3 against
-// 11.8, 4096 x 13824, 32 rows, 18.8 against 17.1; 2048 x 4096 7.7 against 7.9,
-// 4096 x 4096 8.4 against 8.9), so those stay with the pairs.  From 33 rows
-// on the larger A slots leave three ring stages, and the pairs are ahead for
-// some shapes (64 rows, 8192 x 4096: 9.6 against 10.5; 40960 x 5120: 28.8
-// against 32.5; 27648 x 5120: 20.3 against 18.3).
 nvfp4_status swiglu_dispatch(const uint8_t* a_codes, const uint8_t* a_scales, const float* g_a,
                              const uint8_t* w_codes, const uint8_t* w_scales, const float* g_w, int64_t M, int64_t N,
                              int64_t K, cudaStream_t s, const GemmArgs& extra, uint32_t idesc_fmt) {
-  if (M <= SkinnyCfg<32>::kRows && (K / BK <= 16 || N / 128 > 32))
-    return launch_skinny<SkinnyCfg<32>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, nullptr, 0, s,
-                                              idesc_fmt, 1, &extra);
+  if (swiglu_in_skinny(M, N / 128, K / BK)) {
+    const auto kernel = M <= 32   ? launch_skinny<SkinnyCfg<32>, true>
+                        : M <= 64 ? launch_skinny<SkinnyCfg<64>, true>
+                                  : launch_skinny<SkinnyCfg<128>, true>;
+    return kernel(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K, nullptr, 0, s, idesc_fmt, 1, &extra);
+  }
   return launch_pair<PairCfg<NVFP4_GEMM_PAIR_STAGES>, true>(a_codes, a_scales, g_a, w_codes, w_scales, g_w, M, N, K,
                                                            nullptr, 0, s, &extra, idesc_fmt);
 }

@@ -308,10 +308,11 @@ def test_linear_swiglu_quantize_prefill_shape_then_down(N):
 
 
 @pytest.mark.parametrize("M,I,K", [(1, 128, 256), (3, 20480, 512), (8, 256, 1280), (31, 384, 1024),
-                                   (32, 128, 4096), (5, 128, 4352), (33, 256, 768)])
+                                   (32, 128, 4096), (5, 128, 4352), (33, 256, 768), (33, 9856, 512), (64, 6144, 512),
+                                   (65, 9856, 256), (128, 10240, 512)])
 @pytest.mark.parametrize("fmt", ["nvfp4", "mxfp4", "mxfp4_rot"])
 def test_linear_swiglu_quantize_few_rows(N, M, I, K, fmt):
-    """Up to 32 rows run in a kernel of their own, with the same sums and the
+    """Up to 128 rows run in a kernel of their own for some shapes, with the same sums and the
     same epilogue arithmetic as the CTA pairs: its codes and scales equal, byte
     for byte, those that the pairs give these rows within a taller activation,
     and the scales of its padding rows those of zeros."""
