@@ -175,12 +175,17 @@ struct Params {
 
 // Which stages (128 cached tokens of one sequence and KV head) a CTA takes.
 // The stages of all sequences and heads, sequence-major, are one list of T;
-// CTA c takes stages c R .. c R + R - 1, so every CTA has the same work
+// CTA c takes units c R .. c R + R - 1, so every CTA has the same work
 // whatever the lengths.  A (sequence, head)'s s stages then lie with at most
 // (s - 2) / R + 2 CTAs in a row, each of which leaves one record of it; R is
 // at least what keeps that within the workspace's `records` per head.  Where
-// `whole` (room for one record only, or no head longer than a stage), a CTA
+// `whole` (room for one record only, or no head longer than three stages), a CTA
 // takes whole (sequence, head)s instead and no lengths need be summed.
+// A part of a head costs about as much as a stage beside its stages (merging
+// four warps, writing a record), so where a CTA takes several stages each head
+// counts one unit more, after its stages, and a run is R units: without it a
+// run of one-stage heads took several times as long as the others (64 x 40
+// heads of 1-3000 tokens 50 us).
 struct Segment {  // a run of stages of one (sequence, KV head)
   int b, kvh, record, t_begin, t_end;
   bool last;  // of its (sequence, head)
@@ -194,10 +199,13 @@ __device__ __forceinline__ uint32_t stages_of(int tokens) {
 }
 
 struct Walk {
-  uint32_t R;        // stages per CTA; 0: whole (sequence, head)s
-  uint32_t at, end;  // next stage and end of this CTA's run; or (sequence, head)s
-  uint32_t before;   // stages before sequence b
+  uint32_t R;        // units per CTA; 0: whole (sequence, head)s
+  uint32_t at, end;  // next unit and end of this CTA's run; or (sequence, head)s
+  uint32_t before;   // units before sequence b
+  uint32_t extra;    // units of a head beside its stages
   int b;
+
+  __device__ __forceinline__ uint32_t units_of(uint32_t stages) const { return stages ? stages + extra : 0u; }
 
   // By one converged warp.
   __device__ __forceinline__ void start(const Params& p) {
@@ -209,14 +217,22 @@ struct Walk {
     }
     const int lane = threadIdx.x & 31;
     const int per = (p.batch + 31) / 32, b0 = min(p.batch, lane * per), b1 = min(p.batch, b0 + per);
-    uint32_t sum = 0, most = 0;
-    for (int i = b0; i < b1; ++i) {
-      const uint32_t s = stages_of(cached_tokens(p, i));
-      sum += s;
-      most = max(most, s);
+    uint32_t sum = 0, most = 0, filled = 0;
+    for (int i = b0; i < b1; i += 4) {  // four lengths in flight per lane
+      uint32_t s[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[j] = i + j < b1 ? stages_of(cached_tokens(p, i + j)) : 0u;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        sum += s[j];
+        most = max(most, s[j]);
+        filled += s[j] != 0u;
+      }
     }
     most = __reduce_max_sync(0xffffffffu, most);
-    uint32_t incl = sum * p.hkv;  // stages up to this lane's last sequence
+    extra = __reduce_add_sync(0xffffffffu, sum) * p.hkv > gridDim.x ? 1u : 0u;
+    sum += extra * filled;
+    uint32_t incl = sum * p.hkv;  // units up to this lane's last sequence
 #pragma unroll
     for (int sh = 1; sh < 32; sh <<= 1) {
       const uint32_t v = __shfl_up_sync(0xffffffffu, incl, sh);
@@ -224,16 +240,18 @@ struct Walk {
     }
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
     R = max(1u, (total + gridDim.x - 1) / gridDim.x);
-    if (most > R && most <= R + 2) R = most;  // equal lengths: no run crosses a head
+    const uint32_t heads = static_cast<uint32_t>(p.batch) * p.hkv, whole = units_of(most);
+    // Equal lengths, a little longer than a run, of enough heads: no run crosses a head.
+    if (whole > R && whole <= R + 2 && whole * heads == total && 2 * heads >= gridDim.x) R = whole;
     if (most > 1) R = max(R, (most + p.records - 3) / (p.records - 1));
     at = min(blockIdx.x * R, total);
     end = min(at + R, total);
-    // The lane whose sequences hold the first stage looks for its sequence.
+    // The lane whose sequences hold the first unit looks for its sequence.
     uint32_t first = incl - sum * p.hkv;
     int found = p.batch;
     if (at >= first && at < incl) {
       for (found = b0; found < b1; ++found) {
-        const uint32_t n = stages_of(cached_tokens(p, found)) * p.hkv;
+        const uint32_t n = units_of(stages_of(cached_tokens(p, found))) * p.hkv;
         if (at < first + n) break;
         first += n;
       }
@@ -258,21 +276,23 @@ struct Walk {
     }
     while (at < end && b < p.batch) {
       const int len = cached_tokens(p, b);
-      const uint32_t n = stages_of(len);
-      if (at >= before + n * p.hkv) {
-        before += n * p.hkv;
+      const uint32_t n = stages_of(len), units = units_of(n);
+      if (at >= before + units * p.hkv) {
+        before += units * p.hkv;
         ++b;
         continue;
       }
       s->b = b;
-      s->kvh = static_cast<int>((at - before) / n);
-      const uint32_t first = before + s->kvh * n;  // the head's first stage
-      const uint32_t st = at - first, count = min(n - st, end - at);
+      s->kvh = static_cast<int>((at - before) / units);
+      const uint32_t first = before + s->kvh * units;  // the head's first stage
+      const uint32_t st = at - first, taken = min(units - st, end - at);
+      at += taken;
+      if (st >= n) continue;
+      const uint32_t count = min(n - st, taken);
       s->record = static_cast<int>(blockIdx.x - first / R);
       s->last = st + count == n;
       s->t_begin = static_cast<int>(st) * kStageTok;
       s->t_end = min(s->t_begin + static_cast<int>(count) * kStageTok, len);
-      at += count;
       return true;
     }
     return false;
@@ -851,7 +871,7 @@ nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, i
   const int ctas_max = resident_ctas(cache);
   if (ctas_max <= 0) return NVFP4_ERR_CUDA;
   const int64_t stages = (cache->capacity + kStageTok - 1) / kStageTok;
-  const int64_t items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * stages;
+  const int64_t heads = static_cast<int64_t>(cache->batch) * cache->num_kv_heads;
   const int64_t fit = static_cast<int64_t>(partials_bytes / (kRecordBytes * cache->batch * num_q_heads));
   prm->k_codes = cache->k_codes;
   prm->k_scales = cache->k_scales;
@@ -868,7 +888,10 @@ nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, i
   // Never more than asked for, so that a larger workspace changes no result.
   const int64_t want = preferred_records(cache->batch, num_q_heads, cache->capacity);
   prm->records = static_cast<int>(fit < want ? fit : want);
-  prm->whole = stages <= 1 || prm->records < 2;
+  // Up to three stages a head's own work is shorter than what finding and
+  // merging a run's parts costs (us, whole / runs: 1 x 40 heads, 154 tokens 5.9
+  // / 7.0, 384 7.2 / 8.1, 512 8.1 / 6.2; 64 x 40: 10.2 / 11.3, 14.5 / 15.7).
+  prm->whole = stages <= 3 || (stages <= 8 && 2 * heads >= ctas_max) || prm->records < 2;
   if (prm->whole) prm->records = 1;
   prm->logit_mult = softmax_scale * cache->k_gscale * kLog2e;
   prm->fault_skip_stage = take_fault(NVFP4_FAULT_ATTN_SKIP_STAGE) ? 1 : 0;
@@ -876,17 +899,19 @@ nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, i
   // the same call, so nothing left from an earlier call needs clearing.
   prm->o_ws = partials;
   prm->ml_ws = prm->o_ws + static_cast<size_t>(cache->batch) * num_q_heads * prm->records * kD;
-  *grid = static_cast<int>(items < ctas_max ? items : ctas_max);
+  const int64_t ctas = prm->whole ? heads : heads * stages;
+  *grid = static_cast<int>(ctas < ctas_max ? ctas : ctas_max);
   return NVFP4_OK;
 }
 
 // The partial and the combine kernel.  With few heads of many records the
 // combine's blocks take 8 x 128 threads (1 x 40 heads of 64 records: 4.3 ->
-// 3.0 us); with many heads more threads per head would only crowd the SMs.
+// 3.0 us); with more heads than SMs they would only crowd each other (both
+// kernels, 8 x 32 heads of 8-9 records: 13.2 against 15.4 us).
 template <bool kQuant>
 nvfp4_status attention_launch(const nvfp4_kv_cache* cache, const Params& prm, int grid, const CombineOut& out,
                               cudaStream_t s) {
-  const bool wide = prm.records > 8 && static_cast<int64_t>(prm.hq) * prm.batch <= 2 * sm_count();
+  const bool wide = prm.records > 8 && static_cast<int64_t>(prm.hq) * prm.batch <= sm_count();
   if (launch_pdl(partial_kernel(cache), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
       launch_pdl(wide ? attn_combine_kernel<kQuant, 8> : attn_combine_kernel<kQuant, 1>, dim3(prm.hq, prm.batch),
                  dim3(wide ? 8 * kD : kD), 0, s, static_cast<const float*>(prm.o_ws),

@@ -533,7 +533,10 @@ def test_injected_missing_stage_times_out_and_device_stays_usable(N):
     (8, 1, 6144, [6143, 300], 1),                              # one long sequence beside a short one
     (8, 8, 512, [512] * 40, 0),                                # more heads than a run: several heads per CTA
     (6, 2, 126, [126, 5, 64], 0),                              # at most one stage per head
-    (5, 1, 1536, [(37 * i) % 1537 for i in range(70)], 0)])    # 70 sequences of all lengths
+    (5, 1, 1536, [(37 * i) % 1537 for i in range(70)], 0),     # 70 sequences of all lengths
+    (8, 8, 1400, [1400, 3, 128, 1, 90, 0, 1400, 129] * 6, 1),  # runs of one-stage heads beside long ones
+    (8, 8, 2048, [1100] * 40, 0),                              # equal, a little longer than a run
+    (16, 8, 1024, [1024, 7, 500, 0] * 12, 0)])                 # whole heads: many of up to eight stages
 @pytest.mark.parametrize("least", [False, True])
 def test_decode_attention_runs_over_ragged_lengths(N, hq, hkv, cap, lens, fmt, least):
     """Equal runs of stages over ragged caches, with the asked-for workspace
