@@ -391,10 +391,10 @@ nvfp4_status nvfp4_rope_table(float* table, int64_t n_pos, int32_t head_dim, flo
  * writes out.
  *   q_bf16   : [batch, num_q_heads, head_dim] bf16.
  *   out_bf16 : [batch, num_q_heads, head_dim] bf16.
- *   workspace: decode_attention_nvfp4_workspace_size(...) bytes, 16-B aligned;
- *              contents on entry are ignored.  Less is accepted down to one
- *              record (520 bytes) per query head and 1024 tokens of capacity,
- *              at the cost of a coarser split; more changes nothing.
+ *   workspace: at least decode_attention_nvfp4_workspace_size(...) bytes, 16-B
+ *              aligned; contents on entry are ignored.
+ * A sequence's result depends on its own cache, length and query alone, bit for
+ * bit: not on the other sequences, the capacity or the workspace's size.
  * num_q_heads % num_kv_heads == 0, num_q_heads/num_kv_heads <= 8 and an even
  * capacity (scale rows are streamed in 16-byte units) are required (SHAPE);
  * the four cache arrays must be 16-B aligned (ALIGN).
@@ -441,8 +441,8 @@ nvfp4_status decode_attention_nvfp4_quantize(const nvfp4_kv_cache* cache, const 
  *
  * Limits and sharing:
  *   - The scratch holds NVFP4_ATTN_STATIC_SCRATCH_BYTES (24 MiB); a problem
- *     whose smallest workspace (above) exceeds it returns SHAPE without
- *     launching anything.  Every GPU that loads the library keeps
+ *     whose decode_attention_nvfp4_workspace_size exceeds it returns SHAPE
+ *     without launching anything.  Every GPU that loads the library keeps
  *     this array until the process exits.
  *   - All calls share the one array and it keeps the last call's contents;
  *     every value a call reads is written earlier in the same call, so no

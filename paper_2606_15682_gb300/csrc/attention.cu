@@ -1,12 +1,14 @@
 // a5: decode attention straight from the NVFP4 KV cache (Sec. 2.1:
 // z = softmax(Q K_hat^T / sqrt(d)) V_hat with quantized K and V).
 //
-// Split-KV ("flash-decoding").  The cached tokens of all sequences and KV heads
-// are one list of 128-token stages, cut into equal runs, one per resident CTA
-// (struct Walk).  Each CTA has a producer warp that streams its run's FP4 K/V
-// codes and E4M3 scales into a 2-stage ring with 1-D bulk copies, and
-// four consumer warps that each take two 16-token tiles of every stage (one
-// barrier hand-off per two tiles; measured faster than 4 x 64-token stages).  A consumer
+// Split-KV ("flash-decoding").  A work item is one (sequence, KV head,
+// 1024-token chunk), so that a sequence's result depends on nothing but its own
+// cache and query; persistent CTAs share the items out (struct Walk).  Each CTA
+// has a producer warp that streams the items' FP4 K/V codes and E4M3 scales into
+// a 2-stage ring of 128-token stages with 1-D bulk copies (the ring runs on
+// across items), and four consumer warps that each take two 16-token tiles of
+// every stage (one barrier hand-off per two tiles; measured faster than 4 x
+// 64-token stages).  A consumer
 // dequantizes in registers (cvt e2m1x2 -> f16x2, times the E4M3 block scale:
 // exact in f16) and runs mma.sync m16n8k16 with fp32 accumulation:
 //   S^T[16 tok x 8 head] = K_hat[16 tok x 128] . Q^T[128 x 8]   (8 MMAs)
@@ -14,8 +16,8 @@
 // The up to 8 query heads that share a KV head (grouped-query attention) fill
 // the MMA's N = 8.  Softmax is online, in fp32, in the log2 domain, with lazy
 // rescaling (the running max moves only when a tile exceeds it by 2^8).  At
-// the end of a (sequence, head) or of the run the four warps merge their
-// partial (max, sum, O) and write one record; a combine kernel merges them.
+// the end of an item the four warps merge their partial (max, sum, O) and
+// write one record; a combine kernel merges the records of a head's chunks.
 //
 // Lane roles (g = lane/4, t = lane%4), fixed by the m16n8k16 fragment layouts:
 //   K: rows g and g+8 of the S tile, channels 32t..32t+31 (16 bytes, blocks 2t, 2t+1)
@@ -38,8 +40,8 @@ namespace nvfp4 {
 namespace {
 
 constexpr int kD = 128;
-constexpr int kStageTok = 128;        // tokens per ring stage: the unit of work
-constexpr int kChunk = 1024;          // the workspace holds at least one record per 1024 tokens and head
+constexpr int kChunk = 1024;          // tokens per work item
+constexpr int kStageTok = 128;        // tokens per ring stage
 #ifndef NVFP4_ATTN_STAGES
 #define NVFP4_ATTN_STAGES 2
 #endif
@@ -47,10 +49,10 @@ constexpr int kChunk = 1024;          // the workspace holds at least one record
 #define NVFP4_ATTN_MIN_CTAS 4
 #endif
 constexpr int kStages = NVFP4_ATTN_STAGES;  // 2 x 18 KiB ring + merge buffer: 4 CTAs per SM
-constexpr int kConsumers = 4;         // consumer warps, 16 tokens of a stage each
+constexpr int kConsumers = 4;         // consumer warps, two 16-token tiles of a stage each
 constexpr int kThreads = 32 * (1 + kConsumers);
 constexpr uint32_t kStageBytes = kStageTok * (64 + 8) * 2;  // K, V codes + scales: 18 KiB
-static_assert(kStageTok % (16 * kConsumers) == 0, "stage tiling");
+static_assert(kChunk % kStageTok == 0 && kStageTok % (16 * kConsumers) == 0, "stage tiling");
 constexpr uint32_t kOffKc = 0, kOffVc = kStageTok * 64, kOffKs = 2 * kStageTok * 64, kOffVs = kOffKs + kStageTok * 8;
 // Merge buffer: a head's channels with 2 floats of padding per 16, and heads
 // 148 floats apart, so that a half-warp's 8-byte stores (4 channel groups, 4
@@ -168,139 +170,105 @@ struct Params {
   float* o_ws;
   float* ml_ws;
   int* status;
-  int batch, hkv, capacity, hq, group, records, whole;
+  int batch, hkv, capacity, hq, group, n_splits, n_items;
   float logit_mult;  // softmax_scale * g_K * log2(e)
   int fault_skip_stage;  // test-only: CTA 0's producer leaves its first stage unissued
 };
 
-// Which stages (128 cached tokens of one sequence and KV head) a CTA takes.
-// The stages of all sequences and heads, sequence-major, are one list of T;
-// CTA c takes units c R .. c R + R - 1, so every CTA has the same work
-// whatever the lengths.  A (sequence, head)'s s stages then lie with at most
-// (s - 2) / R + 2 CTAs in a row, each of which leaves one record of it; R is
-// at least what keeps that within the workspace's `records` per head.  Where
-// `whole` (room for one record only, or no head longer than three stages), a CTA
-// takes whole (sequence, head)s instead and no lengths need be summed.
-// A part of a head costs about as much as a stage beside its stages (merging
-// four warps, writing a record), so where a CTA takes several stages each head
-// counts one unit more, after its stages, and a run is R units: without it a
-// run of one-stage heads took several times as long as the others (64 x 40
-// heads of 1-3000 tokens 50 us).
-struct Segment {  // a run of stages of one (sequence, KV head)
-  int b, kvh, record, t_begin, t_end;
-  bool last;  // of its (sequence, head)
+struct Item {
+  int b, kvh, split, t_begin, t_end;
 };
+constexpr int kItems = kStages + 2;  // places of items between the producer and the consumers
 
-__device__ __forceinline__ int cached_tokens(const Params& p, int b) {
-  return max(0, min(__ldg(p.seq_lens + b), p.capacity));
+__device__ __forceinline__ int cached_tokens(const int32_t* __restrict__ seq_lens, int b, int capacity) {
+  return max(0, min(__ldg(seq_lens + b), capacity));
 }
-__device__ __forceinline__ uint32_t stages_of(int tokens) {
-  return static_cast<uint32_t>(tokens + kStageTok - 1) / kStageTok;
+__device__ __forceinline__ uint32_t chunks_of(int tokens) {
+  return (static_cast<uint32_t>(tokens) + kChunk - 1) / kChunk;
 }
 
+// Which items a CTA takes where a head has several chunks and the CTAs cannot
+// each have one: of the list of all chunks that hold tokens, the full ones
+// first (sequence-major), then the sequences' ends, items blockIdx.x, blockIdx.x
+// + gridDim.x, ...  Chunks past a sequence's length cost nothing, CTAs take the
+// same number of full chunks but for one, and the short ones fill in behind
+// them.  Only the producer warp walks (each lane holds one sequence of a window
+// of 32), once an item's loads are issued; the consumers get the item from it
+// through shared memory.  (Walked by every warp, an item cost 1 us more.)  GB300,
+// 40 heads on 8 KV heads, against the capacity's chunks in turn: 64 sequences of
+// 2000-16384 tokens 208 -> 146 us, 32 of 512-4096 39.1 -> 32.4, 64 of 3000 56.5 ->
+// 53.9; 64 of 16384, where both orders are the same, 235.7 -> 237.7.
 struct Walk {
-  uint32_t R;        // units per CTA; 0: whole (sequence, head)s
-  uint32_t at, end;  // next unit and end of this CTA's run; or (sequence, head)s
-  uint32_t before;   // units before sequence b
-  uint32_t extra;    // units of a head beside its stages
-  int b;
+  uint32_t at;      // this CTA's next item
+  uint32_t before;  // items before the window
+  uint32_t incl;    // the window's items up to this lane's sequence
+  int base, len;    // first sequence of the window, tokens of this lane's
+  bool ends;        // full chunks, or the sequences' ends
 
-  __device__ __forceinline__ uint32_t units_of(uint32_t stages) const { return stages ? stages + extra : 0u; }
-
-  // By one converged warp.
-  __device__ __forceinline__ void start(const Params& p) {
-    if (p.whole) {
-      R = 0;
-      at = blockIdx.x;
-      end = static_cast<uint32_t>(p.batch) * p.hkv;
-      return;
-    }
-    const int lane = threadIdx.x & 31;
-    const int per = (p.batch + 31) / 32, b0 = min(p.batch, lane * per), b1 = min(p.batch, b0 + per);
-    uint32_t sum = 0, most = 0, filled = 0;
-    for (int i = b0; i < b1; i += 4) {  // four lengths in flight per lane
-      uint32_t s[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[j] = i + j < b1 ? stages_of(cached_tokens(p, i + j)) : 0u;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        sum += s[j];
-        most = max(most, s[j]);
-        filled += s[j] != 0u;
-      }
-    }
-    most = __reduce_max_sync(0xffffffffu, most);
-    extra = __reduce_add_sync(0xffffffffu, sum) * p.hkv > gridDim.x ? 1u : 0u;
-    sum += extra * filled;
-    uint32_t incl = sum * p.hkv;  // units up to this lane's last sequence
+  // By a converged warp.
+  __device__ __forceinline__ void window(const Params& p, int first) {
+    base = first;
+    const int b = base + (threadIdx.x & 31);
+    len = b < p.batch ? cached_tokens(p.seq_lens, b, p.capacity) : 0;
+    incl = (ends ? (len % kChunk != 0 ? 1u : 0u) : static_cast<uint32_t>(len) / kChunk) * p.hkv;
 #pragma unroll
     for (int sh = 1; sh < 32; sh <<= 1) {
       const uint32_t v = __shfl_up_sync(0xffffffffu, incl, sh);
-      if (lane >= sh) incl += v;
+      if ((threadIdx.x & 31) >= sh) incl += v;
     }
-    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-    R = max(1u, (total + gridDim.x - 1) / gridDim.x);
-    const uint32_t heads = static_cast<uint32_t>(p.batch) * p.hkv, whole = units_of(most);
-    // Equal lengths, a little longer than a run, of enough heads: no run crosses a head.
-    if (whole > R && whole <= R + 2 && whole * heads == total && 2 * heads >= gridDim.x) R = whole;
-    if (most > 1) R = max(R, (most + p.records - 3) / (p.records - 1));
-    at = min(blockIdx.x * R, total);
-    end = min(at + R, total);
-    // The lane whose sequences hold the first unit looks for its sequence.
-    uint32_t first = incl - sum * p.hkv;
-    int found = p.batch;
-    if (at >= first && at < incl) {
-      for (found = b0; found < b1; ++found) {
-        const uint32_t n = units_of(stages_of(cached_tokens(p, found))) * p.hkv;
-        if (at < first + n) break;
-        first += n;
-      }
-    }
-    const uint32_t owner = __ballot_sync(0xffffffffu, found < p.batch);
-    const int src = owner ? __ffs(owner) - 1 : 0;
-    b = __shfl_sync(0xffffffffu, found, src);
-    before = __shfl_sync(0xffffffffu, first, src);
   }
-
-  __device__ __forceinline__ bool next(const Params& p, Segment* s) {
-    if (R == 0) {
-      if (at >= end) return false;
-      s->b = static_cast<int>(at) / p.hkv;
-      s->kvh = static_cast<int>(at) - s->b * p.hkv;
-      s->record = 0;
-      s->last = true;
-      s->t_begin = 0;
-      s->t_end = cached_tokens(p, s->b);
-      at += gridDim.x;
-      return true;
-    }
-    while (at < end && b < p.batch) {
-      const int len = cached_tokens(p, b);
-      const uint32_t n = stages_of(len), units = units_of(n);
-      if (at >= before + units * p.hkv) {
-        before += units * p.hkv;
-        ++b;
-        continue;
+  __device__ __forceinline__ void start(const Params& p) {
+    at = blockIdx.x;
+    before = 0;
+    ends = p.capacity < kChunk;  // then there are no others
+    window(p, 0);
+  }
+  __device__ __forceinline__ bool next(const Params& p, Item* it) {
+    for (;;) {
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+      if (at - before < total) break;
+      before += total;
+      if (base + 32 < p.batch) {
+        window(p, base + 32);
+      } else {
+        if (ends) return false;
+        ends = true;
+        window(p, 0);
       }
-      s->b = b;
-      s->kvh = static_cast<int>((at - before) / units);
-      const uint32_t first = before + s->kvh * units;  // the head's first stage
-      const uint32_t st = at - first, taken = min(units - st, end - at);
-      at += taken;
-      if (st >= n) continue;
-      const uint32_t count = min(n - st, taken);
-      s->record = static_cast<int>(blockIdx.x - first / R);
-      s->last = st + count == n;
-      s->t_begin = static_cast<int>(st) * kStageTok;
-      s->t_end = min(s->t_begin + static_cast<int>(count) * kStageTok, len);
-      return true;
     }
-    return false;
+    const int lane = __ffs(__ballot_sync(0xffffffffu, at - before < incl)) - 1;
+    const uint32_t skipped = __shfl_sync(0xffffffffu, incl, lane ? lane - 1 : 0);
+    const uint32_t i = at - before - (lane ? skipped : 0u);  // within the sequence
+    const int tokens = __shfl_sync(0xffffffffu, len, lane);
+    const int full = tokens / kChunk;
+    it->b = base + lane;
+    it->kvh = static_cast<int>(ends ? i : i / full);
+    it->split = ends ? full : static_cast<int>(i) - it->kvh * full;
+    it->t_begin = it->split * kChunk;
+    it->t_end = min(it->t_begin + kChunk, tokens);
+    at += gridDim.x;
+    return true;
   }
 };
 
+// Item i of all chunks of the capacity; empty past the sequence's length.
+__device__ __forceinline__ Item capacity_item(const Params& p, int i) {
+  Item it;
+  const int rest = i / p.n_splits;
+  it.split = i - rest * p.n_splits;
+  it.b = rest / p.hkv;
+  it.kvh = rest - it.b * p.hkv;
+  it.t_begin = it.split * kChunk;
+  it.t_end = min(it.t_begin + kChunk, cached_tokens(p.seq_lens, it.b, p.capacity));
+  return it;
+}
+
 // kE1M2: the cache holds E1M2 elements (decoded to n, the scale carries 1/2).
-template <bool kE1M2>
+// kListed: CTAs take the items of the list (struct Walk); else items blockIdx.x,
+// blockIdx.x + gridDim.x, ... of the capacity, which each warp finds by itself,
+// so that the query's load waits for nothing (1 x 32 heads of 2048 tokens 11.9 us
+// against 12.6).
+template <bool kE1M2, bool kListed>
 __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_kernel(const Params p) {
   extern __shared__ __align__(128) uint8_t smem[];
   uint8_t* ring = smem;
@@ -309,6 +277,8 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
   float* sh_l = sh_m + kConsumers * 8;
   uint64_t* full = reinterpret_cast<uint64_t*>(sh_l + kConsumers * 8);
   uint64_t* empty = full + kStages;
+  uint64_t* listed = empty + kStages;  // an item's place in `items` is written
+  __shared__ Item items[kItems];
   __shared__ volatile int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -317,6 +287,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], kConsumers);
     }
+    for (int i = 0; i < kItems; ++i) mbar_init(&listed[i], 1);
     abort_flag = 0;
     fence_mbar_init();
   }
@@ -326,19 +297,36 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
     for (int b = threadIdx.x; b < p.batch; b += kThreads)
       if (__ldg(p.seq_lens + b) > p.capacity) set_status(p.status, NVFP4_ERR_CAPACITY);
 
-  Walk walk;
-  walk.start(p);
-  Segment it;
   if (warp == 0) {
     // ------------------------------------------------------------ producer ---
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t issued_parity[kStages];
-      bool issued[kStages];
-      for (int s = 0; s < kStages; ++s) issued[s] = false;
-      bool skip_stage = p.fault_skip_stage && blockIdx.x == 0;
-      while (!abort_flag && walk.next(p, &it)) {
+    // The warp goes over the items together; lane 0 issues.
+    int stage = 0;
+    uint32_t phase = 0;
+    uint32_t issued_parity[kStages];
+    bool issued[kStages];
+    for (int s = 0; s < kStages; ++s) issued[s] = false;
+    bool skip_stage = p.fault_skip_stage && blockIdx.x == 0;
+    Walk walk;
+    Item it;
+    if (kListed) walk.start(p);
+    for (uint32_t j = 0; __all_sync(0xffffffffu, !abort_flag); ++j) {
+      if (kListed) {
+        const bool more = walk.next(p, &it);
+        // Place j % kItems is free: at most the last kStages stages issued are
+        // not consumed yet, and they belong to items j - kStages and later, so
+        // item j - kItems has been read by every consumer warp.
+        if (lane == 0) {
+          if (!more) it.b = -1;  // no further item
+          items[j % kItems] = it;
+          mbar_arrive(&listed[j % kItems]);
+        }
+        if (!more) break;
+      } else {
+        const int64_t i = blockIdx.x + static_cast<int64_t>(j) * gridDim.x;
+        if (i >= p.n_items) break;
+        it = capacity_item(p, static_cast<int>(i));
+      }
+      if (lane == 0) {
         const size_t row0 = (static_cast<size_t>(it.b) * p.hkv + it.kvh) * p.capacity;
         for (int t0 = it.t_begin; t0 < it.t_end; t0 += kStageTok) {
           const int n = min(kStageTok, it.t_end - t0);
@@ -367,10 +355,11 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
-      if (abort_flag)
-        for (int s = 0; s < kStages; ++s)
-          if (issued[s]) mbar_wait_bounded(&full[s], issued_parity[s], nullptr);
+      __syncwarp();
     }
+    if (lane == 0 && abort_flag)
+      for (int s = 0; s < kStages; ++s)
+        if (issued[s]) mbar_wait_bounded(&full[s], issued_parity[s], nullptr);
     return;
   }
 
@@ -381,17 +370,24 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
   const int rv[4] = {tile_tok(2 * t), tile_tok(2 * t + 1), tile_tok(2 * t + 8), tile_tok(2 * t + 9)};  // V rows
   int stage = 0;
   uint32_t phase = 0;
-  if (blockIdx.x == 0) {  // sequences without tokens have no segment
-    for (int b = threadIdx.x - 32; b < p.batch; b += 32 * kConsumers) {
-      if (__ldg(p.seq_lens + b) > 0) continue;
-      float* ml = p.ml_ws + static_cast<size_t>(b) * p.hq * p.records * 2;
-      for (int i = 0; i < p.hq * p.records; ++i) {
-        ml[2 * i] = -INFINITY;
-        ml[2 * i + 1] = 0.0f;
+  int item = blockIdx.x;
+  for (uint32_t j = 0; kListed || item < p.n_items; ++j) {
+    Item it;
+    if (kListed) {
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&listed[j % kItems], (j / kItems) & 1u, &abort_flag))) {
+        if (lane == 0 && !abort_flag) {
+          set_status(p.status, NVFP4_ERR_TIMEOUT);
+          abort_flag = 1;
+        }
+        return;
       }
+      it = items[j % kItems];
+      if (it.b < 0) return;
+    } else {
+      it = capacity_item(p, item);
+      item += gridDim.x;
+      if (it.t_begin >= it.t_end) continue;
     }
-  }
-  while (walk.next(p, &it)) {
     // Queries of head slot g: f16 after an exact power-of-two scaling that
     // keeps |q| < 1; the scaling is undone in the logit multiplier.
     const bool head_live = g < p.group;
@@ -456,7 +452,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       for (int sub = 0; sub < kStageTok / (16 * kConsumers); ++sub) {
       const int r0 = 16 * (cw + kConsumers * sub);  // this warp's tile within the stage
       const int tile = t0 + r0;
-      const int valid = it.t_end - tile;  // tokens of this warp's tile inside the segment (may be <= 0)
+      const int valid = it.t_end - tile;  // tokens of this warp's tile inside the item (may be <= 0)
       if (valid > 0) {
         // ---- S^T = K_hat Q^T: 8 k-steps of 16 channels ---------------------
         const uint4 ka = *reinterpret_cast<const uint4*>(st + kOffKc + (r0 + rk0) * 64 + 16 * t);
@@ -494,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
           vs01_raw = s0 | (s1 << 8);
           vs89_raw = s2 | (s3 << 8);
         }
-        if (valid < 16) {  // ragged end of the segment: mask keys, zero the scales of absent values
+        if (valid < 16) {  // ragged end of the item: mask keys, zero the scales of absent values
           if (rk0 >= valid) x0 = x1 = -INFINITY;
           if (rk1 >= valid) x2 = x3 = -INFINITY;
           if (rv[0] >= valid) vs01_raw &= 0xFF00u;
@@ -577,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
     }
 
-    // ---- merge the consumer warps, write this segment's record ------------
+    // ---- merge the consumer warps, write this item's record ---------------
     l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 4);
     l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 4);
     l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 8);
@@ -610,23 +606,14 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
           L += wt * sh_l[w * 8 + h];
         }
       }
-      const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.records + it.record;
+      const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.n_splits + it.split;
       p.o_ws[rec * kD + c] = acc;
       if (c == 0) {
         p.ml_ws[rec * 2] = M;
         p.ml_ws[rec * 2 + 1] = L;
       }
     }
-    if (it.last) {  // the records of this head that no segment leaves
-      const int rest = p.records - it.record - 1;
-      for (int i = threadIdx.x - 32; i < rest * p.group; i += 32 * kConsumers) {
-        const int h = i / rest;
-        const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.records + it.record + 1 + i - h * rest;
-        p.ml_ws[rec * 2] = -INFINITY;
-        p.ml_ws[rec * 2 + 1] = 0.0f;
-      }
-    }
-    named_barrier_consumers();  // the merge buffer is rewritten by the next segment
+    named_barrier_consumers();  // the merge buffer is rewritten by the next item
   }
 }
 
@@ -646,87 +633,49 @@ struct CombineOut {
   uint32_t kgroups;
 };
 
-// One block per head, kD threads times kGroups.  A head's records come first
-// in its slots; the others hold (-inf, 0) and an undefined O that is not used.
-// The weights are formed one record per thread, then the records are added,
-// one channel per thread; kGroups = 8 (few heads with many records) lets each
-// group take every eighth one.  The first records' O is loaded beside the
-// weights' inputs: usually that is all there is.
-template <bool kQuant, int kGroups>
-__global__ void __launch_bounds__(kD* kGroups) attn_combine_kernel(const float* __restrict__ o_ws,
-                                                                   const float* __restrict__ ml_ws, int records,
-                                                                   float gv, const CombineOut out) {
-  constexpr int kT = kD * kGroups, kAhead = kGroups > 1 ? 8 : 4;
-  __shared__ float sh_w[kT], sh_acc[kGroups][kD];
-  __shared__ float2 sh_red[kT / 32];
-  __shared__ int sh_used[kT / 32];
+// One block per head, one channel per thread; records of chunks without tokens
+// are not written and not used.  A lane forms the weight of one record of 32;
+// the warp then adds them in chunk order, kDepth loads of O in flight (32 for few
+// heads of many records, whose time is these loads' latency).
+template <bool kQuant, int kDepth>
+__global__ void __launch_bounds__(kD) attn_combine_kernel(const float* __restrict__ o_ws,
+                                                         const float* __restrict__ ml_ws,
+                                                         const int32_t* __restrict__ seq_lens, int capacity,
+                                                         int n_splits, float gv, const CombineOut out) {
   griddep_wait_and_release();
   const size_t bh = static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = threadIdx.x % kD, group = threadIdx.x / kD;
-  const float2* ml = reinterpret_cast<const float2*>(ml_ws) + bh * records;
-  const float* o = o_ws + bh * records * kD + c;
-  const float2 own = static_cast<int>(threadIdx.x) < records ? __ldg(ml + threadIdx.x) : make_float2(-INFINITY, 0.0f);
-  float ahead[kAhead];
+  const int lane = threadIdx.x & 31, c = threadIdx.x;
+  const float2* ml = reinterpret_cast<const float2*>(ml_ws) + bh * n_splits;
+  const float* o = o_ws + bh * n_splits * kD + c;
+  float2 rec = lane < n_splits ? __ldg(ml + lane) : make_float2(-INFINITY, 0.0f);
+  const int used = static_cast<int>(chunks_of(cached_tokens(seq_lens, blockIdx.y, capacity)));
+  float M = lane < used ? rec.x : -INFINITY;
+  for (int i = lane + 32; i < used; i += 32) M = fmaxf(M, __ldg(ml + i).x);
 #pragma unroll
-  for (int k = 0; k < kAhead; ++k) {
-    const int i = group + k * kGroups;
-    ahead[k] = i < records ? __ldg(o + static_cast<size_t>(i) * kD) : 0.0f;
-  }
-  float m = own.x;
-  int used = own.x != -INFINITY ? static_cast<int>(threadIdx.x) + 1 : 0;  // the records in use come first
-  for (int i = threadIdx.x + kT; i < records; i += kT) {
-    const float x = __ldg(ml + i).x;
-    m = fmaxf(m, x);
-    if (x != -INFINITY) used = i + 1;
-  }
-  used = __reduce_max_sync(0xffffffffu, used);
-#pragma unroll
-  for (int sh = 16; sh; sh >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, sh));
-  if (lane == 0) {
-    sh_red[warp].x = m;
-    sh_used[warp] = used;
-  }
-  __syncthreads();
-  float M = sh_red[0].x;
-  used = sh_used[0];
-#pragma unroll
-  for (int w = 1; w < kT / 32; ++w) {
-    M = fmaxf(M, sh_red[w].x);
-    used = max(used, sh_used[w]);
-  }
-  float acc = 0.0f, l = 0.0f;
-  for (int i0 = 0; i0 < used; i0 += kT) {
-    const int i = i0 + threadIdx.x;
+  for (int sh = 16; sh; sh >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, sh));
+  float acc = 0.0f, L = 0.0f;
+  if (M != -INFINITY) {
     float w = 0.0f;
-    if (i < used) {
-      const float2 x = i0 == 0 ? own : __ldg(ml + i);
-      w = fast_exp2(x.x - M);
-      l += w * x.y;
-    }
-    sh_w[threadIdx.x] = w;
-    __syncthreads();
-    const int count = min(kT, used - i0);
-    if (i0 == 0) {
+    for (int i0 = 0; i0 < used; i0 += kDepth) {
+      float v[kDepth];
 #pragma unroll
-      for (int k = 0; k < kAhead; ++k)
-        if (group + k * kGroups < count) acc += sh_w[group + k * kGroups] * ahead[k];
+      for (int k = 0; k < kDepth; ++k) v[k] = i0 + k < used ? __ldg(o + k * kD) : 0.0f;
+      o += kDepth * kD;
+      if ((i0 & 31) == 0) {
+        if (i0 && i0 + lane < used) rec = __ldg(ml + i0 + lane);
+        w = fast_exp2(rec.x - M);
+      }
+#pragma unroll
+      for (int k = 0; k < kDepth; ++k) {
+        const float wk = __shfl_sync(0xffffffffu, w, (i0 + k) & 31);
+        const float lk = __shfl_sync(0xffffffffu, rec.y, (i0 + k) & 31);
+        if (i0 + k < used) {
+          L += wk * lk;
+          acc += wk * v[k];
+        }
+      }
     }
-#pragma unroll 8
-    for (int k = group + (i0 == 0 ? kAhead * kGroups : 0); k < count; k += kGroups)
-      acc += sh_w[k] * __ldg(o + static_cast<size_t>(i0 + k) * kD);
-    __syncthreads();
   }
-#pragma unroll
-  for (int sh = 16; sh; sh >>= 1) l += __shfl_xor_sync(0xffffffffu, l, sh);
-  if (lane == 0) sh_red[warp].y = l;
-  if (kGroups > 1) sh_acc[group][c] = acc;
-  __syncthreads();
-  if (group) return;
-  float L = sh_red[0].y;
-#pragma unroll
-  for (int w = 1; w < kT / 32; ++w) L += sh_red[w].y;
-#pragma unroll
-  for (int k = 1; k < kGroups; ++k) acc += sh_acc[k][c];
   const float r = L > 0.0f ? __fdiv_rn(acc, L) * gv : 0.0f;
   uint16_t bits;
   asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(bits) : "f"(r));
@@ -771,24 +720,12 @@ __global__ void __launch_bounds__(kD* kGroups) attn_combine_kernel(const float* 
   }
 }
 
-// Records per head that the workspace has to hold at least, and those that
-// decode_attention_nvfp4_workspace_size asks for: with few sequences the CTAs
-// (4 on each of 152 SMs) share a head, and lengths up to four times the mean
-// are still spread evenly; S stages never leave more than S records.
-// num_kv_heads is not known there: at least num_q_heads / 8.
-int min_records(int capacity) { return (capacity + kChunk - 1) / kChunk; }
-int64_t preferred_records(int64_t batch, int64_t num_q_heads, int64_t capacity) {
-  const int64_t stages = (capacity + kStageTok - 1) / kStageTok, heads = batch * ((num_q_heads + 7) / 8);
-  const int64_t spread = 4 * ((608 + heads - 1) / heads) + 1, least = min_records(static_cast<int>(capacity)) + 1;
-  const int64_t want = spread > least ? spread : least;
-  return want < stages ? want : stages;
-}
+int splits_for(int capacity) { return (capacity + kChunk - 1) / kChunk; }
 
-constexpr size_t kRecordBytes = (kD + 2) * sizeof(float);  // O, max and sum of one head's segment
 constexpr size_t kSmemBytes =
-    kStages * kStageBytes + (kConsumers * 8 * kMergeHead + 2 * kConsumers * 8) * sizeof(float) + 2 * kStages * 8;
+    kStages * kStageBytes + (kConsumers * 8 * kMergeHead + 2 * kConsumers * 8) * sizeof(float) + (2 * kStages + kItems) * 8;
 
-template <bool kE1M2>
+template <bool kE1M2, bool kListed>
 int resident_ctas() {
   static std::mutex mu;
   static std::map<int, int> cache;
@@ -797,11 +734,11 @@ int resident_ctas() {
   std::lock_guard<std::mutex> lock(mu);
   auto it = cache.find(d);
   if (it != cache.end()) return it->second;
-  if (cudaFuncSetAttribute(attn_partial_kernel<kE1M2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(attn_partial_kernel<kE1M2, kListed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(kSmemBytes)) != cudaSuccess)
     return 0;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attn_partial_kernel<kE1M2>, kThreads, kSmemBytes) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attn_partial_kernel<kE1M2, kListed>, kThreads, kSmemBytes) !=
           cudaSuccess ||
       per_sm <= 0)
     return 0;
@@ -811,11 +748,16 @@ int resident_ctas() {
 
 // The partial kernel for the cache's element format, and its resident CTAs.
 using PartialKernel = void (*)(const Params);
-PartialKernel partial_kernel(const nvfp4_kv_cache* cache) {
-  return cache->kv_format == NVFP4_KV_E1M2 ? attn_partial_kernel<true> : attn_partial_kernel<false>;
+PartialKernel partial_kernel(const nvfp4_kv_cache* cache, bool listed) {
+  return cache->kv_format == NVFP4_KV_E1M2 ? (listed ? attn_partial_kernel<true, true> : attn_partial_kernel<true, false>)
+                                           : (listed ? attn_partial_kernel<false, true> : attn_partial_kernel<false, false>);
 }
+// CTAs of both forms that are resident at once.
 int resident_ctas(const nvfp4_kv_cache* cache) {
-  return cache->kv_format == NVFP4_KV_E1M2 ? resident_ctas<true>() : resident_ctas<false>();
+  const bool e1m2 = cache->kv_format == NVFP4_KV_E1M2;
+  const int own = e1m2 ? resident_ctas<true, false>() : resident_ctas<false, false>();
+  const int listed = e1m2 ? resident_ctas<true, true>() : resident_ctas<false, true>();
+  return own < listed ? own : listed;
 }
 bool kv_format_ok(const nvfp4_kv_cache* cache) {
   return cache->kv_format == NVFP4_KV_E2M1 || cache->kv_format == NVFP4_KV_E1M2;
@@ -828,17 +770,11 @@ using namespace nvfp4;
 
 NVFP4_API size_t decode_attention_nvfp4_workspace_size(int32_t batch, int32_t num_q_heads, int32_t capacity) {
   if (batch <= 0 || num_q_heads <= 0 || capacity <= 0) return 0;
-  return static_cast<size_t>(batch) * num_q_heads * preferred_records(batch, num_q_heads, capacity) * kRecordBytes;
+  return static_cast<size_t>(batch) * num_q_heads * splits_for(capacity) * (kD + 2) * sizeof(float);
 }
 
 namespace nvfp4 {
 namespace {
-
-// The smallest workspace that a call accepts; with less than
-// decode_attention_nvfp4_workspace_size bytes fewer CTAs share a head.
-size_t least_workspace(const nvfp4_kv_cache* cache, int32_t num_q_heads) {
-  return static_cast<size_t>(cache->batch) * num_q_heads * min_records(cache->capacity) * kRecordBytes;
-}
 
 // Checks shared by the decode-attention entry points (all but the output
 // buffers and the split-KV partials).
@@ -855,7 +791,7 @@ nvfp4_status attention_validate(const nvfp4_kv_cache* cache, const void* q_bf16,
       num_q_heads / cache->num_kv_heads > 8)
     return NVFP4_ERR_SHAPE;
   if (static_cast<int64_t>(cache->batch) > 65535 || num_q_heads > 65535) return NVFP4_ERR_SHAPE;
-  const int64_t n_items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * min_records(cache->capacity);
+  const int64_t n_items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * splits_for(cache->capacity);
   if (n_items >= (1ll << 31)) return NVFP4_ERR_SHAPE;
   return NVFP4_OK;
 }
@@ -863,16 +799,14 @@ nvfp4_status attention_validate(const nvfp4_kv_cache* cache, const void* q_bf16,
 // Alignment of the query and cache arrays, then the partial kernel's
 // parameters with its partials at `partials` and its grid size.
 nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, int32_t num_q_heads,
-                              float softmax_scale, float* partials, size_t partials_bytes, Params* prm,
-                              int* grid) {
+                              float softmax_scale, float* partials, Params* prm, int* grid) {
   if (!aligned(q_bf16, 16) || !aligned(cache->k_codes, 16) || !aligned(cache->v_codes, 16) ||
       !aligned(cache->k_scales, 16) || !aligned(cache->v_scales, 16))
     return NVFP4_ERR_ALIGN;
   const int ctas_max = resident_ctas(cache);
   if (ctas_max <= 0) return NVFP4_ERR_CUDA;
-  const int64_t stages = (cache->capacity + kStageTok - 1) / kStageTok;
-  const int64_t heads = static_cast<int64_t>(cache->batch) * cache->num_kv_heads;
-  const int64_t fit = static_cast<int64_t>(partials_bytes / (kRecordBytes * cache->batch * num_q_heads));
+  const int n_splits = splits_for(cache->capacity);
+  const int64_t n_items = static_cast<int64_t>(cache->batch) * cache->num_kv_heads * n_splits;
   prm->k_codes = cache->k_codes;
   prm->k_scales = cache->k_scales;
   prm->v_codes = cache->v_codes;
@@ -885,37 +819,36 @@ nvfp4_status attention_params(const nvfp4_kv_cache* cache, const void* q_bf16, i
   prm->hq = num_q_heads;
   prm->group = num_q_heads / cache->num_kv_heads;
   prm->batch = cache->batch;
-  // Never more than asked for, so that a larger workspace changes no result.
-  const int64_t want = preferred_records(cache->batch, num_q_heads, cache->capacity);
-  prm->records = static_cast<int>(fit < want ? fit : want);
-  // Up to three stages a head's own work is shorter than what finding and
-  // merging a run's parts costs (us, whole / runs: 1 x 40 heads, 154 tokens 5.9
-  // / 7.0, 384 7.2 / 8.1, 512 8.1 / 6.2; 64 x 40: 10.2 / 11.3, 14.5 / 15.7).
-  prm->whole = stages <= 3 || (stages <= 8 && 2 * heads >= ctas_max) || prm->records < 2;
-  if (prm->whole) prm->records = 1;
+  prm->n_splits = n_splits;
+  prm->n_items = static_cast<int>(n_items);
   prm->logit_mult = softmax_scale * cache->k_gscale * kLog2e;
   prm->fault_skip_stage = take_fault(NVFP4_FAULT_ATTN_SKIP_STAGE) ? 1 : 0;
   // Every record the combine kernel reads is written by the partial kernel of
   // the same call, so nothing left from an earlier call needs clearing.
   prm->o_ws = partials;
-  prm->ml_ws = prm->o_ws + static_cast<size_t>(cache->batch) * num_q_heads * prm->records * kD;
-  const int64_t ctas = prm->whole ? heads : heads * stages;
-  *grid = static_cast<int>(ctas < ctas_max ? ctas : ctas_max);
+  prm->ml_ws = prm->o_ws + static_cast<size_t>(cache->batch) * num_q_heads * n_splits * kD;
+  *grid = static_cast<int>(n_items < ctas_max ? n_items : ctas_max);
   return NVFP4_OK;
 }
 
-// The partial and the combine kernel.  With few heads of many records the
-// combine's blocks take 8 x 128 threads (1 x 40 heads of 64 records: 4.3 ->
-// 3.0 us); with more heads than SMs they would only crowd each other (both
-// kernels, 8 x 32 heads of 8-9 records: 13.2 against 15.4 us).
+// The partial and the combine kernel.
 template <bool kQuant>
 nvfp4_status attention_launch(const nvfp4_kv_cache* cache, const Params& prm, int grid, const CombineOut& out,
                               cudaStream_t s) {
-  const bool wide = prm.records > 8 && static_cast<int64_t>(prm.hq) * prm.batch <= sm_count();
-  if (launch_pdl(partial_kernel(cache), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
-      launch_pdl(wide ? attn_combine_kernel<kQuant, 8> : attn_combine_kernel<kQuant, 1>, dim3(prm.hq, prm.batch),
-                 dim3(wide ? 8 * kD : kD), 0, s, static_cast<const float*>(prm.o_ws),
-                 static_cast<const float*>(prm.ml_ws), prm.records, cache->v_gscale, out) != cudaSuccess)
+  const bool listed = prm.n_splits > 1 && prm.n_items > grid;
+  // 32 loads in flight for few heads with many records (1 x 64 heads of 128
+  // records: 49.8 -> 47.3 us, both kernels); with more heads the blocks hide each
+  // other's latency.  Up to four records the kernel keeps 32 registers a thread,
+  // with which its blocks fit beside four partial CTAs of the next call (24 x 40
+  // heads of one record: 17.8 us, with 38 registers 18.3-20.5).
+  const bool deep = prm.n_splits > 8 && static_cast<int64_t>(prm.hq) * prm.batch <= 2 * sm_count();
+  const auto combine = deep                ? attn_combine_kernel<kQuant, 32>
+                       : prm.n_splits <= 4 ? attn_combine_kernel<kQuant, 4>
+                                           : attn_combine_kernel<kQuant, 8>;
+  if (launch_pdl(partial_kernel(cache, listed), dim3(grid), dim3(kThreads), kSmemBytes, s, prm) != cudaSuccess ||
+      launch_pdl(combine, dim3(prm.hq, prm.batch), dim3(kD), 0, s,
+                 static_cast<const float*>(prm.o_ws), static_cast<const float*>(prm.ml_ws), prm.seq_lens, prm.capacity,
+                 prm.n_splits, cache->v_gscale, out) != cudaSuccess)
     return NVFP4_ERR_CUDA;
   count_launches(2);
   return launch_status();
@@ -931,12 +864,12 @@ NVFP4_API nvfp4_status decode_attention_nvfp4(const nvfp4_kv_cache* cache, const
   if (!out_bf16 || !workspace) return NVFP4_ERR_INVALID_ARG;
   nvfp4_status st = attention_validate(cache, q_bf16, num_q_heads, softmax_scale);
   if (st != NVFP4_OK) return st;
-  if (workspace_bytes < least_workspace(cache, num_q_heads)) return NVFP4_ERR_SHAPE;
+  if (workspace_bytes < decode_attention_nvfp4_workspace_size(cache->batch, num_q_heads, cache->capacity))
+    return NVFP4_ERR_SHAPE;
   if (!aligned(out_bf16, 16) || !aligned(workspace, 16)) return NVFP4_ERR_ALIGN;
   Params prm;
   int grid = 0;
-  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), workspace_bytes, &prm,
-                        &grid);
+  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), &prm, &grid);
   if (st != NVFP4_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   return attention_launch<false>(cache, prm, grid, CombineOut{static_cast<uint16_t*>(out_bf16)}, s);
@@ -950,13 +883,13 @@ NVFP4_API nvfp4_status decode_attention_nvfp4_quantize(const nvfp4_kv_cache* cac
   if (!g_out || !out_codes || !out_scales || !workspace) return NVFP4_ERR_INVALID_ARG;
   nvfp4_status st = attention_validate(cache, q_bf16, num_q_heads, softmax_scale);
   if (st != NVFP4_OK) return st;
-  if (workspace_bytes < least_workspace(cache, num_q_heads)) return NVFP4_ERR_SHAPE;
+  if (workspace_bytes < decode_attention_nvfp4_workspace_size(cache->batch, num_q_heads, cache->capacity))
+    return NVFP4_ERR_SHAPE;
   if (!aligned(out_codes, 16) || !aligned(out_scales, 4) || !aligned(g_out, 4) || !aligned(workspace, 16))
     return NVFP4_ERR_ALIGN;
   Params prm;
   int grid = 0;
-  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), workspace_bytes, &prm,
-                        &grid);
+  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, static_cast<float*>(workspace), &prm, &grid);
   if (st != NVFP4_OK) return st;
   CombineOut o{};
   o.codes = out_codes;
@@ -1007,13 +940,15 @@ NVFP4_API nvfp4_status decode_attention_nvfp4_static_scratch(const nvfp4_kv_cach
   nvfp4_status st = attention_validate(cache, q_bf16, num_q_heads, softmax_scale);
   if (st != NVFP4_OK) return st;
   // The partials must fit in the static scratch; larger problems are refused.
-  if (least_workspace(cache, num_q_heads) > NVFP4_ATTN_STATIC_SCRATCH_BYTES) return NVFP4_ERR_SHAPE;
+  if (decode_attention_nvfp4_workspace_size(cache->batch, num_q_heads, cache->capacity) >
+      NVFP4_ATTN_STATIC_SCRATCH_BYTES)
+    return NVFP4_ERR_SHAPE;
   if (!aligned(out_bf16, 16)) return NVFP4_ERR_ALIGN;
   float* scratch = attn_static_scratch_dev();
   if (!scratch) return NVFP4_ERR_CUDA;
   Params prm;
   int grid = 0;
-  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, scratch, NVFP4_ATTN_STATIC_SCRATCH_BYTES, &prm, &grid);
+  st = attention_params(cache, q_bf16, num_q_heads, softmax_scale, scratch, &prm, &grid);
   if (st != NVFP4_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   return attention_launch<false>(cache, prm, grid, CombineOut{static_cast<uint16_t*>(out_bf16)}, s);

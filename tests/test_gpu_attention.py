@@ -528,20 +528,7 @@ def test_injected_missing_stage_times_out_and_device_stays_usable(N):
         assert_close(f32(out)[b], ref[b], what=f"after the injected timeout, seq {b}")
 
 
-@pytest.mark.parametrize("hq,hkv,cap,lens,fmt", [
-    (4, 2, 2048, [0, 128, 129, 2048, 1, 0, 1280, 127], 0),    # empty sequences, stage edges
-    (8, 1, 6144, [6143, 300], 1),                              # one long sequence beside a short one
-    (8, 8, 512, [512] * 40, 0),                                # more heads than a run: several heads per CTA
-    (6, 2, 126, [126, 5, 64], 0),                              # at most one stage per head
-    (5, 1, 1536, [(37 * i) % 1537 for i in range(70)], 0),     # 70 sequences of all lengths
-    (8, 8, 1400, [1400, 3, 128, 1, 90, 0, 1400, 129] * 6, 1),  # runs of one-stage heads beside long ones
-    (8, 8, 2048, [1100] * 40, 0),                              # equal, a little longer than a run
-    (16, 8, 1024, [1024, 7, 500, 0] * 12, 0)])                 # whole heads: many of up to eight stages
-@pytest.mark.parametrize("least", [False, True])
-def test_decode_attention_runs_over_ragged_lengths(N, hq, hkv, cap, lens, fmt, least):
-    """Equal runs of stages over ragged caches, with the asked-for workspace
-    and with the smallest one that is accepted."""
-    B = len(lens)
+def random_cache(N, B, hkv, cap, lens, fmt):
     gen = torch.Generator(device="cuda").manual_seed(B + cap)
     cache = N.KVCache(B, hkv, cap, 0.013, 0.021, kv_format=fmt)
     for t in (cache.k_codes, cache.v_codes):
@@ -553,13 +540,36 @@ def test_decode_attention_runs_over_ragged_lengths(N, hq, hkv, cap, lens, fmt, l
     for t in (cache.k_scales, cache.v_scales):
         t.copy_(torch.randint(0x28, 0x48, t.shape, generator=gen, device="cuda", dtype=torch.int32).to(torch.uint8))
     cache.seq_lens.copy_(torch.tensor(lens, dtype=torch.int32))
-    q = torch.randn(B, hq, 128, generator=gen, device="cuda").to(torch.bfloat16)
-    need = B * hq * ((cap + 1023) // 1024) * 520 if least else N.decode_attention_nvfp4_workspace_size(B, hq, cap)
+    return cache, gen
+
+
+def attend(N, cache, q, extra=0):
+    """Decode attention with a workspace of `extra` bytes more than asked for, filled with NaN."""
+    B, hq, _ = q.shape
+    need = N.decode_attention_nvfp4_workspace_size(B, hq, cache.capacity) + extra
     ws = torch.full((need // 4,), float("nan"), dtype=torch.float32, device="cuda")
     out = torch.full((B, hq, 128), float("nan"), dtype=torch.bfloat16, device="cuda")
     N.decode_attention_nvfp4(cache, q, 1 / math.sqrt(128), out, ws)
     torch.cuda.synchronize()
     assert N.nvfp4_get_device_status() == 0
+    return out
+
+
+@pytest.mark.parametrize("hq,hkv,cap,lens,fmt", [
+    (4, 2, 2048, [0, 128, 129, 2048, 1, 0, 1280, 127], 0),    # empty sequences, stage edges
+    (8, 1, 6144, [6143, 300], 1),                              # one long sequence beside a short one
+    (8, 8, 512, [512] * 40, 0),                                # one chunk per head
+    (6, 2, 126, [126, 5, 64], 0),                              # at most one stage per head
+    (5, 1, 1536, [(37 * i) % 1537 for i in range(70)], 0),     # 70 sequences of all lengths
+    (8, 8, 1400, [1400, 3, 128, 1, 90, 0, 1400, 129] * 6, 1),  # runs of one-stage chunks beside long ones
+    (8, 8, 2048, [1100] * 40, 0),                              # equal, a little longer than a chunk
+    (16, 8, 1024, [1024, 7, 500, 0] * 25, 0),                  # more one-chunk heads than CTAs
+    (8, 8, 4096, [0, 0, 4096, 1025, 0, 1024, 2, 0, 2049] * 3, 0)])  # runs that begin and end at empty sequences
+def test_decode_attention_over_ragged_lengths(N, hq, hkv, cap, lens, fmt):
+    B = len(lens)
+    cache, gen = random_cache(N, B, hkv, cap, lens, fmt)
+    q = torch.randn(B, hq, 128, generator=gen, device="cuda").to(torch.bfloat16)
+    out = attend(N, cache, q)
     grid = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6] if not fmt else
                         [n / 2 for n in range(8)] + [(n - 16) / 2 for n in range(8, 16)], dtype=torch.float64, device="cuda")
 
@@ -576,6 +586,29 @@ def test_decode_attention_runs_over_ragged_lengths(N, hq, hkv, cap, lens, fmt, l
         p = torch.softmax(qq @ k[b, :, :n].transpose(1, 2) / math.sqrt(128), dim=-1)
         ref = (p @ v[b, :, :n]).reshape(hq, 128)
         assert_close(f32(out[b]), ref.cpu().numpy(), what=f"sequence {b} of {n}")
+
+
+@pytest.mark.parametrize("hq,hkv,cap,lens,fmt", [
+    (16, 8, 8192, [5000, 0, 8192, 1030, 1024, 300, 2049, 7777, 6144, 1, 4000, 129] * 2, 0),  # runs of chunks
+    (8, 2, 6000, [6000, 700, 3333], 1),                                                     # a CTA for each chunk
+    (8, 8, 1000, [1000, 5, 640, 999] * 24, 0)])                                             # one-chunk heads, several per CTA
+def test_decode_attention_of_a_sequence_is_its_own(N, hq, hkv, cap, lens, fmt):
+    """A sequence's result does not depend on the sequences beside it, on the
+    capacity or on the workspace's size: bit for bit that of a batch of one
+    whose capacity just holds it."""
+    B = len(lens)
+    cache, gen = random_cache(N, B, hkv, cap, lens, fmt)
+    q = torch.randn(B, hq, 128, generator=gen, device="cuda").to(torch.bfloat16)
+    out = attend(N, cache, q)
+    assert torch.equal(out, attend(N, cache, q, extra=1 << 20))
+    for b, n in enumerate(lens):
+        if n == 0:
+            continue
+        own = N.KVCache(1, hkv, (n + 1) & ~1, 0.013, 0.021, kv_format=fmt)
+        for name in ("k_codes", "k_scales", "v_codes", "v_scales"):
+            getattr(own, name).copy_(getattr(cache, name)[b:b + 1, :, :(n + 1) & ~1])
+        own.seq_lens.fill_(n)
+        assert torch.equal(out[b:b + 1], attend(N, own, q[b:b + 1].contiguous())), f"sequence {b} of {n}"
 
 
 @pytest.mark.parametrize("n_new,hkv", [(1, 1), (3, 3), (7, 8), (608, 8), (611, 8), (1231, 6), (2433, 8), (2431, 4)])
