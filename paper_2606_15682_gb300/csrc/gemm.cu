@@ -31,9 +31,6 @@
 namespace nvfp4 {
 namespace {
 
-#ifndef NVFP4_GEMM_COPY_WARPS
-#define NVFP4_GEMM_COPY_WARPS 2
-#endif
 #ifndef NVFP4_GEMM_PAIR_STAGES
 #define NVFP4_GEMM_PAIR_STAGES 5
 #endif
@@ -485,8 +482,8 @@ __global__ void __launch_bounds__(C::kThreads, 1)
 // tile with tcgen05.mma.cta_group::2: each CTA holds its own 128 rows of A and
 // its own 128-row half of the W tile in shared memory, and its 128 x 256 slice
 // of the accumulator in its own TMEM.  Per SM this halves the W bytes loaded
-// and the scale copies issued for the same FLOPs.  W scales (all 256 rows) go
-// to both CTAs so that each TMEM receives the full set.  The leader (rank 0)
+// and the scale copies issued for the same FLOPs.  Each CTA loads the W scales
+// of all 256 rows, so that each TMEM receives the full set.  The leader (rank 0)
 // issues the copies and the MMAs; all loads are counted on its barriers.
 //
 // Per 256-deep k-block the MMAs take 512 cycles.  What kept it at 717 was no
@@ -494,20 +491,22 @@ __global__ void __launch_bounds__(C::kThreads, 1)
 // five loads and two expects (617 cycles per stage with MMAs and copies taken
 // out), scale buffers held until the MMAs were done, and an MMA issuer that
 // spent more than the last MMA's 128 cycles between two k-blocks.  So:
-//   - the codes come from warp 0 of each CTA, the scales of both CTAs from the
-//     peer's warps 1 and 2, whose leader counterparts issue MMAs and copies; W
-//     scales, the same for both, are multicast;
+//   - each CTA loads its codes from warp 0 and its scales from another warp
+//     (leader 3, peer 1); in the leader warp 1 issues the MMAs, warp 2 the copies;
+//   - a CTA's W scales of a stage are two 128-row tiles of a 3-D map, one load.
+//     (One multicast load for both CTAs was no faster, and no load goes to
+//     several CTAs: replicas of this library run on several GPUs at once.)
 //   - a stage's scale buffers are free for the next load once the copies have
-//     read them (the peer's `full` barrier), and TMEM slots once the MMAs have;
+//     read them (`full`), and TMEM slots once the MMAs have;
 //   - codes and copies arrive on one barrier, so the MMA issuer waits once per
 //     k-block, and it tests the next stage's barrier right after its commit;
 //   - warps walk these loops converged and one elected lane issues, which
-//     leaves descriptors in uniform registers.
-// GB300, back to back: 8192 x 55296 x 5120 719 -> 638 us, 8192 x 5120 x 27648
-// 366 -> 316, 8192 x 5120 x 8192 113 -> 97, 2048 x 17920 x 1536 29.2 -> 25.4
-// (a form that kept W in shared memory for K <= 1536: 26.5).
-// Sharing W between two pairs by multicast (clusters of four) changed no
-// pair's rate, and only 144 SMs fit such clusters.
+//     leaves descriptors in uniform registers (one copy warp then does what two
+//     did).
+// GB300, back to back: 8192 x 55296 x 5120 717 -> 641 us, 8192 x 5120 x 27648
+// 361 -> 311, 8192 x 5120 x 8192 114 -> 97, 2048 x 17920 x 1536 29.1 -> 24.9
+// (a form that kept W in shared memory for K <= 1536: 26.5).  The leader's warp 0
+// with the scale loads beside the codes, and two copy warps: 661, 320, 99, 25.5.
 
 __device__ __forceinline__ void mma_fp4_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                              uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
@@ -552,25 +551,16 @@ __device__ __forceinline__ void tma_load_2d_to(void* smem_dst, const void* tmap,
       "l"(reinterpret_cast<uint64_t>(tmap)), "r"(remote), "r"(x), "r"(y)
       : "memory");
 }
-// The same into the CTAs of `mask` (at the same offset in each).
-__device__ __forceinline__ void tma_load_2d_multicast(void* smem_dst, const void* tmap, uint64_t* bar, int x, int y,
-                                                      uint32_t lead, uint32_t mask) {
+// The same for a 3-D box at (0, y, z).
+__device__ __forceinline__ void tma_load_3d_to(void* smem_dst, const void* tmap, uint64_t* bar, int y, int z,
+                                               uint32_t lead) {
   uint32_t remote;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(bar)), "r"(lead));
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      ".multicast::cluster [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(remote), "r"(x), "r"(y), "h"(static_cast<uint16_t>(mask))
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(remote), "r"(0), "r"(y), "r"(z)
       : "memory");
-}
-// Arrive on the barrier at this shared-memory offset in CTA `rank` of the
-// cluster, adding `bytes` to the transactions that its phase waits for.
-// Relaxed: it orders no memory; the loads' completion does.
-__device__ __forceinline__ void mbar_arrive_expect_tx_cluster(uint64_t* bar, uint32_t rank, uint32_t bytes) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(bar)), "r"(rank));
-  asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(remote), "r"(bytes)
-               : "memory");
 }
 // After a pipeline gave up: let the copies that this thread issued land before
 // its CTA (or the CTA they go to) exits.  Copies whose barrier another CTA
@@ -596,8 +586,8 @@ struct PairCfg {
   static constexpr int BN = 256;                 // MMA N (both halves of the pair)
   static constexpr int kStages = STAGES_;
   static constexpr int kEpiWarps = 8;            // 128 rows x 256 accumulator columns per CTA
-  static constexpr int kCopyWarps = NVFP4_GEMM_COPY_WARPS;  // warps issuing the scale copies (1, 2 or 4)
-  static constexpr int kEpi0 = 2 + kCopyWarps;   // first epilogue warp
+  static constexpr int kScaleWarp = 3;           // the leader's scale producer; the peer's is warp 1
+  static constexpr int kEpi0 = 4;                // first epilogue warp
   static constexpr int kThreads = 32 * (kEpi0 + kEpiWarps);
   static constexpr uint32_t kTileBytesA = BM * BK / 2;   // own 128 rows
   static constexpr uint32_t kTileBytesB = 128 * BK / 2;  // own half of the 256-row W tile
@@ -664,17 +654,17 @@ __global__ void __launch_bounds__(C::kThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      // One commit per copy warp once the stage's scales are in TMEM, in the
-      // leader also an expect_tx that covers both CTAs' code bytes.  In the
-      // peer it frees the stage's scale buffers for the next load.
-      mbar_init(&full[s], C::kCopyWarps + (leader ? 1 : 0));
+      // The commit of the copies that put the stage's scales into TMEM, in the
+      // leader also an expect_tx that covers both CTAs' code bytes.  It frees
+      // the stage's scale buffers for the next load.
+      mbar_init(&full[s], leader ? 2 : 1);
       mbar_init(&empty[s], 1);
       mbar_init(&sffull[s], 1);
     }
     mbar_init(tfull, 1);
     mbar_init(tempty, 2 * C::kEpiWarps);
     mbar_init(drain, 1);
-    mbar_init(drain_cp, C::kCopyWarps);
+    mbar_init(drain_cp, 1);
     abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tmap_a);
@@ -725,6 +715,14 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     if (abort_flag) drain_delay();
   };
 
+  // A CTA's own A scales and both tiles of the W scales (a half unit needs only
+  // the first); 8 rows of 256 bytes are the four 512-byte atoms of one (128-row
+  // tile, k-block).
+  auto load_scales = [&](int stage, int kb, int a_tile, int w_tile) {
+    if (leader) mbar_arrive_expect_tx(&sffull[stage], 2 * (C::kSfaBytes + C::kSfbBytes));
+    tma_load_2d_to(sSFA + stage * C::kSfaBytes, &tmap_sfa, &sffull[stage], 0, a_tile * kgroups * 2 + kb * 8, 0);
+    tma_load_3d_to(sSFB + stage * C::kSfbBytes, &tmap_sfb, &sffull[stage], kb * 8, w_tile, 0);
+  };
   if (warp == 0) {
     // ------------------------------------------------------ producer: codes ---
     produce(empty,
@@ -744,35 +742,15 @@ __global__ void __launch_bounds__(C::kThreads, 1)
               tma_load_2d_to(a_dst, &tmap_a, &full[stage], kx, rows.x, 0);
               tma_load_2d_to(b_dst, map_b, &full[stage], kx, rows.y, 0);
             });
-  } else if (warp == 1 && !leader) {
-    // --------------------------------- producer (peer): both CTAs' A scales ---
-    // Scale atoms through a [bytes / 256, 256] view: one (128-row tile,
-    // k-block) group of four 512-byte atoms is 8 rows of that view.
+  } else if (leader ? warp == C::kScaleWarp : warp == 1) {
+    // ----------------------------------------------------- producer: scales ---
+    // A stage's scale buffers are free once the copies have read them: the
+    // peer's `full` barrier says so, the leader's a little later (codes landed).
     produce(full,
-            [&](int ms, int, int) {
-              return make_int2(min(ms * 2, args.tiles_m - 1) * kgroups * 2,
-                               min(ms * 2 + 1, args.tiles_m - 1) * kgroups * 2);
+            [&](int ms, int nb, int half) {
+              return make_int2(min(ms * 2 + static_cast<int>(rank), args.tiles_m - 1), nb * 2 + max(half, 0));
             },
-            [&](int stage, int kb, int2 rows, bool wide) {
-              uint8_t* dst = sSFA + stage * C::kSfaBytes;
-              mbar_arrive_expect_tx_cluster(&sffull[stage], 0,
-                                            2 * (C::kSfaBytes + (wide ? C::kSfbBytes : C::kSfaBytes)));
-              tma_load_2d_multicast(dst, &tmap_sfa, &sffull[stage], 0, rows.x + kb * 8, 0, 1u);
-              tma_load_2d_to(dst, &tmap_sfa, &sffull[stage], 0, rows.y + kb * 8, 0);
-            });
-  } else if (warp == 2 && !leader) {
-    // ------------------------------ producer (peer): W scales, to both CTAs ---
-    produce(full,
-            [&](int, int nb, int half) {
-              const int row = (nb * 2 + max(half, 0)) * kgroups * 2;
-              return make_int2(row, row + kgroups * 2);
-            },
-            [&](int stage, int kb, int2 rows, bool wide) {
-              uint8_t* dst = sSFB + stage * C::kSfbBytes;
-              tma_load_2d_multicast(dst, &tmap_sfb, &sffull[stage], 0, rows.x + kb * 8, 0, 3u);
-              if (wide)
-                tma_load_2d_multicast(dst + C::kSfaBytes, &tmap_sfb, &sffull[stage], 0, rows.y + kb * 8, 0, 3u);
-            });
+            [&](int stage, int kb, int2 tiles, bool) { load_scales(stage, kb, tiles.x, tiles.y); });
   } else if (warp == 1 && leader) {
     // ------------------------------------------------ MMA issuer (leader) ---
     // The whole warp walks the loop and one elected lane issues, so that the
@@ -819,12 +797,8 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     }
     if (issuer) tc_commit_pair(drain, 0x1);
     mbar_wait_bounded(drain, 0, nullptr);
-  } else if (warp >= 2 && warp < 2 + C::kCopyWarps && leader) {
+  } else if (warp == 2 && leader) {
     // ------------------------------------- leader: block scales -> TMEM ---
-    // The K=64 steps of a stage are spread over the copy warps: copies issued
-    // from different warps proceed concurrently, copies from one thread do not.
-    constexpr int kPerWarp = 4 / C::kCopyWarps;
-    const int kk0 = (__shfl_sync(0xffffffffu, warp, 0) - 2) * kPerWarp;
     const bool issuer = elect_one();
     int stage = 0;
     uint32_t phase = 0;
@@ -845,7 +819,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
         const uint64_t sfb_desc = sfb_desc0 + static_cast<uint32_t>(stage) * (C::kSfbBytes >> 4);
         if (issuer) {
 #pragma unroll
-          for (int kk = kk0; kk < kk0 + kPerWarp; ++kk) {
+          for (int kk = 0; kk < 4; ++kk) {
             copy_sf_to_tmem_pair(sfa_col + kk * 4, sfa_desc + kk * (512 >> 4));
             copy_sf_to_tmem_pair(sfb_col + kk * 8, sfb_desc + kk * (512 >> 4));
             if (wide) copy_sf_to_tmem_pair(sfb_col + kk * 8 + 4, sfb_desc + (C::kSfaBytes + kk * 512) / 16);
@@ -1154,13 +1128,13 @@ __global__ void __launch_bounds__(C::kThreads, 1)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], C::kCopyWarps + (leader ? 1 : 0));  // as in the pair kernel
+      mbar_init(&full[s], leader ? 2 : 1);  // as in the pair kernel
       mbar_init(&empty[s], 1);
       mbar_init(&sffull[s], 1);
     }
     mbar_init(tfull, 1);
     mbar_init(drain, 1);
-    mbar_init(drain_cp, C::kCopyWarps);
+    mbar_init(drain_cp, 1);
     abort_flag = 0;
     fence_mbar_init();
     prefetch_tmap(&tmap_a);
@@ -1202,34 +1176,24 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     }
     if (abort_flag) drain_delay();
   };
+  const int a_tile = min(mb, args.tiles_m - 1);  // a spare CTA reloads the last tile
+  auto load_scales = [&](int stage, int kb) {
+    if (leader) mbar_arrive_expect_tx(&sffull[stage], 2 * (C::kSfaBytes + C::kSfbBytes));
+    tma_load_2d_to(sSFA + stage * C::kSfaBytes, &tmap_sfa, &sffull[stage], 0, a_tile * kgroups * 2 + kb * 8, lead);
+    tma_load_3d_to(sSFB + stage * C::kSfbBytes, &tmap_sfb, &sffull[stage], kb * 8, nb * 2, lead);
+  };
   if (warp == 0) {
     // ------------------------------------------------------ producer: codes ---
-    const int a_row = min(mb, args.tiles_m - 1) * BM;  // a spare CTA reloads the last tile
     const int b_row = nb * BN + static_cast<int>(half) * 128;
     produce(empty, [&](int stage, int kb) {
       if (leader) mbar_arrive_expect_tx(&full[stage], 2 * (C::kTileBytesA + C::kTileBytesB));
-      tma_load_2d_to(sA + stage * C::kTileBytesA, &tmap_a, &full[stage], kb * (BK / 2), a_row, lead);
+      tma_load_2d_to(sA + stage * C::kTileBytesA, &tmap_a, &full[stage], kb * (BK / 2), a_tile * BM, lead);
       tma_load_2d_to(sB + stage * C::kTileBytesB, &tmap_b, &full[stage], kb * (BK / 2), b_row, lead);
       if (kb == k0) gemm_stamp(2);
     });
-  } else if (warp == 1 && !leader) {
-    // --------------------------------- producer (peer): both CTAs' A scales ---
-    const int row0 = min(ms * 2, args.tiles_m - 1) * kgroups * 2, row1 = min(ms * 2 + 1, args.tiles_m - 1) * kgroups * 2;
-    produce(full, [&](int stage, int kb) {
-      uint8_t* dst = sSFA + stage * C::kSfaBytes;
-      mbar_arrive_expect_tx_cluster(&sffull[stage], lead, 2 * (C::kSfaBytes + C::kSfbBytes));
-      tma_load_2d_multicast(dst, &tmap_sfa, &sffull[stage], 0, row0 + kb * 8, lead, 1u << lead);
-      tma_load_2d_to(dst, &tmap_sfa, &sffull[stage], 0, row1 + kb * 8, lead);
-    });
-  } else if (warp == 2 && !leader) {
-    // ------------------------------ producer (peer): W scales, to both CTAs ---
-    const int row = nb * 2 * kgroups * 2;
-    produce(full, [&](int stage, int kb) {
-      uint8_t* dst = sSFB + stage * C::kSfbBytes;
-      tma_load_2d_multicast(dst, &tmap_sfb, &sffull[stage], 0, row + kb * 8, lead, 3u << lead);
-      tma_load_2d_multicast(dst + C::kSfaBytes, &tmap_sfb, &sffull[stage], 0, row + kgroups * 2 + kb * 8, lead,
-                            3u << lead);
-    });
+  } else if (leader ? warp == C::kScaleWarp : warp == 1) {
+    // ----------------------------------------------------- producer: scales ---
+    produce(full, load_scales);
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer (leader) ---
     const bool issuer = elect_one();
@@ -1260,10 +1224,8 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       tc_commit_pair(drain, static_cast<uint16_t>(1u << lead));
     }
     mbar_wait_bounded(drain, 0, nullptr);
-  } else if (warp >= 2 && warp < 2 + C::kCopyWarps && leader) {
+  } else if (warp == 2 && leader) {
     // ------------------------------------- leader: block scales -> TMEM ---
-    constexpr int kPerWarp = 4 / C::kCopyWarps;
-    const int kk0 = (__shfl_sync(0xffffffffu, warp, 0) - 2) * kPerWarp;
     const bool issuer = elect_one();
     int stage = 0;
     uint32_t phase = 0;
@@ -1278,7 +1240,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       const uint64_t sfb_desc = sfb_desc0 + static_cast<uint32_t>(stage) * (C::kSfbBytes >> 4);
       if (issuer) {
 #pragma unroll
-        for (int kk = kk0; kk < kk0 + kPerWarp; ++kk) {
+        for (int kk = 0; kk < 4; ++kk) {
           copy_sf_to_tmem_pair(sfa_col + kk * 4, sfa_desc + kk * (512 >> 4));
           copy_sf_to_tmem_pair(sfb_col + kk * 8, sfb_desc + kk * (512 >> 4));
           copy_sf_to_tmem_pair(sfb_col + kk * 8 + 4, sfb_desc + (C::kSfaBytes + kk * 512) / 16);
@@ -2110,16 +2072,17 @@ bool make_code_map(CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t 
 
 // MMA-layout block scales of a [rows, K] operand viewed as [bytes / 256, 256]
 // bytes; a box of 8 rows is one (128-row tile, k-block) group of four atoms.
-bool make_scale_map(CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t K) {
+// pair: [row tiles, K / 32, 256] bytes and boxes of two row tiles.
+bool make_scale_map(CUtensorMap* map, const uint8_t* base, int64_t rows, int64_t K, bool pair) {
   auto enc = tensor_map_encoder();
   if (!enc) return false;
-  const int64_t bytes = ((rows + 127) / 128) * 128 * (K / 16);
-  cuuint64_t dims[2] = {256, static_cast<cuuint64_t>(bytes / 256)};
-  cuuint64_t strides[1] = {256};
-  cuuint32_t box[2] = {256, 8};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+  const cuuint64_t tile_rows = static_cast<cuuint64_t>(K / 32), tiles = static_cast<cuuint64_t>((rows + 127) / 128);
+  cuuint64_t dims[3] = {256, pair ? tile_rows : tile_rows * tiles, tiles};
+  cuuint64_t strides[2] = {256, 256 * tile_rows};
+  cuuint32_t box[3] = {256, 8, 2};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, pair ? 3 : 2, const_cast<uint8_t*>(base), dims, strides, box,
+                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -2239,7 +2202,7 @@ nvfp4_status launch_pair(const uint8_t* a_codes, const uint8_t* a_scales, const 
   CUtensorMap ma, mb, mb_half, msa, msb, mo;
   if (!make_code_map(&ma, a_codes, M, K, BM) || !make_code_map(&mb, w_codes, N, K, 128) ||
       !make_code_map(&mb_half, w_codes, N, K, 64) ||
-      !make_scale_map(&msa, a_scales, M, K) || !make_scale_map(&msb, w_scales, N, K))
+      !make_scale_map(&msa, a_scales, M, K, false) || !make_scale_map(&msb, w_scales, N, K, true))
     return NVFP4_ERR_CUDA;
   if (kSwiGLU) mo = ma;  // not read by the fused epilogue
   else if (!make_out_map(&mo, out_bf16, M, N, ldo)) return NVFP4_ERR_CUDA;
@@ -2356,7 +2319,7 @@ nvfp4_status launch_splitk(const uint8_t* a_codes, const uint8_t* a_scales, cons
   if (tiles * 2 * splits >= (1ll << 31)) return NVFP4_ERR_SHAPE;
   CUtensorMap ma, mb, msa, msb, mo;
   if (!make_code_map(&ma, a_codes, M, K, BM) || !make_code_map(&mb, w_codes, N, K, 128) ||
-      !make_scale_map(&msa, a_scales, M, K) || !make_scale_map(&msb, w_scales, N, K) ||
+      !make_scale_map(&msa, a_scales, M, K, false) || !make_scale_map(&msb, w_scales, N, K, true) ||
       !make_out_map(&mo, out_bf16, M, N, ldo))
     return NVFP4_ERR_CUDA;
   GemmArgs args = {};

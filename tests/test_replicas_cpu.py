@@ -2,6 +2,7 @@
 gloo ranks on the CPU: each rank contributes its own timings, every rank gets
 the maximum, and the job's rate counts all ranks' work over that time."""
 import os
+import re
 import socket
 import sys
 
@@ -48,3 +49,17 @@ def test_single_rank_is_identity():
     import bench
     assert bench.reduce_max_over_ranks([3.0, 4.0], 1) == [3.0, 4.0]
     assert bench.whole_job_rate(5.0, 1, 1.0) == 5000.0
+
+
+def test_no_load_is_multicast_to_several_ctas():
+    """The library runs as replicas on several GPUs, where no kernel issues a
+    copy that a cluster's CTAs share (tcgen05.commit may arrive in several)."""
+    csrc = os.path.join(ROOT, "paper_2606_15682_gb300", "csrc")
+    copies = 0
+    for name in sorted(os.listdir(csrc)):
+        with open(os.path.join(csrc, name)) as f:
+            for asm in re.findall(r"asm(?: volatile)?\s*\((.*?)\);", f.read(), re.S):
+                if "cp.async.bulk" in asm or "multimem" in asm:
+                    copies += 1
+                    assert "multicast" not in asm and "multimem" not in asm, (name, asm)
+    assert copies
