@@ -513,15 +513,14 @@ nvfp4_status nvfp4_get_device_status(int32_t* status_host, void* stream);
  *     consumers' bounded wait on it runs out after ~2 s: the call reports
  *     NVFP4_ERR_TIMEOUT through nvfp4_get_device_status, its output is
  *     undefined, and the device stays usable.
- *   NVFP4_FAULT_GEMM_SKIP_STAGE: in the next launch of a CTA-pair GEMM kernel
- *     (the 256 x 256 tiles that nvfp4_linear / mxfp4_linear use when N % 256
- *     == 0, with or without a split of K across a cluster, and the fused
- *     SwiGLU calls), both CTAs of the first pair leave their first ring stage
- *     of their K range neither armed nor loaded; the MMA
+ *   NVFP4_FAULT_GEMM_SKIP_STAGE: in the next GEMM launch (nvfp4_linear,
+ *     mxfp4_linear, nvfp4_linear_dynamic and the fused SwiGLU calls, whichever
+ *     kernel serves the shape), the first CTA, or both CTAs of the first CTA
+ *     pair, leave their first ring stage neither armed nor loaded; the MMA
  *     issuer's and the scale copiers' bounded waits run out after ~2 s, every
- *     role of the pair stops, the MMAs issued so far drain and TMEM is freed.
- *     The call reports NVFP4_ERR_TIMEOUT, its output is undefined, and the
- *     device stays usable.
+ *     role of the CTA or pair stops, the MMAs issued so far drain and TMEM is
+ *     freed.  The call reports NVFP4_ERR_TIMEOUT, its output is undefined, and
+ *     the device stays usable.
  *   NVFP4_FAULT_NONE disarms.  Other values -> INVALID_ARG.
  */
 #define NVFP4_FAULT_NONE 0

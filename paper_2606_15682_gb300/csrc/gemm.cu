@@ -207,8 +207,8 @@ struct GemmArgs {
   // Quantization of the fused output: 0 NVFP4 with the static scale g_out,
   // 1 MXFP4, 2 MXFP4 after the H_32 block rotation.
   uint32_t q_mode;
-  // Test-only (nvfp4_debug_inject_fault): both CTAs of pair 0 leave their
-  // first stage unissued (CTA-pair kernel).
+  // Test-only (nvfp4_debug_inject_fault): the first CTA, or both CTAs of the
+  // first pair, leave their first stage neither armed nor loaded.
   int fault_skip_stage;
   // Row super-tiles per raster group (unit_coords).
   int group_m;
@@ -308,6 +308,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     uint32_t issued_parity[kStages];
     bool issued[kStages];
     for (int s = 0; s < kStages; ++s) issued[s] = false;
+    bool skip = args.fault_skip_stage && cta_id == 0;
 #ifdef NVFP4_TIMELINE
     bool first_issue = true;
 #endif
@@ -319,6 +320,11 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       const uint8_t* sfb_tiles = args.sfb + (static_cast<size_t>(nb) * (BN / 128) * kgroups) * 512;
       for (int kb = 0; kb < kblocks; ++kb) {
         if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
+        if (skip) {
+          skip = false;
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          continue;
+        }
         mbar_arrive_expect_tx(&full[stage], C::kStageBytes);
         tma_load_2d(sA + stage * C::kTileBytesA, &tmap_a, &full[stage], kb * (BK / 2), mb * BM);
         bulk_load(sSFA + stage * C::kSfaBytes, sfa_tile + static_cast<size_t>(kb) * C::kSfaBytes, C::kSfaBytes,
@@ -1565,9 +1571,11 @@ __global__ void __launch_bounds__(C::kThreads, 2)
     const bool issuer = elect_one();
     int stage = 0;
     uint32_t phase = 0;
+    bool skip = args.fault_skip_stage && blockIdx.x == 0;
     for (int kb = k0; kb < k1; ++kb) {
       if (!mbar_wait_bounded(&free[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
-      if (issuer) load(stage, kb);
+      if (issuer && !skip) load(stage, kb);
+      skip = false;
       if (++stage == kStages) { stage = 0; phase ^= 1u; }
     }
     if (abort_flag) drain_delay();
@@ -1759,6 +1767,7 @@ struct DynArgs {
   int M, N, K;
   int tiles_n;
   int* status;
+  int fault_skip_stage;  // as in GemmArgs
 };
 
 __device__ __forceinline__ void named_barrier(uint32_t id, uint32_t threads) {
@@ -1840,10 +1849,16 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued = 0, issued_parity = 0;  // one bit per stage
+      bool skip = args.fault_skip_stage && cta_id == 0;
       for (int u = cta_id; u < total_units && !abort_flag; u += n_ctas) {
         const uint8_t* sfb_tile = args.sfb + (static_cast<size_t>(u) * kgroups) * 512;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, &abort_flag)) { fail(); break; }
+          if (skip) {
+            skip = false;
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            continue;
+          }
           mbar_arrive_expect_tx(&full[stage], C::kTileBytesB + C::kSfbBytes);
           bulk_load(sSFB + stage * C::kSfbBytes, sfb_tile + static_cast<size_t>(kb) * C::kSfbBytes, C::kSfbBytes,
                     &full[stage]);
@@ -2146,6 +2161,7 @@ nvfp4_status launch(const uint8_t* a_codes, const uint8_t* a_scales, const float
   args.tiles_n = static_cast<int>(tiles_n);
   args.group_m = raster_group(K, units / tiles_n);
   args.status = status_word_dev();
+  args.fault_skip_stage = take_fault(NVFP4_FAULT_GEMM_SKIP_STAGE) ? 1 : 0;
   const int ctas = static_cast<int>(units < ctas_max ? units : ctas_max);
   if (launch_pdl(nvfp4_gemm_kernel<C>, dim3(ctas), dim3(C::kThreads), C::kSmemBytes, stream, ma, mb, mo, args) !=
       cudaSuccess)
@@ -2456,6 +2472,7 @@ nvfp4_status launch_skinny(const uint8_t* a_codes, const uint8_t* a_scales, cons
   args.splits = splits;
   args.prefetch_kb = kSkinnyPrefetch;
   args.status = status_word_dev();
+  args.fault_skip_stage = take_fault(NVFP4_FAULT_GEMM_SKIP_STAGE) ? 1 : 0;
   args.out = static_cast<uint16_t*>(out_bf16);
   args.ldo = ldo;
   cudaLaunchConfig_t cfg = {};
@@ -2513,6 +2530,7 @@ nvfp4_status launch_dynamic(const uint16_t* x, int64_t M, int64_t K, int64_t ldx
   args.K = static_cast<int>(K);
   args.tiles_n = static_cast<int>(tiles_n);
   args.status = status_word_dev();
+  args.fault_skip_stage = take_fault(NVFP4_FAULT_GEMM_SKIP_STAGE) ? 1 : 0;
   const int sms = sm_count();
   if (sms <= 0) return NVFP4_ERR_CUDA;
   const int ctas = static_cast<int>(tiles_n < sms ? tiles_n : sms);

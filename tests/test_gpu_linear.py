@@ -228,6 +228,49 @@ def test_injected_missing_stage_in_split_k_cluster_times_out(N):
     assert_close(f32(out), O.linear(a_c, a_s, 1.0, w_c, w_s, 1.0), what="after the injected timeout")
 
 
+@pytest.mark.parametrize("M,Nn,K,swiglu", [(32, 1536, 5120, False),   # skinny, clusters that split K
+                                           (128, 7168, 5120, False),
+                                           (8, 5120, 2048, True),     # skinny, SwiGLU epilogue
+                                           (300, 512, 1024, False)])  # single CTAs
+def test_injected_missing_stage_in_the_other_gemm_kernels(N, M, Nn, K, swiglu):
+    """The fault reaches whichever kernel serves the call and is spent there:
+    the call reports NVFP4_ERR_TIMEOUT, the next one gives the same bytes as the
+    one before the fault."""
+    import time
+    gen = torch.Generator().manual_seed(41)
+    dev = "cuda"
+    a_c, a_s = (torch.from_numpy(x).to(dev) for x in random_operand(M, K, gen))
+    w_c, w_s = (torch.from_numpy(x).to(dev) for x in random_operand(Nn, K, gen))
+    a_s, w_s = (torch.from_numpy(O.scales_to_mma(u8(x))).to(dev) for x in (a_s, w_s))
+    g = torch.full((1,), 0.01, device=dev)
+
+    def run():
+        if swiglu:
+            out = torch.full((M, Nn // 4), 0xEE, dtype=torch.uint8, device=dev)
+            sc = torch.full((N.nvfp4_scales_bytes(M, Nn // 2, 1),), 0xEE, dtype=torch.uint8, device=dev)
+            N.nvfp4_linear_swiglu_quantize(a_c, a_s, g, w_c, w_s, g, M, Nn // 2, K, g, out, sc)
+            outs = (out, sc)
+        else:
+            outs = (torch.full((M, Nn), float("nan"), dtype=torch.bfloat16, device=dev),)
+            N.nvfp4_linear(a_c, a_s, g, w_c, w_s, g, outs[0], M, Nn, K)
+        torch.cuda.synchronize()
+        return outs
+    before = run()
+    assert N.nvfp4_get_device_status() == 0
+    N.nvfp4_debug_inject_fault(N.FAULT_GEMM_SKIP_STAGE)
+    try:
+        t0 = time.time()
+        run()
+        waited = time.time() - t0
+        assert N.nvfp4_get_device_status() == 6
+        assert 1.0 < waited < 20.0, f"bounded wait expected (~2-4 s), took {waited:.1f} s"
+        after = run()
+        assert N.nvfp4_get_device_status() == 0
+    finally:
+        N.nvfp4_debug_inject_fault(N.FAULT_NONE)
+    assert all(torch.equal(x, y) for x, y in zip(before, after))
+
+
 # ------------------------------------ gate_up with SwiGLU + quantize fused ---
 
 def test_interleave_gate_up_matches_oracle(N):

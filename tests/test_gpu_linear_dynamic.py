@@ -147,3 +147,27 @@ def test_unsupported_shapes_are_rejected(N):
     with pytest.raises(N.NVFP4Error) as e:
         N.nvfp4_linear_dynamic(x, wc, wsf, gw, out, 16)
     assert e.value.code == 4
+
+
+def test_injected_missing_stage_times_out_and_next_call_is_exact(N):
+    """The first CTA leaves its first W stage unissued (K = 1536: one k-block more
+    than the ring has stages, so the producer waits too): the bounded waits run
+    out, the call reports NVFP4_ERR_TIMEOUT, the next one is exact."""
+    import time
+    M, Nn, K = 16, 1536, 1536
+    x = activation(M, K, 5)
+    wc, wsf, gw = quantized_weight(N, synth.weight(Nn, K, 6, device="cuda"))
+    want, _ = fused(N, x, wc, wsf, gw, Nn, Nn)
+    out = torch.empty(M, Nn, dtype=torch.bfloat16, device="cuda")
+    N.nvfp4_debug_inject_fault(N.FAULT_GEMM_SKIP_STAGE)
+    try:
+        t0 = time.time()
+        N.nvfp4_linear_dynamic(x, wc, wsf, gw, out, Nn)
+        torch.cuda.synchronize()
+        waited = time.time() - t0
+    finally:
+        N.nvfp4_debug_inject_fault(N.FAULT_NONE)
+    assert N.nvfp4_get_device_status() == 6
+    assert 1.0 < waited < 20.0, f"bounded wait expected (~2-4 s), took {waited:.1f} s"
+    got, _ = fused(N, x, wc, wsf, gw, Nn, Nn)
+    assert torch.equal(got, want)
