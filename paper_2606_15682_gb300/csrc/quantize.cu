@@ -54,13 +54,15 @@ __global__ void __launch_bounds__(kThreads) amax_kernel(const uint16_t* __restri
   griddep_wait_and_release();
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t m = 0;
-  for (uint32_t c0 = blockIdx.x * blockDim.x; c0 < map.total; c0 += stride * kUnroll) {
+  // 64 bits: a step may reach past 2^32 near the end.
+  for (uint64_t c0 = blockIdx.x * blockDim.x; c0 < map.total; c0 += stride * kUnroll) {
     uint4 v[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
-      const uint32_t c = c0 + u * stride + threadIdx.x;
+      const uint64_t c = c0 + u * stride + threadIdx.x;
       uint32_t r, j;
-      v[u] = c < map.total ? __ldg(reinterpret_cast<const uint4*>(x + map.elem(c, &r, &j))) : make_uint4(0, 0, 0, 0);
+      v[u] = c < map.total ? __ldg(reinterpret_cast<const uint4*>(x + map.elem(static_cast<uint32_t>(c), &r, &j)))
+                           : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) m = max(m, amax_bits_bf16x8(v[u]));
@@ -190,10 +192,12 @@ __device__ __forceinline__ void zero_scale_padding(uint32_t rows, uint32_t kbloc
   const uint64_t tile_off = static_cast<uint64_t>(rows >> 7) * kgroups * 512u;
   const uint64_t scale_bytes = tile_off + static_cast<uint64_t>(kgroups) * 512u;
   const bool wide = (reinterpret_cast<uintptr_t>(scales) & 15u) == 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < kgroups * 32u; i += gridDim.x * blockDim.x) {
-    const uint32_t l = i & 31u;
+  // 64 bits: a row of 2^33 columns has 2^32 chunks.
+  const uint64_t chunks = static_cast<uint64_t>(kgroups) * 32u;
+  for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i < chunks; i += gridDim.x * blockDim.x) {
+    const uint32_t l = static_cast<uint32_t>(i) & 31u;
     const uint32_t first = used > l ? (used - l + 31u) >> 5 : 0u;  // first padding word of the chunk
-    const uint64_t off = tile_off + static_cast<uint64_t>(i) * 16u;
+    const uint64_t off = tile_off + i * 16u;
     if (!in_bounds(status, off + 16 <= scale_bytes)) continue;
     if (first == 0 && wide) {
       *reinterpret_cast<uint4*>(scales + off) = make_uint4(0, 0, 0, 0);
@@ -522,15 +526,16 @@ __global__ void __launch_bounds__(kThreads) mx_quantize_kernel(const uint16_t* _
   if (kMMA) zero_scale_padding(rows, nb * 2, scales, status);
 }
 
-template <bool kToMMA>
+// Index: 64 bits where a step could reach past 2^32.
+template <bool kToMMA, class Index>
 __global__ void relayout_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, uint32_t rows,
                                 uint32_t kblocks) {
   griddep_wait_and_release();
   const uint32_t kgroups = kblocks >> 2;
   const uint32_t padded = (rows + 127u) & ~127u;
-  const uint32_t n = padded * kblocks;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t r = i / kblocks, kb = i % kblocks;
+  const Index n = static_cast<Index>(padded) * kblocks;
+  for (Index i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t r = static_cast<uint32_t>(i / kblocks), kb = static_cast<uint32_t>(i % kblocks);
     const uint64_t m = mma_scale_offset(r, kb, kgroups);
     if (kToMMA) {
       dst[m] = r < rows ? src[i] : 0;
@@ -737,8 +742,12 @@ NVFP4_API nvfp4_status nvfp4_scales_relayout(const uint8_t* src, uint8_t* dst, i
   if (rows == 0 || cols == 0) return NVFP4_OK;
   const uint32_t kblocks = static_cast<uint32_t>(cols / 16);
   const uint64_t n = static_cast<uint64_t>((rows + 127) / 128 * 128) * kblocks;
-  if (launch_pdl(to == NVFP4_SCALES_MMA ? relayout_kernel<true> : relayout_kernel<false>, dim3(grid_for(n, 256)),
-                 dim3(256), 0, s, src, dst, static_cast<uint32_t>(rows), kblocks) != cudaSuccess)
+  const int grid = grid_for(n, 256);
+  const bool wide = n + static_cast<uint64_t>(grid) * 256 >= (1ull << 32);
+  const auto kernel = to == NVFP4_SCALES_MMA
+                          ? (wide ? relayout_kernel<true, uint64_t> : relayout_kernel<true, uint32_t>)
+                          : (wide ? relayout_kernel<false, uint64_t> : relayout_kernel<false, uint32_t>);
+  if (launch_pdl(kernel, dim3(grid), dim3(256), 0, s, src, dst, static_cast<uint32_t>(rows), kblocks) != cudaSuccess)
     return NVFP4_ERR_CUDA;
   count_launches(1);
   return launch_status();

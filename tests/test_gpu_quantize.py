@@ -302,3 +302,61 @@ def test_dynamic_small_paths_and_padding_rows(N, rows, cols, offset):
     assert np.float32(g.item()) == g_ref and np.array_equal(u8(codes), rc)
     assert np.array_equal(u8(scales), O.scales_to_mma(rs))
     assert (u8(buf[:offset]) == 0xEE).all() and (u8(buf[offset + size:]) == 0xEE).all()
+
+
+def test_indexes_past_32_bits(N):
+    """The largest sizes: a one-row tensor just below 2^33 columns, whose padding
+    rows are just below 2^32 16-byte chunks, and one just below 2^35 elements,
+    2^32 chunks of the amax pass."""
+    if torch.cuda.mem_get_info()[0] < 120 << 30:
+        pytest.skip("needs 120 GB of free device memory")
+    dev, cols = "cuda", (1 << 33) - 64
+    x = torch.zeros(1, cols, dtype=torch.bfloat16, device=dev)
+    x[0, -1], x[0, 5] = 2.0, -1.0
+    g = torch.empty(1, dtype=torch.float32, device=dev)
+    codes = torch.empty(1, cols // 2, dtype=torch.uint8, device=dev)
+    scales = torch.full((N.nvfp4_scales_bytes(1, cols, N.SCALES_MMA),), 0xEE, dtype=torch.uint8, device=dev)
+    N.nvfp4_tensor_scale(x, g)
+    N.nvfp4_quantize(x, g, codes, scales, N.SCALES_MMA)
+    torch.cuda.synchronize()
+    assert N.nvfp4_get_device_status() == 0
+    g_ref = O.tensor_scale(np.array([[2.0]], np.float32))
+    assert np.float32(g.item()) == g_ref
+    ends = f32(torch.cat([x[:, :64], x[:, -64:]], dim=1))
+    rc, rs = O.quantize(ends, g_ref)
+    assert np.array_equal(u8(codes[:, :32]), rc[:, :32]) and np.array_equal(u8(codes[:, -32:]), rc[:, 32:])
+    # Row 0's word of each 64-column group lies at the start of its 512 bytes; all else is padding.
+    words = scales.view(torch.int32).view(-1, 128)
+    assert np.array_equal(u8(words[0, :1].view(torch.uint8)), rs[0, :4])
+    assert np.array_equal(u8(words[-1, :1].view(torch.uint8)), rs[0, 4:])
+    for part in words.split(1 << 23):
+        assert not part[:, 1:].any()
+    del x, codes, scales, words, part
+    x = torch.zeros(1, (1 << 35) - 8 * 1000, dtype=torch.bfloat16, device=dev)
+    x[0, -1] = 3.0
+    N.nvfp4_tensor_scale(x, g)
+    torch.cuda.synchronize()
+    assert np.float32(g.item()) == O.tensor_scale(np.array([[3.0]], np.float32))
+    del x
+    torch.cuda.empty_cache()
+
+
+def test_relayout_past_32_bits(N):
+    """2^32 + 2^13 scales: every column group of the MMA layout is moved."""
+    rows, cols = 128, (1 << 29) + 1024
+    if torch.cuda.mem_get_info()[0] < 30 << 30:
+        pytest.skip("needs 30 GB of free device memory")
+    n = rows * (cols // 16)
+    src = torch.randint(0, 256, (1 << 20,), dtype=torch.uint8, device="cuda").repeat(n // (1 << 20) + 1)[:n].contiguous()
+    src[-8192:] = torch.arange(8192, device="cuda").to(torch.uint8)
+    mma = torch.empty(n, dtype=torch.uint8, device="cuda")
+    back = torch.empty(n, dtype=torch.uint8, device="cuda")
+    N.nvfp4_scales_relayout(src, mma, rows, cols, N.SCALES_ROWMAJOR, N.SCALES_MMA)
+    N.nvfp4_scales_relayout(mma, back, rows, cols, N.SCALES_MMA, N.SCALES_ROWMAJOR)
+    torch.cuda.synchronize()
+    assert N.nvfp4_get_device_status() == 0
+    assert torch.equal(back, src)
+    # Row r's four scales of group k are at 512 k + 16 (r % 32) + 4 (r / 32).
+    rm = src.view(rows, -1, 4)
+    for k in (0, 1, cols // 128, cols // 64 - 1):
+        assert np.array_equal(u8(mma[512 * k:512 * (k + 1)]).reshape(32, 4, 4).transpose(1, 0, 2).reshape(rows, 4), u8(rm[:, k]))
