@@ -73,7 +73,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // has completed and its memory is visible (a no-op without a programmatic
 // dependency), then let the next kernel begin launching.  Called by every
 // kernel of the library before its first global-memory access, so only
-// prologues (barrier set-up, TMEM allocation) overlap the previous kernel.
+// prologues (barrier set-up, TMEM allocation) overlap the previous kernel; the
+// one exception is the skinny GEMM's prefetch of W into L2, which reads nothing
+// into the SM.
 __device__ __forceinline__ void griddep_wait_and_release() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

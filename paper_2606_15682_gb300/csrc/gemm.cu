@@ -131,18 +131,13 @@ __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   return v;
 }
 
-// The CTA-pair epilogue writes its staged boxes with coalesced st.global
-// rather than TMA stores, leaving the TMA unit to the operand loads that bound
-// the kernel: 32B prefill gate_up 731 -> 721 us, qkv 147.5 -> 145.4 us, the
-// other shapes unchanged (bit-identical outputs).  0: TMA stores.
-#ifndef NVFP4_GEMM_LSU_STORE
-#define NVFP4_GEMM_LSU_STORE 1
-#endif
-
 // Write one staged 32 x 64 bf16 box (rows of 128 B whose 16-byte chunks sit at
 // chunk ^ (row % 8)) to out[y.., x..] with coalesced 16-byte stores: per
 // instruction the warp writes 4 rows x 128 B; rows at or past M and chunks at or
-// past N (N % 16 == 0, so a chunk is inside or outside) are skipped.
+// past N (N % 16 == 0, so a chunk is inside or outside) are skipped.  The
+// CTA-pair epilogue's stores: against TMA stores of the same boxes they leave
+// the TMA unit to the operand loads (32B prefill gate_up 731 -> 721 us, qkv 147.5
+// -> 145.4, the other shapes unchanged).
 __device__ __forceinline__ void store_box_lsu(uint32_t buf, uint16_t* out, int64_t ldo, int x, int y, int M, int N,
                                               int lane, int* status) {
   const int cc = lane & 7;
@@ -218,8 +213,8 @@ struct GemmArgs {
   // Split-K kernel: CTA pairs per cluster, each taking one range of K; skinny
   // kernel: CTAs per cluster.
   int splits;
-  // Skinny kernel: rows of the A box, and W k-blocks prefetched into L2.
-  int a_box_rows, prefetch_kb;
+  // Skinny kernel: rows of the A box.
+  int a_box_rows;
   // bf16 output [M, N] with row pitch ldo elements (the stores that do not
   // go through the output tensor map).
   uint16_t* out;
@@ -616,7 +611,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     nvfp4_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                            const __grid_constant__ CUtensorMap tmap_b_half,
                            const __grid_constant__ CUtensorMap tmap_sfa, const __grid_constant__ CUtensorMap tmap_sfb,
-                           const __grid_constant__ CUtensorMap tmap_out, const GemmArgs args) {
+                           const GemmArgs args) {
   constexpr int BN = C::BN;
   constexpr int kStages = C::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -678,7 +673,6 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     prefetch_tmap(&tmap_b_half);
     prefetch_tmap(&tmap_sfa);
     prefetch_tmap(&tmap_sfb);
-    prefetch_tmap(&tmap_out);
   }
   if (warp == 1) {
     tmem_alloc_pair(tmem_slot, kTmemCols);
@@ -953,8 +947,7 @@ __global__ void __launch_bounds__(C::kThreads, 1)
     constexpr int kEpi0 = C::kEpi0;
     const int quarter = warp & 3;
     const int colbase = ((warp - kEpi0) >> 2) * 128;
-    uint8_t* buf_ptr = sEpi + (warp - kEpi0) * kEpiBufBytes;
-    const uint32_t buf = smem_u32(buf_ptr);
+    const uint32_t buf = smem_u32(sEpi + (warp - kEpi0) * kEpiBufBytes);
     const float scale = args.ga ? __fmul_rn(__ldg(args.ga), __ldg(args.gb)) : 1.0f;
     int local = 0;
     for (int u = pair_id; u < total_units; u += n_pairs, ++local) {
@@ -979,8 +972,6 @@ __global__ void __launch_bounds__(C::kThreads, 1)
       if (half >= 0 && colbase) continue;  // a half tile: columns 0..127 of the accumulator
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        if (lane == 0) bulk_wait_read_all();
-        __syncwarp();
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           const uint32_t* v = r + 64 * h + 8 * c;
@@ -991,21 +982,11 @@ __global__ void __launch_bounds__(C::kThreads, 1)
                        pack_bf16x2(__uint_as_float(v[6]) * scale, __uint_as_float(v[7]) * scale));
         }
         const int x = nb * BN + 128 * max(half, 0) + colbase + h * kEpiCols, y = mb * BM + quarter * 32;
-        if (NVFP4_GEMM_LSU_STORE) {
-          __syncwarp();
-          if (x < args.N && y < args.M) store_box_lsu(buf, args.out, args.ldo, x, y, args.M, args.N, lane, args.status);
-          __syncwarp();  // the next box overwrites the staging buffer
-        } else {
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0 && x < args.N && y < args.M) {
-            tma_store_2d(&tmap_out, buf_ptr, x, y);
-            bulk_commit_group();
-          }
-        }
+        __syncwarp();
+        if (x < args.N && y < args.M) store_box_lsu(buf, args.out, args.ldo, x, y, args.M, args.N, lane, args.status);
+        __syncwarp();  // the next box overwrites the staging buffer
       }
     }
-    if (lane == 0) bulk_wait_all();
   }
 
   tc_fence_before();
@@ -1548,7 +1529,7 @@ __global__ void __launch_bounds__(C::kThreads, 2)
     fence_mbar_init();
     prefetch_tmap(&tmap_a);
     prefetch_tmap(&tmap_b);
-    for (int kb = k0; kb < min(k1, k0 + args.prefetch_kb); ++kb) tma_prefetch_2d(&tmap_b, kb * (BK / 2), nb * 128);
+    for (int kb = k0; kb < min(k1, k0 + kSkinnyPrefetch); ++kb) tma_prefetch_2d(&tmap_b, kb * (BK / 2), nb * 128);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, C::kTmemCols);
@@ -1775,9 +1756,6 @@ __device__ __forceinline__ void named_barrier(uint32_t id, uint32_t threads) {
 }
 __device__ __forceinline__ void st_shared_v2_u32(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
-}
-__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ void st_shared_u8(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
@@ -2205,7 +2183,7 @@ int resident_pairs() {
   return clusters;
 }
 
-// kSwiGLU: out_bf16 is unused (no output map); the fused outputs go through
+// kSwiGLU: out_bf16 is unused; the fused outputs go through
 // args.q_codes / q_scales / g_out, which the caller fills in `extra`.
 template <class C, bool kSwiGLU = false>
 nvfp4_status launch_pair(const uint8_t* a_codes, const uint8_t* a_scales, const float* g_a, const uint8_t* w_codes,
@@ -2215,13 +2193,11 @@ nvfp4_status launch_pair(const uint8_t* a_codes, const uint8_t* a_scales, const 
   const int64_t tiles_m = (M + BM - 1) / BM, tiles_n = (N + C::BN - 1) / C::BN;  // a column tail reads zeros
   const int64_t units = ((tiles_m + 1) / 2) * tiles_n;
   if (units >= (1ll << 31)) return NVFP4_ERR_SHAPE;
-  CUtensorMap ma, mb, mb_half, msa, msb, mo;
+  CUtensorMap ma, mb, mb_half, msa, msb;
   if (!make_code_map(&ma, a_codes, M, K, BM) || !make_code_map(&mb, w_codes, N, K, 128) ||
       !make_code_map(&mb_half, w_codes, N, K, 64) ||
       !make_scale_map(&msa, a_scales, M, K, false) || !make_scale_map(&msb, w_scales, N, K, true))
     return NVFP4_ERR_CUDA;
-  if (kSwiGLU) mo = ma;  // not read by the fused epilogue
-  else if (!make_out_map(&mo, out_bf16, M, N, ldo)) return NVFP4_ERR_CUDA;
   const int pairs_max = resident_pairs<C, kSwiGLU>();
   if (pairs_max <= 0) return NVFP4_ERR_CUDA;
   GemmArgs args = {};
@@ -2264,7 +2240,7 @@ nvfp4_status launch_pair(const uint8_t* a_codes, const uint8_t* a_scales, const 
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, nvfp4_gemm_pair_kernel<C, kSwiGLU>, ma, mb, mb_half, msa, msb, mo, args) != cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, nvfp4_gemm_pair_kernel<C, kSwiGLU>, ma, mb, mb_half, msa, msb, args) != cudaSuccess)
     return NVFP4_ERR_CUDA;
   count_launches(1);
   return launch_status();
@@ -2470,7 +2446,6 @@ nvfp4_status launch_skinny(const uint8_t* a_codes, const uint8_t* a_scales, cons
   args.N = static_cast<int>(N);
   args.K = static_cast<int>(K);
   args.splits = splits;
-  args.prefetch_kb = kSkinnyPrefetch;
   args.status = status_word_dev();
   args.fault_skip_stage = take_fault(NVFP4_FAULT_GEMM_SKIP_STAGE) ? 1 : 0;
   args.out = static_cast<uint16_t*>(out_bf16);

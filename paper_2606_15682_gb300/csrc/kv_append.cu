@@ -2,8 +2,8 @@
 // m, Eq. 2) and write them into the NVFP4 KV cache; optionally rotate K by
 // RoPE first (the fused RoPE -> shift -> quantize -> append step).
 //
-// One thread per 16-element block of a 128-channel row, so the block scale is
-// computed once; reads of 16 threads cover whole K and V rows.
+// A thread takes the same 16-element block of one, two or four heads of a token,
+// of K or of V, so each block scale is computed once; eight lanes cover a row.
 #include <cfloat>
 
 #include "common.cuh"
@@ -21,9 +21,10 @@ constexpr int kThreads = 256;
 // A thread takes one 16-element block (of K or of V) of U consecutive heads of
 // one token.  Eight lanes cover a row's blocks, a warp four head groups of K or
 // of V (so that no lane idles while K is rotated); the RoPE partner block
-// (channels 64 apart) is on lane l ^ 4.  The rotation depends on the token and the block only, so its (cos,
-// sin) values, four times the bytes of a K block, are loaded once for U heads,
-// and everything else that the thread reads is issued with them.
+// (channels 64 apart) is on lane l ^ 4.  The rotation depends on the token and
+// the block only, so its (cos, sin) values, four times the bytes of a K block,
+// are loaded once for U heads, and everything else that the thread reads is
+// issued with them.
 template <bool kRope, bool kE1M2, int U>
 __global__ void __launch_bounds__(kThreads) kv_append_kernel(
     const uint16_t* __restrict__ k_in, const uint16_t* __restrict__ v_in, const int32_t* __restrict__ seq_idx,

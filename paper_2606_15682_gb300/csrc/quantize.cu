@@ -98,12 +98,10 @@ __global__ void tensor_scale_finalize(float* g) {
   *g = amax > 0.0f ? __fdiv_rn(amax, 2688.0f) : 1.0f;
 }
 
-// One thread quantizes one 16-element block: two 128-bit loads (the second
-// half of the 32 bytes is in L1 after the first load of the warp), one scale
-// computation, one 64-bit code store.  A warp covers 32 consecutive blocks.
-// Where one pass of the quantizer reads: the thread's kUnroll 16-element
-// blocks of the iteration that starts at the warp-uniform block index bidx0
-// (block bidx0 + u * stride + lane).
+// What a thread holds in one pass of the quantizer: its U 16-element blocks
+// (two 128-bit loads, one scale computation and one 64-bit code store each) of
+// the iteration that starts at the warp-uniform block index bidx0 (block bidx0 +
+// u * stride + lane; a warp covers 32 consecutive blocks per slot).
 template <int U = kUnroll>
 struct BlockSlots {
   uint4 v0[U], v1[U];
