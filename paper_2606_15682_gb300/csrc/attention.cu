@@ -197,7 +197,8 @@ __device__ __forceinline__ uint32_t chunks_of(int tokens) {
 // through shared memory.  (Walked by every warp, an item cost 1 us more.)  GB300,
 // 40 heads on 8 KV heads, against the capacity's chunks in turn: 64 sequences of
 // 2000-16384 tokens 208 -> 146 us, 32 of 512-4096 39.1 -> 32.4, 64 of 3000 56.5 ->
-// 53.9; 64 of 16384, where both orders are the same, 235.7 -> 237.7.
+// 53.9; 64 of 16384, where both orders are the same, 236.0 -> 235.4 (E1M2 302.5
+// -> 310.4, ragged 268 -> 188).
 struct Walk {
   uint32_t at;      // this CTA's next item
   uint32_t before;  // items before the window
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
     float m_run[2] = {-INFINITY, -INFINITY};
     float l_run[2] = {0.0f, 0.0f};
 
-    for (int t0 = it.t_begin; t0 < it.t_end; t0 += kStageTok) {
+    for (int left = it.t_end - it.t_begin; left > 0; left -= kStageTok) {  // the item's tokens from this stage on
       int ok = 1;
       if (lane == 0) {
         ok = !abort_flag && mbar_wait_bounded(&full[stage], phase, &abort_flag);
@@ -451,8 +452,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
 #pragma unroll
       for (int sub = 0; sub < kStageTok / (16 * kConsumers); ++sub) {
       const int r0 = 16 * (cw + kConsumers * sub);  // this warp's tile within the stage
-      const int tile = t0 + r0;
-      const int valid = it.t_end - tile;  // tokens of this warp's tile inside the item (may be <= 0)
+      const int valid = left - r0;  // tokens of this warp's tile inside the item (may be <= 0)
       if (valid > 0) {
         // ---- S^T = K_hat Q^T: 8 k-steps of 16 channels ---------------------
         const uint4 ka = *reinterpret_cast<const uint4*>(st + kOffKc + (r0 + rk0) * 64 + 16 * t);
@@ -592,6 +592,15 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
       sh_l[cw * 8 + 2 * t] = l_run[0]; sh_l[cw * 8 + 2 * t + 1] = l_run[1];
     }
     named_barrier_consumers();
+    if (kListed) {
+      // Read again rather than kept in registers through the stages (E1M2, 64 x
+      // 16384 tokens: 320 -> 310 us); the place is rewritten after item j + 1.
+      const volatile Item* done = &items[j % kItems];
+      it.b = done->b;
+      it.kvh = done->kvh;
+      it.split = done->split;
+    }
+    const size_t rec0 = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group) * p.n_splits + it.split;
     for (int idx = threadIdx.x - 32; idx < p.group * kD; idx += 32 * kConsumers) {
       const int h = idx / kD, c = idx % kD;
       float M = -INFINITY;
@@ -606,7 +615,7 @@ __global__ void __launch_bounds__(kThreads, NVFP4_ATTN_MIN_CTAS) attn_partial_ke
           L += wt * sh_l[w * 8 + h];
         }
       }
-      const size_t rec = (static_cast<size_t>(it.b) * p.hq + it.kvh * p.group + h) * p.n_splits + it.split;
+      const size_t rec = rec0 + static_cast<size_t>(h) * p.n_splits;
       p.o_ws[rec * kD + c] = acc;
       if (c == 0) {
         p.ml_ws[rec * 2] = M;
