@@ -611,6 +611,26 @@ def test_decode_attention_of_a_sequence_is_its_own(N, hq, hkv, cap, lens, fmt):
         assert torch.equal(out[b:b + 1], attend(N, own, q[b:b + 1].contiguous())), f"sequence {b} of {n}"
 
 
+def test_injected_missing_stage_where_items_come_from_the_list(N):
+    """As above with more chunks than CTAs, where the consumers get their items
+    from the producer warp: the call reports NVFP4_ERR_TIMEOUT and the next one
+    gives the same bits as the one before."""
+    import time
+    cache, gen = random_cache(N, 40, 8, 2048, [2048] * 39 + [1500], 0)
+    q = torch.randn(40, 8, 128, generator=gen, device="cuda").to(torch.bfloat16)
+    before = attend(N, cache, q)
+    N.nvfp4_debug_inject_fault(N.FAULT_ATTN_SKIP_STAGE)
+    try:
+        t0 = time.time()
+        run_attention(N, cache, q, 1 / math.sqrt(128))
+        waited = time.time() - t0
+    finally:
+        N.nvfp4_debug_inject_fault(N.FAULT_NONE)
+    assert N.nvfp4_get_device_status() == 6
+    assert 1.0 < waited < 20.0, f"bounded wait expected (~2-4 s), took {waited:.1f} s"
+    assert torch.equal(attend(N, cache, q), before)
+
+
 @pytest.mark.parametrize("n_new,hkv", [(1, 1), (3, 3), (7, 8), (608, 8), (611, 8), (1231, 6), (2433, 8), (2431, 4)])
 @pytest.mark.parametrize("fmt", [0, 1])
 def test_append_heads_per_thread(N, n_new, hkv, fmt):

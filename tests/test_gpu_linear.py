@@ -52,7 +52,8 @@ def run_linear(N, a_codes, a_scales_rm, g_a, w_codes, w_scales_rm, g_w, M, Nn, K
                                     (256, 256, 512), (300, 512, 1024), (640, 768, 768), (129, 1280, 2048),
                                     (16, 1536, 1536), (256, 5120, 3584),
                                     # ... and with K >= 4096: split-K clusters of 2, 3 or 4 pairs, even
-                                    # and uneven K ranges, M tails, a spare CTA per pair when M <= 128
+                                    # and uneven K ranges, M tails, a spare CTA per pair; M <= 128: the
+                                    # skinny kernel
                                     (256, 512, 4096), (16, 1536, 4608), (1, 256, 4096), (300, 768, 5120),
                                     (100, 512, 6400), (256, 7168, 4096), (256, 5120, 4352),
                                     # CTA-pair path (enough 256 x 256 tiles to occupy the pairs):
@@ -61,7 +62,7 @@ def run_linear(N, a_codes, a_scales_rm, g_a, w_codes, w_scales_rm, g_w, M, Nn, K
                                     # more 256 x 256 tiles than pairs: a second round of tiles, with an M
                                     # tail (K = 1536)
                                     (512, 10240, 1024), (300, 15360, 1536), (640, 7680, 1280),
-                                    # N % 256 != 0 with K >= 2048 (single CTAs), and a pair shape with K = 4096
+                                    # N % 256 != 0 (CTA pairs with a column tail), and a pair shape with K = 4096
                                     # and a one-row M tail
                                     (640, 10112, 2048), (512, 10576, 2048), (257, 15360, 4096)])
 def test_random_codes(N, M, Nn, K):
@@ -391,8 +392,9 @@ def test_linear_swiglu_quantize_few_rows(N, M, I, K, fmt):
     assert not scales[M:].any()
 
 
-def test_linear_swiglu_quantize_invalid_g_out_zeroes_and_reports(N):
-    M, I, K = 256, 128, 256
+@pytest.mark.parametrize("M", [256, 20])  # CTA pairs, skinny kernel
+def test_linear_swiglu_quantize_invalid_g_out_zeroes_and_reports(N, M):
+    I, K = 128, 256
     gen = torch.Generator().manual_seed(3)
     a_c, a_s = random_operand(M, K, gen)
     w_c, w_s = random_operand(2 * I, K, gen)
