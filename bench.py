@@ -48,11 +48,11 @@ CSRC = os.path.join(ROOT, "paper_2606_15682_gb300", "csrc")
 # same kernel and shape (commands in profiles/).  Each entry holds only while the kernel sources
 # hash to the value they had at capture time; otherwise the line reports traffic = null.
 NCU_TRAFFIC = {
-    "gemm": {"bytes": 205226240 + 862310656, "sources": ("gemm.cu", "common.cuh"), "sha": "2008d5f823588b75",
+    "gemm": {"bytes": 215494144 + 865210624, "sources": ("gemm.cu", "common.cuh"), "sha": "c4befea42e53aac5",
              "shape": (8192, 55296, 5120),
              "profile": "profiles/gemm_qwen32b_prefill_gate_up_m8192_n55296_k5120.md"},
-    "attention": {"bytes": 1209425664 + 5265408, "sources": ("attention.cu", "common.cuh"),
-                  "sha": "95321c047075933d", "shape": (64, 16384),
+    "attention": {"bytes": 1208737280 + 22180864, "sources": ("attention.cu", "common.cuh"),
+                  "sha": "ddab0fa73b64e881", "shape": (64, 16384),
                   "profile": "profiles/attention_qwen14b_decode_b64_t16384.md (attn_partial_kernel)"},
 }
 

@@ -146,11 +146,11 @@ nvfp4_status nvfp4_scales_relayout(const uint8_t* src, uint8_t* dst, int64_t row
  * paper's compute speedup comes from, Sec. 5.3):
  *   out[m, n] = bf16_rne( (g_a * g_w) * sum_k a[m,k] * w[n,k] )
  * with a[m,k] = e2m1 * e4m3 of A (no g) and likewise for W; the sum is
- * accumulated in fp32 by the tensor core (tcgen05 block-scaled MMA).  When
- * N % 256 == 0, K >= 4096 and the 256 x 256 tiles are too few to occupy the
- * GPU (decode-sized M), K is split into 2-4 contiguous ranges whose fp32 partial
- * sums are added in range order in the cluster's shared memory: the result
- * is deterministic for a given shape.
+ * accumulated in fp32 by the tensor core (tcgen05 block-scaled MMA).  Where
+ * the tiles are too few to occupy the GPU (M <= 128 with K > 1536; larger
+ * decode-sized M with N % 256 == 0 and K >= 4096), K is split into 2-8
+ * contiguous ranges whose fp32 partial sums are added in range order in the
+ * cluster's shared memory: the result is deterministic for a given shape.
  *   a_codes  : [M, K/2] bytes (K-major), 16-B aligned.
  *   a_scales : MMA layout for [M, K].
  *   w_codes  : [N, K/2] bytes (K-major, i.e. the nn.Linear weight [N, K]).
