@@ -564,6 +564,7 @@ def attend(N, cache, q, extra=0):
     (8, 8, 1400, [1400, 3, 128, 1, 90, 0, 1400, 129] * 6, 1),  # runs of one-stage chunks beside long ones
     (8, 8, 2048, [1100] * 40, 0),                              # equal, a little longer than a chunk
     (16, 8, 1024, [1024, 7, 500, 0] * 25, 0),                  # more one-chunk heads than CTAs
+    (8, 4, 1200, [(53 * i) % 1201 for i in range(100)], 0),    # four windows of sequences, mostly ends
     (8, 8, 4096, [0, 0, 4096, 1025, 0, 1024, 2, 0, 2049] * 3, 0)])  # runs that begin and end at empty sequences
 def test_decode_attention_over_ragged_lengths(N, hq, hkv, cap, lens, fmt):
     B = len(lens)
